@@ -57,8 +57,9 @@ ADJ_MIXED_PP_PER_CLK_PER_SM = 224.0 / 17.0
 # cosine, 7 issue slots (2 integer adds, shift, or, FMA to radians,
 # argument scale, accumulate): the MUFU binds at 16 updates/clk/SM.
 RECUR_PP_PER_CLK_PER_SM = 16.0
-# The FP32 separable product (angle addition) per update: 2 FP32
-# multiply-adds on the FMA pipe, no MUFU: 128 / 2 = 64 updates/clk/SM.
+# An FP32 angle-addition product on the FMA pipe, per update: 2 FP32
+# multiply-adds, no MUFU: 128 / 2 = 64 updates/clk/SM.  (The FP32 separable
+# product runs on the tensor cores; this is the bound it no longer has.)
 SIMT_PP_PER_CLK_PER_SM = 64.0
 # The FP32 separable adjoint per update: 4 FP32 multiply-adds (the column
 # sums U, V and the row sums P, Q), no MUFU: 128 / 4 = 32 updates/clk/SM
@@ -342,10 +343,10 @@ class Leg:
 MAIN_KERNEL = {"direct": "direct", "naive": "naive", "recur": "recur",
                "sep_fp32": "simt", "sep_fp16x3": "gemm", "sep_fp16": "gemm",
                "sep_bf16": "gemm"}
-GEMM_PASSES = {"sep_fp16x3": 3.0, "sep_fp16": 1.0, "sep_bf16": 1.0}
+GEMM_PASSES = {"sep_fp32": 3.0, "sep_fp16x3": 3.0, "sep_fp16": 1.0, "sep_bf16": 1.0}
 # methods whose kernels store the hologram tile by tile (into mapped host
 # memory in place when the output is a pinned host buffer)
-PROGRESSIVE = {"direct", "naive", "recur", "sep_fp32"}
+PROGRESSIVE = {"direct", "naive", "recur"}
 
 
 def build_legs(cg, h, which, methods, dev, stream, shard=None):
@@ -443,9 +444,10 @@ def build_legs(cg, h, which, methods, dev, stream, shard=None):
             f_bwd = (lambda m=m: cg.cgh_backward(
                 pts, A, z, c.lam, c.p, c.Nx, c.Ny, G, method=m, handle=h,
                 stream=stream))
-            mult = 3.0 if m == "sep_fp16x3" else 0.0
+            mult = GEMM_PASSES.get(m, 0.0)
             legs.append(Leg(m + "_fwd", f_fwd, c.pp, 4.0 * c.pp * mult, 1 if mult else 0,
                             kernel=MAIN_KERNEL[m], method=m))
+            mult = 3.0 if m == "sep_fp16x3" else 0.0
             legs[-1].size = (c.N, c.Nx, c.Ny)
             legs.append(Leg(m + "_bwd", f_bwd, c.pp, 2 * 4.0 * c.pp * mult,
                             2 if mult else 0,
@@ -455,8 +457,8 @@ def build_legs(cg, h, which, methods, dev, stream, shard=None):
     raise SystemExit(f"unknown workload {which}")
 
 
-ALU_KERNELS = ("direct", "naive", "batch", "bwd_direct", "recur", "simt", "bwd_simt")
-GEMM_KERNELS = ("gemm", "bwd_gemm", "batch_sep")
+ALU_KERNELS = ("direct", "naive", "batch", "bwd_direct", "recur", "bwd_simt")
+GEMM_KERNELS = ("gemm", "bwd_gemm", "batch_sep", "simt")
 
 
 def alu_recipe(kernel, tile=None):
@@ -482,10 +484,6 @@ def alu_recipe(kernel, tile=None):
                 "MUFU limit of the row rotation recipe: a sincos (2 MUFU ops) per "
                 "row of 4 pixels, 16 per clk/SM; 3 FP32 ops per update allow 42.7",
                 lambda m, fr: min(2.0 * m, fr / 3.0), 0.5)
-    if kernel == "simt":
-        return (SIMT_PP_PER_CLK_PER_SM,
-                "FMA-pipe limit of the FP32 angle-addition product: 2 FP32 "
-                "multiply-adds per update, 128 per clk/SM", lambda m, f: f / 2.0, 0.0)
     if kernel == "bwd_simt":
         return (BWD_SIMT_PP_PER_CLK_PER_SM,
                 "FMA-pipe limit of the FP32 angle-addition adjoint: 4 FP32 "

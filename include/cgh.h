@@ -91,12 +91,12 @@ typedef enum {
      * 32-bit fixed-point turns), hardware cosine.  A comparison point for
      * CGH_DIRECT_FP32 (same accuracy bound). */
     CGH_RECUR_FP32 = 5,
-    /* The separable form in FP32 on the FMA pipe: with per-axis tables of
-     * A_j (cos, -sin) theta_x and (cos, sin) theta_y (exact fixed-point
-     * phase, accurate sincospi), cos(theta_x + theta_y) is two FP32
-     * multiply-adds per point-pixel update, no special-function operation;
-     * an FP32 matrix product of depth 2N on the SIMT cores.  Same accuracy
-     * bound as CGH_DIRECT_FP32. */
+    /* The separable form at FP32 accuracy: per-axis tables of A_j (cos, -sin)
+     * theta_x and (cos, sin) theta_y (exact fixed-point phase, sine and
+     * cosine to FP32 rounding), each FP32 entry split without loss of range
+     * into two FP16 numbers, multiplied on the tensor cores (three products)
+     * 64 values of k at a time, the partial sums added in FP32 registers
+     * with round to nearest.  Same accuracy bound as CGH_DIRECT_FP32. */
     CGH_SEP_FP32 = 6
 } cgh_method;
 
@@ -143,7 +143,7 @@ cgh_status cgh_forward_rows(cgh_handle h, const float *points, const float *A,
  * e.g. PyTorch pinned tensors, on a unified-addressing system) are used in
  * place: the kernels read such inputs over the host link, and the methods
  * that store the hologram tile by tile as they run (CGH_DIRECT_FP32,
- * CGH_RECUR_FP32, CGH_NAIVE_FP32, CGH_SEP_FP32) write such an output there
+ * CGH_RECUR_FP32, CGH_NAIVE_FP32) write such an output there
  * directly.  The tensor-core methods, and any other buffer (pageable
  * memory, device memory), go through the handle's workspace and one copy.
  * The result is the same either way. */
@@ -459,7 +459,7 @@ typedef enum {
     CGH_K_AUX = 10,           /* small helpers (conversions, fills)     */
     CGH_K_BATCH_SEP = 11,     /* separable batch (its whole graph)      */
     CGH_K_RECUR = 12,         /* Eq. 2 recurrence kernel                */
-    CGH_K_SIMT = 13,          /* FP32 separable product (FMA pipe)      */
+    CGH_K_SIMT = 13,          /* FP32 separable product (tensor cores)  */
     CGH_K_BWD_SIMT = 14,      /* FP32 separable adjoint (FMA pipe)      */
     CGH_K_COUNT = 16
 } cgh_kernel_id;

@@ -240,7 +240,7 @@ cgh_status cgh_ctx::forward(const float *points, const float *A,
     case CGH_RECUR_FP32:
         return forward_recur(points, A, z, N, lambda, p, Nx, Ny, out, s);
     case CGH_SEP_FP32:
-        return forward_simt(points, A, z, N, lambda, p, Nx, Ny, out, s);
+        return forward_sep32(points, A, z, N, lambda, p, Nx, Ny, out, s);
     case CGH_SEP_BF16:
     case CGH_SEP_FP16:
     case CGH_SEP_FP16X3:
@@ -393,7 +393,6 @@ cgh_status cgh_create(cgh_handle *out, int device) {
     }
     h->load_tune_cache();
     if (const char *f = getenv("CGH_FAIL_ALLOC_AFTER")) h->fail_alloc_after = atoi(f);
-    if (const char *f = getenv("CGH_SIMT_STAGE")) h->simt_stage = atoi(f);
     if (const char *f = getenv("CGH_GEMM_TILES")) {
         const int v = atoi(f);
         if (v >= CGH_GEMM_AUTO && v <= CGH_GEMM_PAIRS_GEN) h->gemm_tiles = v;
@@ -477,8 +476,8 @@ cgh_status cgh_forward_host(cgh_handle h, const float *points_host,
     // Mapped (pinned) host inputs are read in place by the per-point
     // prologue.  A mapped output is written in place by the methods whose
     // kernels store the hologram tile by tile while they run (direct,
-    // recurrence, naive, FP32 separable): those stores hide under the
-    // compute.  The tensor-core GEMM stores the whole hologram in one burst
+    // recurrence, naive): those stores hide under the
+    // compute.  The tensor-core GEMMs store the whole hologram in one burst
     // at its end, which crosses the host link faster as one copy (measured
     // at 1920x1024: 207 us in place against 120 us staged).  Other buffers
     // are staged through the handle's workspace.
@@ -486,7 +485,7 @@ cgh_status cgh_forward_host(cgh_handle h, const float *points_host,
     const float *m_A = N > 0 ? (const float *)mapped_device_ptr(A_host) : nullptr;
     const float *m_z = N > 0 ? (const float *)mapped_device_ptr(z_host) : nullptr;
     const bool progressive = method == CGH_DIRECT_FP32 || method == CGH_NAIVE_FP32 ||
-                             method == CGH_RECUR_FP32 || method == CGH_SEP_FP32;
+                             method == CGH_RECUR_FP32;
     float *m_out = progressive ? (float *)mapped_device_ptr(out_host) : nullptr;
     const size_t pts_b = m_pts ? 0 : align256((size_t)N * 2 * sizeof(float));
     const size_t a_b = m_A ? 0 : align256((size_t)N * sizeof(float));
@@ -549,7 +548,7 @@ cgh_status cgh_forward_host_async(cgh_handle h, const float *points_host,
         return h->fail(CGH_ERR_INVALID_ARG,
                        "cgh_forward_host_async needs page-locked, mapped host buffers");
     const bool progressive = method == CGH_DIRECT_FP32 || method == CGH_NAIVE_FP32 ||
-                             method == CGH_RECUR_FP32 || method == CGH_SEP_FP32;
+                             method == CGH_RECUR_FP32;
     // this call's ticket: its event slot must be free (the call that many
     // tickets back has finished)
     const uint64_t ticket = h->host_calls + 1;

@@ -96,10 +96,6 @@ struct cgh_ctx {
     // direct forward: the tables kernel builds the point records itself (1)
     // or reads them from a prologue launch (0); CGH_DIRECT_FUSED_TABLES
     int direct_fused_tables = 1;
-    // stage shape of the FP32 separable product (index into the compiled
-    // shapes; 1 = 32 values of k x 2 stages, the fastest measured);
-    // CGH_SIMT_STAGE at cgh_create
-    int simt_stage = 1;
     // fault injection: workspace allocations left before one is made to
     // fail (-1: never); set from CGH_FAIL_ALLOC_AFTER at cgh_create
     int fail_alloc_after = -1;
@@ -130,9 +126,9 @@ struct cgh_ctx {
     cgh_status forward_recur(const float *points, const float *A,
                              const float *z, int N, double lambda, double p,
                              int Nx, int Ny, float *out, cudaStream_t s);
-    cgh_status forward_simt(const float *points, const float *A,
-                            const float *z, int N, double lambda, double p,
-                            int Nx, int Ny, float *out, cudaStream_t s);
+    cgh_status forward_sep32(const float *points, const float *A, const float *z, int N,
+                             double lambda, double p, int Nx, int Ny, float *out,
+                             cudaStream_t s);
     cgh_status forward_separable(const float *points, const float *A,
                                  const float *z, int N, double lambda, double p,
                                  int Nx, int Ny, float *out, int method,

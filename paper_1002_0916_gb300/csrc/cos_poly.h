@@ -4,6 +4,8 @@
 // COS5_C: degree 5 in d^2, max error in FP32 evaluation 1.27e-06;
 // sin(d) ~= d * sum_k S_k (d^2)^k for d in [0, pi]:
 // SIN5_C: degree 5 in d^2, max error in FP32 evaluation 4.44e-07.
+// sin(pi/2 x) ~= x * sum_k QSIN_C_k (x^2)^k and cos(pi/2 x) ~= sum_k QCOS_C_k
+// (x^2)^k for |x| <= 1/2: max error in FP32 8.32e-08 and 5.51e-08.
 #pragma once
 
 namespace cgh {
@@ -29,5 +31,16 @@ constexpr float SIN5_C2 = 0.008332425728440285f;
 constexpr float SIN5_C3 = -0.00019809025980066508f;
 constexpr float SIN5_C4 = 2.700008735700976e-06f;
 constexpr float SIN5_C5 = -2.037002744259553e-08f;
+
+constexpr float QSIN_C0 = 1.5707963705062866f;
+constexpr float QSIN_C1 = -0.6459634900093079f;
+constexpr float QSIN_C2 = 0.07968010008335114f;
+constexpr float QSIN_C3 = -0.004601663444191217f;
+
+constexpr float QCOS_C0 = 1.0f;
+constexpr float QCOS_C1 = -1.2337005138397217f;
+constexpr float QCOS_C2 = 0.25366923213005066f;
+constexpr float QCOS_C3 = -0.020860297605395317f;
+constexpr float QCOS_C4 = 0.0009040222503244877f;
 
 }  // namespace cgh

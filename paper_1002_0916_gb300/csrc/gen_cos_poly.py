@@ -2,6 +2,10 @@
 """Fit the software cosine and sine used next to the hardware (MUFU) ones in
 the direct kernels, and write cos_poly.h.
 
+Also sin(pi/2 x) as x times a polynomial of degree 3 in x^2 and cos(pi/2 x) as
+a polynomial of degree 4 in x^2 for |x| <= 1/2 (x in quarter turns), to FP32
+rounding, for the tables that take the octant from the fixed-point phase.
+
 cos(d) for d in [0, pi] as a polynomial in s = d^2 of degree 6 (and 5), and
 sin(d) as d times a polynomial in s of degree 5, fitted by an iteratively
 reweighted least-squares minimax approximation (Lawson's algorithm: repeated
@@ -38,6 +42,38 @@ def fit(deg=DEG, iters=200, odd=False):
     return c
 
 
+def fit_quarter(deg, odd, iters=200):
+    """sin(pi/2 x) / x (odd, relative error) or cos(pi/2 x) in s = x^2, |x| <= 1/2,
+    with the cosine's constant term fixed at 1."""
+    s = np.linspace(1e-9, 0.25, 40001)
+    x = np.sqrt(s)
+    f = np.sin(np.pi / 2 * x) / x if odd else (np.cos(np.pi / 2 * x) - 1.0) / s
+    V = np.vander(s, deg + 1 if odd else deg, increasing=True)
+    scale = 1.0 / f if odd else s  # error of the value itself
+    w = np.ones_like(s)
+    for _ in range(iters):
+        c, *_ = np.linalg.lstsq(V * (w * scale)[:, None], f * scale * w, rcond=None)
+        e = np.abs((V @ c - f) * scale)
+        w = w * (e / e.max() + 1e-3)
+        w /= w.sum()
+    return c if odd else np.concatenate([[1.0], c])
+
+
+def quarter_error(c, odd):
+    """Largest error in FP32, each multiply-add rounded once (float64 holds a
+    product of two FP32 numbers exactly)."""
+    x = np.linspace(-0.5, 0.5, 400001).astype(np.float32)
+    s = (x * x).astype(np.float32)
+    c32 = np.asarray(c, dtype=np.float32)
+    p = np.full_like(s, c32[-1])
+    for k in range(len(c32) - 2, -1, -1):
+        p = (p.astype(np.float64) * s + float(c32[k])).astype(np.float32)
+    if odd:
+        p = (p * x).astype(np.float32)
+    d = np.pi / 2 * x.astype(np.float64)
+    return float(np.max(np.abs(p - (np.sin(d) if odd else np.cos(d)))))
+
+
 def fp32_error(c, odd=False):
     d = np.linspace(0.0, np.pi, 200001).astype(np.float32)
     s = (d * d).astype(np.float32)
@@ -63,6 +99,7 @@ def main():
     c = fit()
     c5 = fit(5)
     s5 = fit(5, odd=True)
+    qs, qc = fit_quarter(3, True), fit_quarter(4, False)
     lines = ["// cos_poly.h -- written by gen_cos_poly.py; do not edit.",
              "// cos(d) ~= sum_k C_k (d^2)^k for d in [0, pi] (Lawson minimax fits):",
              f"// COS_C: degree {DEG} in d^2, max error in FP32 evaluation "
@@ -72,6 +109,9 @@ def main():
              "// sin(d) ~= d * sum_k S_k (d^2)^k for d in [0, pi]:",
              f"// SIN5_C: degree 5 in d^2, max error in FP32 evaluation "
              f"{fp32_error(s5, odd=True):.2e}.",
+             "// sin(pi/2 x) ~= x * sum_k QSIN_C_k (x^2)^k and cos(pi/2 x) ~= sum_k QCOS_C_k",
+             f"// (x^2)^k for |x| <= 1/2: max error in FP32 {quarter_error(qs, True):.2e} and "
+             f"{quarter_error(qc, False):.2e}.",
              "#pragma once", "", "namespace cgh {", ""]
     for k, v in enumerate(c):
         lines.append(f"constexpr float COS_C{k} = {float(np.float32(v))!r}f;")
@@ -81,6 +121,10 @@ def main():
     lines.append("")
     for k, v in enumerate(s5):
         lines.append(f"constexpr float SIN5_C{k} = {float(np.float32(v))!r}f;")
+    for name, poly in (("QSIN_C", qs), ("QCOS_C", qc)):
+        lines.append("")
+        for k, v in enumerate(poly):
+            lines.append(f"constexpr float {name}{k} = {float(np.float32(v))!r}f;")
     lines += ["", "}  // namespace cgh", ""]
     open(OUT, "w").write("\n".join(lines))
     print(open(OUT).read())

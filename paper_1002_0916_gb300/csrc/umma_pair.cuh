@@ -124,6 +124,16 @@ __device__ __forceinline__ void remote_arrive(uint32_t cluster_addr) {
                  : "memory");
 }
 
+// Arrive on the mbarrier at cluster address `cluster_addr` after this
+// thread's reads of tensor memory (ordered by tcgen05.wait::ld and
+// tcgen05.fence::before_thread_sync).  No generic memory is handed over, so
+// the arrive is relaxed.
+__device__ __forceinline__ void arrive_pair(uint32_t cluster_addr) {
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(
+                     cluster_addr)
+                 : "memory");
+}
+
 }  // namespace umma2
 
 template <int BNP, bool SPLIT, int STAGES>
