@@ -61,9 +61,9 @@ RECUR_PP_PER_CLK_PER_SM = 16.0
 # multiply-adds, no MUFU: 128 / 2 = 64 updates/clk/SM.  (The FP32 separable
 # product runs on the tensor cores; this is the bound it no longer has.)
 SIMT_PP_PER_CLK_PER_SM = 64.0
-# The FP32 separable adjoint per update: 4 FP32 multiply-adds (the column
-# sums U, V and the row sums P, Q), no MUFU: 128 / 4 = 32 updates/clk/SM
-# (the row's sincos and sums, shared by 16 updates, not counted).
+# An angle-addition adjoint on the FMA pipe, per update: 4 FP32 multiply-adds
+# (the column sums U, V and the row sums P, Q), no MUFU: 128 / 4 = 32
+# updates/clk/SM (the row's sincos and sums, shared by 16 updates, not counted).
 BWD_SIMT_PP_PER_CLK_PER_SM = 32.0
 # The paper's Table 1 (1,920 x 1,024 pixels), times in ms, for context.
 PAPER_TABLE1 = {
@@ -447,18 +447,18 @@ def build_legs(cg, h, which, methods, dev, stream, shard=None):
             mult = GEMM_PASSES.get(m, 0.0)
             legs.append(Leg(m + "_fwd", f_fwd, c.pp, 4.0 * c.pp * mult, 1 if mult else 0,
                             kernel=MAIN_KERNEL[m], method=m))
-            mult = 3.0 if m == "sep_fp16x3" else 0.0
+            # both products of the separable adjoint are one launch
             legs[-1].size = (c.N, c.Nx, c.Ny)
             legs.append(Leg(m + "_bwd", f_bwd, c.pp, 2 * 4.0 * c.pp * mult,
-                            2 if mult else 0,
+                            1 if mult else 0,
                             kernel={"direct": "bwd_direct", "sep_fp32": "bwd_simt"}.get(
                                 m, "bwd_gemm")))
         return c, legs
     raise SystemExit(f"unknown workload {which}")
 
 
-ALU_KERNELS = ("direct", "naive", "batch", "bwd_direct", "recur", "bwd_simt")
-GEMM_KERNELS = ("gemm", "bwd_gemm", "batch_sep", "simt")
+ALU_KERNELS = ("direct", "naive", "batch", "bwd_direct", "recur")
+GEMM_KERNELS = ("gemm", "bwd_gemm", "batch_sep", "simt", "bwd_simt")
 
 
 def alu_recipe(kernel, tile=None):
@@ -484,10 +484,6 @@ def alu_recipe(kernel, tile=None):
                 "MUFU limit of the row rotation recipe: a sincos (2 MUFU ops) per "
                 "row of 4 pixels, 16 per clk/SM; 3 FP32 ops per update allow 42.7",
                 lambda m, fr: min(2.0 * m, fr / 3.0), 0.5)
-    if kernel == "bwd_simt":
-        return (BWD_SIMT_PP_PER_CLK_PER_SM,
-                "FMA-pipe limit of the FP32 angle-addition adjoint: 4 FP32 "
-                "multiply-adds per update, 128 per clk/SM", lambda m, f: f / 4.0, 0.0)
     if kernel == "recur":
         return (RECUR_PP_PER_CLK_PER_SM,
                 "MUFU limit of the Eq. 2 recurrence recipe: 1 hardware cosine per "
@@ -711,7 +707,7 @@ def measure_extras(cg, h, dev, stream, flush, K, sms, peaks, pipe_rates, gpu_id,
         else:
             e["shapes"] = {"direct_tile": list(cg.cgh_direct_tile_for(h, c.N, c.Nx, c.Ny)),
                            "tuned": tune}
-            for m in sorted({leg.method for leg in legs if leg.method in GEMM_PASSES}):
+            for m in sorted({leg.method for leg in legs if leg.method in TUNABLE[1:]}):
                 e["shapes"]["gemm_plan_" + m] = list(cg.cgh_gemm_plan_for(h, c.N, c.Nx,
                                                                           c.Ny, m))
         if "frac_of_measured_rates" in roof:
@@ -996,7 +992,7 @@ def run_ours(args):
             "steps": K, "warmup": args.warmup, "ms_per_step": ms,
             "higher_is_better": True, "scaling": "weak" if shard is None else "strong",
             "vs_baseline": value / PAPER_PP_PER_S if args.workload == "paper" else None,
-            "dtype": ("f32+f16x3" if any(leg.method in GEMM_PASSES for leg in legs)
+            "dtype": ("f32+f16x3" if any(leg.method in TUNABLE[1:] for leg in legs)
                       else "f32"),
             "data": "synthetic", "config": cfg,
             "timing": ("ms_per_step, value, gpu_launches: timed region 1 (K whole steps, "

@@ -201,11 +201,10 @@ cgh_status cgh_host_wait_ticket(cgh_handle h, uint64_t ticket);
  * with phi = P_j r^2, r^2 = (x_h - x_j)^2 + (y_h - y_j)^2 (derivatives of
  * Eq. 1; dP_j/dz_j = -P_j/z_j).  Any of the three outputs may be NULL to
  * skip it.  method: CGH_DIRECT_FP32 (FP32, point-owned sums, deterministic),
- * CGH_SEP_FP32 (the same point-owned FP32 sums with cos(phi) and sin(phi)
- * expanded by angle addition into per-column sums of G cos, G sin of the
- * row angle and per-row sums of G cos, G sin of the column angle;
- * deterministic) or CGH_SEP_FP16X3 (two split-FP16 tensor-core GEMMs, G V and
- * G^T U, with the pixel sums fused into their epilogues).  Other methods:
+ * CGH_SEP_FP32 or CGH_SEP_FP16X3 (both: two tensor-core products, G V and
+ * G^T U, at the accuracy of CGH_SEP_FP32's forward -- every FP32 factor split
+ * into two FP16 numbers, partial sums added in FP32 -- with the pixel sums
+ * fused into their epilogues; deterministic).  Other methods:
  * CGH_ERR_INVALID_ARG.  Errors as cgh_forward. */
 cgh_status cgh_backward(cgh_handle h, const float *points, const float *A,
                         const float *z, int N, double lambda, double p,
@@ -360,14 +359,15 @@ cgh_status cgh_set_direct_schedule(cgh_handle h, int schedule);
  *                    a table kernel writing them to global memory and the
  *                    GEMM reading them back; same entry values bit for bit,
  *                    so the same hologram (single hologram forward only;
- *                    the adjoint and cgh_batch take CGH_GEMM_PAIRS then);
+ *                    cgh_batch takes CGH_GEMM_PAIRS then);
  *   CGH_GEMM_AUTO:   the handle's tuned plan for the size (cgh_tune), else
- *                    CTA pairs for single holograms and adjoints of more
+ *                    CTA pairs for single holograms of more
  *                    than 128 rows, one-CTA tiles otherwise and for
  *                    cgh_batch (whose persistent work list balances better
  *                    with the smaller items).
  * Every mode computes the same products with FP32 accumulation; results
- * agree to rounding. */
+ * agree to rounding.  The adjoint has one tiling of its own (CTA pairs) and
+ * does not depend on this setting. */
 typedef enum {
     CGH_GEMM_AUTO = 0,
     CGH_GEMM_SINGLE = 1,
@@ -453,14 +453,14 @@ typedef enum {
     CGH_K_SEP_TABLES = 4,     /* U / V exponential tables               */
     CGH_K_GEMM = 5,           /* tcgen05 GEMM (forward)                 */
     CGH_K_BWD_DIRECT = 6,     /* direct adjoint point-owned sums        */
-    CGH_K_BWD_GEMM = 7,       /* separable adjoint GEMMs + fused sums   */
+    CGH_K_BWD_GEMM = 7,       /* separable adjoint products + fused sums */
     CGH_K_BWD_REDUCE = 8,     /* adjoint partial-sum reduction          */
     CGH_K_BATCH = 9,          /* direct batch (its whole graph)         */
     CGH_K_AUX = 10,           /* small helpers (conversions, fills)     */
     CGH_K_BATCH_SEP = 11,     /* separable batch (its whole graph)      */
     CGH_K_RECUR = 12,         /* Eq. 2 recurrence kernel                */
     CGH_K_SIMT = 13,          /* FP32 separable product (tensor cores)  */
-    CGH_K_BWD_SIMT = 14,      /* FP32 separable adjoint (FMA pipe)      */
+    CGH_K_BWD_SIMT = 14,      /* the same, method CGH_SEP_FP32           */
     CGH_K_COUNT = 16
 } cgh_kernel_id;
 

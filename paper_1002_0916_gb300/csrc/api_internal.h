@@ -129,6 +129,10 @@ struct cgh_ctx {
     cgh_status forward_sep32(const float *points, const float *A, const float *z, int N,
                              double lambda, double p, int Nx, int Ny, float *out,
                              cudaStream_t s);
+    // timer: the cgh_kernel_id of its product launch
+    cgh_status backward_sep32(const float *points, const float *A, const float *z, int N,
+                              double lambda, double p, int Nx, int Ny, const float *G,
+                              float *gpts, float *gA, float *gz, int timer, cudaStream_t s);
     cgh_status forward_separable(const float *points, const float *A,
                                  const float *z, int N, double lambda, double p,
                                  int Nx, int Ny, float *out, int method,

@@ -314,22 +314,8 @@ cudaError_t launch_umma_gen(const PointRec *rec, int N, int Npad, int kind, int 
                             unsigned *status, cudaStream_t s);
 cudaError_t launch_umma_pair(const GemmOperands &op, int bnp, unsigned *status,
                              cudaStream_t s);
-struct AdjEpiArgs;
-cudaError_t launch_umma_pair_adjoint(const GemmOperands &op, const AdjEpiArgs &ea,
-                                     int sms, unsigned *status, cudaStream_t s,
-                                     int *tile_n);
 cudaError_t launch_umma_gemm(const GemmOperands &op, unsigned *status,
                              cudaStream_t s);
-// Split GEMM whose epilogue reduces the adjoint sums over its columns into
-// part[n_tile][npad][3] (see umma_epi.cuh); rows are k = 2j + {0: cos, 1:
-// sin}.  *tile_n receives the column width of one n_tile (128, or a CTA-pair
-// width >= 160), so part needs ceil(N / 128) tiles at most.
-cudaError_t launch_umma_adjoint(const GemmOperands &op, const PointRec *rec,
-                                const float *points, int npoints, int npad,
-                                int axis, float *part, unsigned *status,
-                                cudaStream_t s, int *tile_n);
-int umma_tile_n();
-
 // separable.cu: U / V tables of the separable form, the point records
 // built inside the kernel from the caller's points.
 cudaError_t launch_sep_tables(const PointSource &src, int Npad, int Nx, int Ny, int Kp,

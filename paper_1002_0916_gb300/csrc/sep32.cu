@@ -45,47 +45,19 @@
 
 #include "api_internal.h"
 #include "common.cuh"
-#include "cos_poly.h"
 #include "point_rec.cuh"
+#include "sep32.cuh"
 #include "sep_table.cuh"
 #include "umma.cuh"
 #include "umma_pair.cuh"
 
 namespace cgh {
 
+int sm_count_of_current_device();
 bool make_gemm_map(CUtensorMap *m, const void *base, long long inner, long long rows,
                    long long ld, int box_rows, bool bf16);
 
 // ---------------------------------------------------------------- tables
-// R entries are scaled by 2^S32_EXP, a block's L entries to below it.
-constexpr int S32_EXP = 14;
-constexpr float S32_R_SCALE = 16384.0f;
-
-// sin and cos of a 0.64 fixed-point phase: the nearest quarter turn is taken
-// off in fixed point, so that the remainder x (quarter turns, |x| <= 1/2)
-// rounds to FP32 with a relative error (2^-25) however large the phase, then
-// polynomials (cos_poly.h), a swap and two sign bits.  The hardware sincos of
-// the rounded angle would be cheaper but has an absolute error of 2^-21, more
-// than the rest of this path together; sincospif of the rounded turn took 9.1
-// us against 7.6 (tables at 1023x767x1999) and left more error in the hologram
-// (1.76e-7 against 1.62e-7 at 1920x1024x1024).
-__device__ __forceinline__ void sincos_fixed(uint64_t ph, float &s, float &c) {
-    const float x = (float)(int)(uint32_t)(ph >> 30) * TURN_PER_U32;
-    const uint32_t t = (uint32_t)(ph >> 32) + 0x20000000u;  // top 2 bits: the quadrant
-    const float z = x * x;
-    float ps = fmaf(QSIN_C3, z, QSIN_C2), pc = fmaf(QCOS_C4, z, QCOS_C3);
-    ps = fmaf(ps, z, QSIN_C1);
-    pc = fmaf(pc, z, QCOS_C2);
-    ps = fmaf(ps, z, QSIN_C0);
-    pc = fmaf(pc, z, QCOS_C1);
-    ps *= x;
-    pc = fmaf(pc, z, QCOS_C0);
-    const bool odd = (t & 0x40000000u) != 0;
-    const float a = odd ? ps : pc, b = odd ? pc : ps;
-    c = __uint_as_float(__float_as_uint(a) ^ ((t + 0x40000000u) & 0x80000000u));
-    s = __uint_as_float(__float_as_uint(b) ^ (t & 0x80000000u));
-}
-
 // One point's walk along an axis: the exact fixed-point phase and its first
 // and second differences (Eq. 2, modulo one turn), and the factors of its
 // cosine and sine entries (0 for a padding point).
@@ -182,7 +154,8 @@ constexpr int S32_EPI_WARPS = 8;
 constexpr int S32_THREADS = 64 + 32 * S32_EPI_WARPS;
 
 struct Sep32Args {
-    int M, N, K;
+    int units, tiles_m, tiles_n, KB;  // forward: tiles, K blocks; units of either
+    int M, N;
     float *D;
     long long ldd;
     const float *scale;  // one factor per K block
@@ -226,14 +199,177 @@ __device__ __forceinline__ void sep32_promote(uint32_t taddr, int nu, float f,
     }
 }
 
-// Grid: x = 2 x column tiles, y = row tiles of 256, z = K slices; clusters of
-// two CTAs along x.
-template <int BNP, int STAGES>
+// Forward epilogue: with K slices, publish the partial tile ([column / 4]
+// [row][4 columns]: 16-byte stores of neighbouring rows are consecutive),
+// count in, and let the last slice add all of them; then store the row,
+// clipped to the frame.  Called by every epilogue warp.
+template <int BNP>
+__device__ __forceinline__ void sep32_store(const Sep32Args &g, bool ok, int mt, int nt, int slice,
+                                            int rank, int half, int lrow, int m0, int np0,
+                                            int *s_last, float (&acc)[Sep32Cols<BNP>::U0 * 16]) {
+    using C = Sep32Cols<BNP>;
+    constexpr int BM = 128;
+    const int nu = half ? C::U1 : C::U0, c0 = half * C::U0 * 16;
+    bool store = ok;
+    if (g.S > 1) {
+        const size_t tile = (size_t)mt * g.tiles_n + nt;
+        const size_t plane = (size_t)BM * BNP;
+        float *dst = g.part + ((tile * g.S + slice) * 2 + rank) * plane;
+        if (ok) {
+#pragma unroll
+            for (int c = 0; c < C::U0 * 16; c += 4)
+                if (c < nu * 16)
+                    *reinterpret_cast<float4 *>(dst + ((size_t)((c0 + c) >> 2) * BM + lrow) * 4) =
+                        make_float4(acc[c], acc[c + 1], acc[c + 2], acc[c + 3]);
+        }
+        __threadfence();
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * S32_EPI_WARPS) : "memory");
+        if (threadIdx.x == 64)
+            *s_last = atomicAdd(&g.count[tile * 2 + rank], 1u) == (unsigned)(g.S - 1);
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * S32_EPI_WARPS) : "memory");
+        store = ok && *(volatile int *)s_last;
+        if (store) {
+            __threadfence();
+#pragma unroll
+            for (int c = 0; c < C::U0 * 16; ++c) acc[c] = 0.0f;
+            for (int z = 0; z < g.S; ++z) {
+                const float *src = g.part + ((tile * g.S + z) * 2 + rank) * plane;
+#pragma unroll
+                for (int c = 0; c < C::U0 * 16; c += 4)
+                    if (c < nu * 16) {
+                        const float4 v = __ldcg(reinterpret_cast<const float4 *>(
+                            src + ((size_t)((c0 + c) >> 2) * BM + lrow) * 4));
+                        acc[c] += v.x;
+                        acc[c + 1] += v.y;
+                        acc[c + 2] += v.z;
+                        acc[c + 3] += v.w;
+                    }
+            }
+        }
+    }
+    const int row = m0 + lrow;
+    if (!store || row >= g.M) return;
+    float *drow = g.D + (long long)row * g.ldd;
+#pragma unroll
+    for (int c = 0; c < C::U0 * 16; c += 4) {
+        const int col = np0 + c0 + c;
+        if (c >= nu * 16 || col >= g.N) break;
+        if (g.vec && col + 4 <= g.N) {
+            *reinterpret_cast<float4 *>(drow + col) =
+                make_float4(acc[c], acc[c + 1], acc[c + 2], acc[c + 3]);
+        } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (col + e < g.N) drow[col + e] = acc[c + e];
+        }
+    }
+}
+
+// Adjoint epilogue.  GEMM row k = 2j + c (c = 0: cosine row, 1: sine row of
+// point j); with (W_c, W_s) = rows 2j, 2j + 1 of D at column u, (cu, su) =
+// cos, sin of theta_axis(u, j) and d = u - u_j, sum over the columns
+//     C = cu W_c - su W_s,   S = su W_c + cu W_s
+// with weights 1 for C and d, d^2 for S.  The two lanes of a point hold the
+// two rows: the even lane takes the first half of the warp's columns, the odd
+// lane the second, and each sends the other the value it lacks.  With the odd
+// lane's phase a quarter turn ahead, (c', s') its cosine and sine, and r the
+// received value (negated when it comes from the odd lane), both lanes compute
+// C = own c' + r s' and -S = r c' - own s'.  d = i + delta with i the column's
+// index in the lane's run: the sums are taken with i and shifted at the end.
+// Columns beyond the frame have zero operands, hence W = 0.
+// (Reading the weights from the split tables instead of stepping the phase by
+// Eq. 2 and taking sincos_fixed cost 7.8 us a tile, waiting on L2.)
+template <int U0>
+__device__ __forceinline__ void adj32_reduce(const Adj32Prod &pr, const Adj32Args &ga, int t,
+                                             int row, int n0, const float (&acc)[U0 * 16]) {
+    constexpr int RUN = U0 * 8;  // columns per lane
+    const int j = row >> 1;
+    const bool odd = (row & 1) != 0, valid = j < ga.n;
+    const int u0 = n0 + (odd ? RUN : 0);
+    uint64_t ph = 0, d = 0, dd = 0;
+    if (valid) {
+        const PointRec &r = ga.rec[j];
+        const uint64_t b = pr.axis ? r.by : r.bx;
+        ph = axis_phase(r.c, b, pr.axis ? r.ay : r.ax, u0) + (odd ? 1ull << 62 : 0ull);
+        d = r.c * (uint64_t)(2 * (int64_t)u0 + 1) - b;
+        dd = 2 * r.c;
+    }
+    float C = 0.0f, S0 = 0.0f, S1 = 0.0f, S2 = 0.0f;
+#pragma unroll
+    for (int i = 0; i < RUN; ++i) {
+        const float own = odd ? acc[RUN + i] : acc[i];
+        const float r = __shfl_xor_sync(0xffffffffu, odd ? -acc[i] : acc[RUN + i], 1);
+        float s, c;
+        sincos_fixed(ph, s, c);
+        ph += d;
+        d += dd;
+        C = fmaf(own, c, fmaf(r, s, C));
+        const float v = fmaf(own, s, -r * c);
+        S0 += v;
+        S1 = fmaf(v, (float)i, S1);
+        S2 = fmaf(v, (float)(i * i), S2);
+    }
+    const float delta = valid ? (float)u0 - ga.points[2 * j + pr.axis] : 0.0f;
+    S2 = fmaf(delta, fmaf(delta, S0, 2.0f * S1), S2);
+    S1 = fmaf(delta, S0, S1);
+    C += __shfl_xor_sync(0xffffffffu, C, 1);
+    S1 += __shfl_xor_sync(0xffffffffu, S1, 1);
+    S2 += __shfl_xor_sync(0xffffffffu, S2, 1);
+    if (valid && !odd) {
+        float *p = pr.part + ((size_t)t * ga.npad + j) * 3;
+        p[0] = C;
+        p[1] = S1;
+        p[2] = S2;
+    }
+}
+
+struct Sep32Maps {
+    CUtensorMap A, B, A2, B2;  // hi and lo planes: M x K and N x K, K-major
+};
+
+// One unit of work: a tile of one product over one K slice.
+struct Sep32Unit {
+    int which, mt, nt, slice, kb0, nkb;
+};
+
+template <bool ADJ>
+__device__ __forceinline__ Sep32Unit sep32_unit(int u, const Sep32Args &g, const Adj32Args &ga) {
+    Sep32Unit w;
+    int tn = g.tiles_n, tm = g.tiles_m, S = g.S, KB = g.KB;
+    w.which = 0;
+    if constexpr (ADJ) {
+        tm = ga.tiles_m;
+        w.which = u >= ga.p[0].units;
+        if (w.which) u -= ga.p[0].units;
+        tn = w.which ? ga.p[1].tiles_n : ga.p[0].tiles_n;
+        S = w.which ? ga.p[1].S : ga.p[0].S;
+        KB = w.which ? ga.p[1].KB : ga.p[0].KB;
+    }
+    w.nt = u % tn;
+    u /= tn;
+    w.mt = u % tm;
+    w.slice = u / tm;
+    w.kb0 = (int)((long long)KB * w.slice / S);
+    w.nkb = (int)((long long)KB * (w.slice + 1) / S) - w.kb0;
+    return w;
+}
+
+// The r-th unit of cluster c of n: round by round, every other round in
+// reverse order, so that units sorted longest first spread evenly; units or
+// more: none in this round.
+__device__ __forceinline__ int sep32_unit_index(int r, int c, int n) {
+    return r * n + ((r & 1) ? n - 1 - c : c);
+}
+
+// Persistent: clusters of two CTAs (one per SM) take the units in
+// sep32_unit_index order; loads and MMAs run ahead into the next unit while
+// the epilogue of the last one finishes.  ADJ: both products of the adjoint
+// in one list, the longer K first.
+template <int BNP, int STAGES, bool ADJ>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(S32_THREADS, 1)
-sep32_pair_kernel(const __grid_constant__ CUtensorMap tA,
-                  const __grid_constant__ CUtensorMap tB,
-                  const __grid_constant__ CUtensorMap tA2,
-                  const __grid_constant__ CUtensorMap tB2, Sep32Args g, uint32_t idesc) {
+sep32_pair_kernel(const __grid_constant__ Sep32Maps maps0,
+                  const __grid_constant__ Sep32Maps maps1, const __grid_constant__ Sep32Args g,
+                  const __grid_constant__ Adj32Args ga, uint32_t idesc) {
     using S = PairShape<BNP, true, STAGES>;
     using C = Sep32Cols<BNP>;
     extern __shared__ uint8_t smem_raw[];
@@ -248,12 +384,7 @@ sep32_pair_kernel(const __grid_constant__ CUtensorMap tA,
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const uint32_t rank = umma2::cluster_rank();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = blockIdx.y * 2 * S::BM + (int)rank * S::BM;  // this CTA's rows
-    const int np0 = (blockIdx.x >> 1) * BNP;                     // the pair's columns
-    const int nb = np0 + (int)rank * S::BNH;                     // this CTA's B rows
-    const int KB = (g.K + S::BK - 1) / S::BK;
-    const int kb0 = (int)((long long)KB * blockIdx.z / g.S);
-    const int nkb = (int)((long long)KB * (blockIdx.z + 1) / g.S) - kb0;
+    const int cl = blockIdx.x >> 1, ncl = gridDim.x >> 1;
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
@@ -266,10 +397,10 @@ sep32_pair_kernel(const __grid_constant__ CUtensorMap tA,
             mbar_init(&acc_empty[b], 2 * S32_EPI_WARPS);
         }
         mbar_fence_init();
-        umma::prefetch_tmap(&tA);
-        umma::prefetch_tmap(&tB);
-        umma::prefetch_tmap(&tA2);
-        umma::prefetch_tmap(&tB2);
+        umma::prefetch_tmap(&maps0.A);
+        umma::prefetch_tmap(&maps0.B);
+        umma::prefetch_tmap(&maps0.A2);
+        umma::prefetch_tmap(&maps0.B2);
     }
     if (warp == 1) {
         umma2::tmem_alloc2(&tmem_base, 512);
@@ -283,71 +414,83 @@ sep32_pair_kernel(const __grid_constant__ CUtensorMap tA,
 
     if (warp == 0 && lane == 0) {
         // ------------------------------------------ producer (both CTAs)
-        int issued = 0;
-        for (int i = 0; i < nkb; ++i) {
-            const int s = i % STAGES;
-            if (i >= STAGES &&
-                !mbar_wait_bounded(&empty[s], (uint32_t)(((i / STAGES) - 1) & 1))) {
-                abort_flag = 1;
-                set_status(g.status, DEV_TIMEOUT);
-            }
-            if (abort_flag) break;
-            uint8_t *st = smem + (size_t)s * S::STAGE_BYTES;
-            // the even CTA's barrier counts the bytes of both CTAs' loads
-            if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * S::STAGE_BYTES);
-            const uint32_t bar = umma2::map_to_rank(&full[s], 0);
-            const int k = (kb0 + i) * S::BK;
-            umma2::tma_load_2d_pair(st, &tA, k, m0, bar);
-            umma2::tma_load_2d_pair(st + S::A_BYTES, &tB, k, nb, bar);
-            umma2::tma_load_2d_pair(st + S::A_BYTES + S::B_BYTES, &tA2, k, m0, bar);
-            umma2::tma_load_2d_pair(st + 2 * S::A_BYTES + S::B_BYTES, &tB2, k, nb, bar);
-            ++issued;
-        }
-        if (abort_flag && rank == 0) {
-            // let the stages' copies land before shared memory goes (the odd
-            // CTA leaves only after the closing cluster barrier)
-            for (int i = issued - STAGES < 0 ? 0 : issued - STAGES; i < issued; ++i)
-                mbar_wait_bounded(&full[i % STAGES], (uint32_t)((i / STAGES) & 1));
-        } else if (!abort_flag) {
-            // wait (bounded) for the commits of the last stages, so that no
-            // arrive is in flight when the CTA's shared memory passes on
-            for (int i = nkb - STAGES < 0 ? 0 : nkb - STAGES; i < nkb; ++i)
-                mbar_wait_bounded(&empty[i % STAGES], (uint32_t)((i / STAGES) & 1));
-        }
-    } else if (warp == 1 && lane == 0) {
-        if (rank == 0) {
-            // ---------------------------------------- MMA issuer (even CTA)
-            for (int i = 0; i < nkb; ++i) {
-                const int s = i % STAGES, b = i % C::NBUF;
-                if (!mbar_wait_bounded(&acc_empty[b],
-                                                 (uint32_t)(((i / C::NBUF) & 1) ^ 1)) ||
-                    !mbar_wait_bounded(&full[s], (uint32_t)((i / STAGES) & 1))) {
+        unsigned n = 0;  // K blocks issued
+        for (int r = 0; r * ncl < g.units && !abort_flag; ++r) {
+            const int u = sep32_unit_index(r, cl, ncl);
+            if (u >= g.units) break;
+            const Sep32Unit w = sep32_unit<ADJ>(u, g, ga);
+            const Sep32Maps *maps = w.which ? &maps1 : &maps0;
+            const int m0 = w.mt * 2 * S::BM + (int)rank * S::BM;  // this CTA's rows
+            const int nb = w.nt * BNP + (int)rank * S::BNH;       // its B rows
+            for (int i = 0; i < w.nkb; ++i, ++n) {
+                const int s = (int)(n % STAGES);
+                if (n >= STAGES &&
+                    !mbar_wait_bounded(&empty[s], ((n / STAGES) - 1) & 1)) {
                     abort_flag = 1;
                     set_status(g.status, DEV_TIMEOUT);
                 }
                 if (abort_flag) break;
-                umma::fence_after_sync();
-                const uint32_t a = smem_u32(smem + (size_t)s * S::STAGE_BYTES);
-                const uint32_t bb = a + S::A_BYTES;
-                const uint32_t a2 = bb + S::B_BYTES, b2 = a2 + S::A_BYTES;
-                const uint64_t ad = umma::sw128_kmajor_desc(a);
-                const uint64_t bd = umma::sw128_kmajor_desc(bb);
-                const uint64_t ad2 = umma::sw128_kmajor_desc(a2);
-                const uint64_t bd2 = umma::sw128_kmajor_desc(b2);
-                const uint32_t d = tmem + (uint32_t)b * C::STRIDE;
-                // the small cross products first: the sum's low bits are
-                // dropped only by the four hi*hi steps
+                uint8_t *st = smem + (size_t)s * S::STAGE_BYTES;
+                // the even CTA's barrier counts the bytes of both CTAs' loads
+                if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * S::STAGE_BYTES);
+                const uint32_t bar = umma2::map_to_rank(&full[s], 0);
+                const int k = (w.kb0 + i) * S::BK;
+                umma2::tma_load_2d_pair(st, &maps->A, k, m0, bar);
+                umma2::tma_load_2d_pair(st + S::A_BYTES, &maps->B, k, nb, bar);
+                umma2::tma_load_2d_pair(st + S::A_BYTES + S::B_BYTES, &maps->A2, k, m0, bar);
+                umma2::tma_load_2d_pair(st + 2 * S::A_BYTES + S::B_BYTES, &maps->B2, k, nb, bar);
+            }
+        }
+        const unsigned lo = n > STAGES ? n - STAGES : 0;
+        if (abort_flag && rank == 0) {
+            // let the stages' copies land before shared memory goes (the odd
+            // CTA leaves only after the closing cluster barrier)
+            for (unsigned i = lo; i < n; ++i) mbar_wait_bounded(&full[i % STAGES], (i / STAGES) & 1);
+        } else if (!abort_flag) {
+            // wait (bounded) for the commits of the last stages, so that no
+            // arrive is in flight when the CTA's shared memory passes on
+            for (unsigned i = lo; i < n; ++i)
+                mbar_wait_bounded(&empty[i % STAGES], (i / STAGES) & 1);
+        }
+    } else if (warp == 1 && lane == 0) {
+        if (rank == 0) {
+            // ---------------------------------------- MMA issuer (even CTA)
+            unsigned n = 0;
+            for (int r = 0; r * ncl < g.units && !abort_flag; ++r) {
+                const int u = sep32_unit_index(r, cl, ncl);
+                if (u >= g.units) break;
+                const int nkb = sep32_unit<ADJ>(u, g, ga).nkb;
+                for (int i = 0; i < nkb; ++i, ++n) {
+                    const int s = (int)(n % STAGES), b = (int)(n % C::NBUF);
+                    if (!mbar_wait_bounded(&acc_empty[b], ((n / C::NBUF) & 1) ^ 1) ||
+                        !mbar_wait_bounded(&full[s], (n / STAGES) & 1)) {
+                        abort_flag = 1;
+                        set_status(g.status, DEV_TIMEOUT);
+                    }
+                    if (abort_flag) break;
+                    umma::fence_after_sync();
+                    const uint32_t a = smem_u32(smem + (size_t)s * S::STAGE_BYTES);
+                    const uint32_t bb = a + S::A_BYTES;
+                    const uint32_t a2 = bb + S::B_BYTES, b2 = a2 + S::A_BYTES;
+                    const uint64_t ad = umma::sw128_kmajor_desc(a);
+                    const uint64_t bd = umma::sw128_kmajor_desc(bb);
+                    const uint64_t ad2 = umma::sw128_kmajor_desc(a2);
+                    const uint64_t bd2 = umma::sw128_kmajor_desc(b2);
+                    const uint32_t d = tmem + (uint32_t)b * C::STRIDE;
+                    // the small cross products first: the sum's low bits are
+                    // dropped only by the four hi*hi steps
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    umma2::mma2_f16(d, ad + 2 * kk, bd2 + 2 * kk, idesc, kk != 0);
+                    for (int kk = 0; kk < 4; ++kk)
+                        umma2::mma2_f16(d, ad + 2 * kk, bd2 + 2 * kk, idesc, kk != 0);
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    umma2::mma2_f16(d, ad2 + 2 * kk, bd + 2 * kk, idesc, 1);
+                    for (int kk = 0; kk < 4; ++kk)
+                        umma2::mma2_f16(d, ad2 + 2 * kk, bd + 2 * kk, idesc, 1);
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    umma2::mma2_f16(d, ad + 2 * kk, bd + 2 * kk, idesc, 1);
-                umma2::commit2(&empty[s], 0x3);
-                umma2::commit2(&acc_full[b], 0x3);
+                    for (int kk = 0; kk < 4; ++kk)
+                        umma2::mma2_f16(d, ad + 2 * kk, bd + 2 * kk, idesc, 1);
+                    umma2::commit2(&empty[s], 0x3);
+                    umma2::commit2(&acc_full[b], 0x3);
+                }
             }
         }
     } else if (warp >= 2) {
@@ -359,83 +502,41 @@ sep32_pair_kernel(const __grid_constant__ CUtensorMap tA,
         const int lrow = q * 32 + lane;
         const uint32_t t0 = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0;
         const uint32_t lead_empty = umma2::map_to_rank(&acc_empty[0], 0);
-        float acc[C::U0 * 16];
-#pragma unroll
-        for (int i = 0; i < C::U0 * 16; ++i) acc[i] = 0.0f;
         bool ok = true;
-        float f_next = __ldg(g.scale + kb0);
-        for (int i = 0; i < nkb; ++i) {
-            const int b = i % C::NBUF;
-            const float f = f_next;
-            f_next = __ldg(g.scale + kb0 + (i + 1 < nkb ? i + 1 : i));
-            ok = __all_sync(0xffffffffu, mbar_wait_bounded(
-                                             &acc_full[b], (uint32_t)((i / C::NBUF) & 1)));
-            umma::fence_after_sync();
-            if (!ok || abort_flag) {
+        unsigned n = 0;
+        for (int r = 0; r * ncl < g.units; ++r) {
+            const int u = sep32_unit_index(r, cl, ncl);
+            if (u >= g.units) break;
+            const Sep32Unit w = sep32_unit<ADJ>(u, g, ga);
+            float acc[C::U0 * 16];
+#pragma unroll
+            for (int i = 0; i < C::U0 * 16; ++i) acc[i] = 0.0f;
+            float f_next = ADJ ? 1.0f : __ldg(g.scale + w.kb0);
+            for (int i = 0; i < w.nkb && ok; ++i, ++n) {
+                const int b = (int)(n % C::NBUF);
+                const float f = f_next;
+                if (!ADJ) f_next = __ldg(g.scale + w.kb0 + (i + 1 < w.nkb ? i + 1 : i));
+                ok = __all_sync(0xffffffffu,
+                                mbar_wait_bounded(&acc_full[b], (n / C::NBUF) & 1));
+                umma::fence_after_sync();
                 if (!ok) set_status(g.status, DEV_TIMEOUT);
-                ok = false;
-                break;
+                ok = __all_sync(0xffffffffu, ok && !abort_flag);
+                if (!ok) break;
+                sep32_promote<C::U0>(t0 + (uint32_t)b * C::STRIDE, nu, f, acc);
+                umma::fence_before_sync();
+                __syncwarp();
+                if (lane == 0) umma2::arrive_pair(lead_empty + (uint32_t)b * 8u);
             }
-            sep32_promote<C::U0>(t0 + (uint32_t)b * C::STRIDE, nu, f, acc);
-            umma::fence_before_sync();
-            __syncwarp();
-            if (lane == 0) umma2::arrive_pair(lead_empty + (uint32_t)b * 8u);
-        }
-        bool store = ok;
-        if (g.S > 1) {
-            // publish the partial tile ([column / 4][row][4 columns]: 16-byte
-            // stores of neighbouring rows are consecutive), then count in
-            const size_t tile = (size_t)blockIdx.y * (gridDim.x >> 1) + (blockIdx.x >> 1);
-            const size_t plane = (size_t)S::BM * BNP;
-            float *dst = g.part + ((tile * g.S + blockIdx.z) * 2 + rank) * plane;
-            if (ok) {
-#pragma unroll
-                for (int c = 0; c < C::U0 * 16; c += 4)
-                    if (c < nu * 16)
-                        *reinterpret_cast<float4 *>(
-                            dst + ((size_t)((c0 + c) >> 2) * S::BM + lrow) * 4) =
-                            make_float4(acc[c], acc[c + 1], acc[c + 2], acc[c + 3]);
-            }
-            __threadfence();
-            asm volatile("bar.sync 1, %0;" ::"n"(32 * S32_EPI_WARPS) : "memory");
-            if (threadIdx.x == 64)
-                s_last = atomicAdd(&g.count[tile * 2 + rank], 1u) == (unsigned)(g.S - 1);
-            asm volatile("bar.sync 1, %0;" ::"n"(32 * S32_EPI_WARPS) : "memory");
-            store = ok && s_last;
-            if (store) {
-                __threadfence();
-#pragma unroll
-                for (int c = 0; c < C::U0 * 16; ++c) acc[c] = 0.0f;
-                for (int z = 0; z < g.S; ++z) {
-                    const float *src = g.part + ((tile * g.S + z) * 2 + rank) * plane;
-#pragma unroll
-                    for (int c = 0; c < C::U0 * 16; c += 4)
-                        if (c < nu * 16) {
-                            const float4 v = __ldcg(reinterpret_cast<const float4 *>(
-                                src + ((size_t)((c0 + c) >> 2) * S::BM + lrow) * 4));
-                            acc[c] += v.x;
-                            acc[c + 1] += v.y;
-                            acc[c + 2] += v.z;
-                            acc[c + 3] += v.w;
-                        }
-                }
-            }
-        }
-        const int row = m0 + lrow;
-        if (store && row < g.M) {
-            float *drow = g.D + (long long)row * g.ldd;
-#pragma unroll
-            for (int c = 0; c < C::U0 * 16; c += 4) {
-                const int col = np0 + c0 + c;
-                if (c >= nu * 16 || col >= g.N) break;
-                if (g.vec && col + 4 <= g.N) {
-                    *reinterpret_cast<float4 *>(drow + col) =
-                        make_float4(acc[c], acc[c + 1], acc[c + 2], acc[c + 3]);
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        if (col + e < g.N) drow[col + e] = acc[c + e];
-                }
+            const int m0 = w.mt * 2 * S::BM + (int)rank * S::BM;
+            if constexpr (ADJ) {
+                static_assert(C::U0 == C::U1, "equal column halves");
+                if (ok)
+                    adj32_reduce<C::U0>(ga.p[w.which], ga, (w.slice * (w.which ? ga.p[1].tiles_n : ga.p[0].tiles_n) + w.nt) * 2 + half,
+                                        m0 + lrow, w.nt * BNP + c0, acc);
+            } else {
+                // (every warp, also after a timeout: it meets at barriers)
+                sep32_store<BNP>(g, ok, w.mt, w.nt, w.slice, (int)rank, half, lrow, m0,
+                                 w.nt * BNP, &s_last, acc);
             }
         }
     }
@@ -484,21 +585,19 @@ static Sep32Plan sep32_plan(int M, int N, int KB, int sms) {
     return best;
 }
 
-struct Sep32Operands {
-    const __half *A_hi, *A_lo, *B_hi, *B_lo;
-    long long lda, ldb;
-};
+template <int BNP>
+static bool make_sep32_maps(Sep32Maps *m, const Sep32Operands &op, int M, int N, int K) {
+    return make_gemm_map(&m->A, op.A_hi, K, M, op.lda, 128, false) &&
+           make_gemm_map(&m->B, op.B_hi, K, N, op.ldb, BNP / 2, false) &&
+           make_gemm_map(&m->A2, op.A_lo, K, M, op.lda, 128, false) &&
+           make_gemm_map(&m->B2, op.B_lo, K, N, op.ldb, BNP / 2, false);
+}
 
-template <int BNP, int STAGES>
-static cudaError_t launch_sep32_t(const Sep32Operands &op, const Sep32Args &g, cudaStream_t s) {
+template <int BNP, int STAGES, bool ADJ>
+static cudaError_t launch_sep32_kernel(const Sep32Maps &m0, const Sep32Maps &m1,
+                                       const Sep32Args &g, const Adj32Args &ga, cudaStream_t s) {
     using S = PairShape<BNP, true, STAGES>;
-    CUtensorMap tA, tB, tA2, tB2;
-    if (!make_gemm_map(&tA, op.A_hi, g.K, g.M, op.lda, S::BM, false) ||
-        !make_gemm_map(&tB, op.B_hi, g.K, g.N, op.ldb, S::BNH, false) ||
-        !make_gemm_map(&tA2, op.A_lo, g.K, g.M, op.lda, S::BM, false) ||
-        !make_gemm_map(&tB2, op.B_lo, g.K, g.N, op.ldb, S::BNH, false))
-        return cudaErrorInvalidValue;
-    auto kern = sep32_pair_kernel<BNP, STAGES>;
+    auto kern = sep32_pair_kernel<BNP, STAGES, ADJ>;
     static bool attr_set[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
@@ -508,9 +607,17 @@ static cudaError_t launch_sep32_t(const Sep32Operands &op, const Sep32Args &g, c
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
     }
-    dim3 grid(2 * ((g.N + BNP - 1) / BNP), (g.M + 255) / 256, g.S);
-    return launch_dependent(kern, grid, dim3(S32_THREADS), S::SMEM, s, tA, tB, tA2, tB2, g,
+    const int pairs = sm_count_of_current_device() / 2;
+    const int clusters = g.units < pairs ? g.units : pairs > 0 ? pairs : 1;
+    return launch_dependent(kern, dim3(2 * clusters), dim3(S32_THREADS), S::SMEM, s, m0, m1, g, ga,
                             umma::idesc_f16(2 * S::BM, BNP, false));
+}
+
+template <int BNP, int STAGES>
+static cudaError_t launch_sep32_t(const Sep32Operands &op, const Sep32Args &g, cudaStream_t s) {
+    Sep32Maps m;
+    if (!make_sep32_maps<BNP>(&m, op, g.M, g.N, 64 * g.KB)) return cudaErrorInvalidValue;
+    return launch_sep32_kernel<BNP, STAGES, false>(m, m, g, Adj32Args{}, s);
 }
 
 static cudaError_t launch_sep32(int bn, const Sep32Operands &op, const Sep32Args &g,
@@ -521,6 +628,67 @@ static cudaError_t launch_sep32(int bn, const Sep32Operands &op, const Sep32Args
     case 160: return launch_sep32_t<160, 4>(op, g, s);
     case 192: return launch_sep32_t<192, 4>(op, g, s);
     case 256: return launch_sep32_t<256, 3>(op, g, s);
+    }
+    return cudaErrorInvalidValue;
+}
+
+// ------------------------------------------------------ adjoint products
+static const int kAdj32BN[] = {192, 224, 256};
+
+// The width and slices with the least modelled time (the constants of
+// sep32_plan): units of both products on the SM pairs, longest first, so the
+// total spread over the pairs plus part of a unit, or the longest unit alone.
+// A unit's epilogue adds 1.8 us at 192 columns to 2.9 at 256 that the next
+// unit's MMAs do not cover (1920x1080x4096: 142 us at 224 columns, 149 at 256,
+// 159 at 192); a K slice costs nothing else, since the epilogue is linear in D
+// and every slice writes its own partial sums.
+Adj32Plan adj32_plan(int n, int Nx, int Ny, int sms) {
+    Adj32Plan best{256, {1, 1}};
+    double best_cost = 1e300;
+    const double pairs = sms / 2 > 0 ? sms / 2 : 1;
+    const long long mt = (2LL * n + 255) / 256;
+    const int N[2] = {Nx <= Ny ? Nx : Ny, Nx <= Ny ? Ny : Nx};  // columns; K = the other
+    const int KB[2] = {(N[1] + 63) / 64, (N[0] + 63) / 64};
+    for (int bn : kAdj32BN) {
+        const double tkb = 1.1 * (0.55 + 0.00125 * bn), epi = 0.011 * bn;
+        for (int S0 = 1; S0 <= 16 && S0 <= KB[0]; ++S0)
+            for (int S1 = 1; S1 <= 16 && S1 <= KB[1]; ++S1) {
+                const double n0 = (double)(mt * ((N[0] + bn - 1) / bn) * S0);
+                const double n1 = (double)(mt * ((N[1] + bn - 1) / bn) * S1);
+                const double u0 = ((KB[0] + S0 - 1) / S0) * tkb + epi;
+                const double u1 = ((KB[1] + S1 - 1) / S1) * tkb + epi;
+                const double longest = u0 > u1 ? u0 : u1;
+                const double total = (n0 * u0 + n1 * u1) / pairs;
+                const double cost = n0 + n1 <= pairs ? longest : total + 0.3 * longest;
+                if (cost < best_cost * 0.99) {
+                    best_cost = cost;
+                    best = Adj32Plan{bn, {S0, S1}};
+                }
+            }
+    }
+    return best;
+}
+
+template <int BNP, int STAGES>
+static cudaError_t launch_adj32_t(const Sep32Operands (&op)[2], const int (&N)[2],
+                                  const int (&K)[2], const Adj32Args &ga, unsigned *status,
+                                  cudaStream_t s) {
+    Sep32Maps m[2];
+    for (int i = 0; i < 2; ++i)
+        if (!make_sep32_maps<BNP>(&m[i], op[i], 2 * ga.n, N[i], K[i])) return cudaErrorInvalidValue;
+    Sep32Args g{};
+    g.status = status;
+    g.units = ga.p[0].units + ga.p[1].units;
+    return launch_sep32_kernel<BNP, STAGES, true>(m[0], m[1], g, ga, s);
+}
+
+cudaError_t launch_adj32(int bn, const Sep32Operands (&op)[2], const int (&N)[2],
+                         const int (&K)[2], const Adj32Args &ga, unsigned *status,
+                         cudaStream_t s) {
+    switch (bn) {
+    case 192: return launch_adj32_t<192, 4>(op, N, K, ga, status, s);
+    case 224: return launch_adj32_t<224, 3>(op, N, K, ga, status, s);
+    case 256: return launch_adj32_t<256, 3>(op, N, K, ga, status, s);
     }
     return cudaErrorInvalidValue;
 }
@@ -569,7 +737,10 @@ cgh_status cgh_ctx::forward_sep32(const float *points, const float *A, const flo
         Sep32Args g{};
         g.M = Ny;
         g.N = Nx;
-        g.K = Kp;
+        g.tiles_m = (Ny + 255) / 256;
+        g.tiles_n = (Nx + plan.bn - 1) / plan.bn;
+        g.units = g.tiles_m * g.tiles_n * plan.S;
+        g.KB = Kp / 64;
         g.D = out;
         g.ldd = Nx;
         g.scale = scale;

@@ -55,13 +55,13 @@ struct GemmShape {
     static_assert(SMEM <= 232448, "shared memory");
 };
 
-template <int BN, bool SPLIT, int STAGES, int MODE>
+template <int BN, bool SPLIT, int STAGES>
 __global__ void __launch_bounds__(192, 1)
 umma_gemm_kernel(const __grid_constant__ CUtensorMap tA,
                  const __grid_constant__ CUtensorMap tB,
                  const __grid_constant__ CUtensorMap tA2,
                  const __grid_constant__ CUtensorMap tB2, GemmArgs g,
-                 AdjEpiArgs ea, uint32_t idesc) {
+                 uint32_t idesc) {
     using S = GemmShape<BN, SPLIT, STAGES>;
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full[STAGES];
@@ -173,16 +173,13 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tA,
         // ----------------------------------------------------- epilogue
         const int q = warp & 3;  // the 32-lane quarter of TMEM this warp reads
         const int row = m0 + q * 32 + lane;
-        // warp-uniform, so the .sync.aligned TMEM loads and the shuffles
-        // below are executed by whole warps
+        // warp-uniform, so the .sync.aligned TMEM loads below are executed by
+        // whole warps
         const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&accum_bar, 0));
         umma::fence_after_sync();
         pdl_trigger();  // only the epilogue is left
         if (!ok) set_status(g.status, DEV_TIMEOUT);
-        if (MODE == 1 && ok && !abort_flag) {
-            adjoint_epilogue<BN, SPLIT, S::ACC1>(tmem + ((uint32_t)(q * 32) << 16),
-                                                 row, n0, g, ea, lane, blockIdx.x);
-        } else if (ok && !abort_flag) {
+        if (ok && !abort_flag) {
             const uint32_t t_row = tmem + ((uint32_t)(q * 32) << 16);
             float *drow = g.D + (long long)row * g.ldd;
             const bool vec = ((g.ldd & 3) == 0) && ((((uintptr_t)g.D) & 15) == 0);
@@ -274,9 +271,9 @@ bool make_f32_map(CUtensorMap *m, const void *base, long long inner, long long r
     return r == CUDA_SUCCESS;
 }
 
-template <int BN, bool SPLIT, int STAGES, int MODE>
-static cudaError_t launch_gemm_t(const GemmOperands &op, const AdjEpiArgs &ea,
-                                 unsigned *status, cudaStream_t s) {
+template <int BN, bool SPLIT, int STAGES>
+static cudaError_t launch_gemm_t(const GemmOperands &op, unsigned *status,
+                                 cudaStream_t s) {
     using S = GemmShape<BN, SPLIT, STAGES>;
     CUtensorMap tA, tB, tA2, tB2;
     if (!make_map(&tA, op.A_hi, op.K, op.M, op.lda, S::BM, op.bf16) ||
@@ -290,7 +287,7 @@ static cudaError_t launch_gemm_t(const GemmOperands &op, const AdjEpiArgs &ea,
         tA2 = tA;
         tB2 = tB;
     }
-    auto kern = umma_gemm_kernel<BN, SPLIT, STAGES, MODE>;
+    auto kern = umma_gemm_kernel<BN, SPLIT, STAGES>;
     static bool attr_set[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
@@ -304,7 +301,7 @@ static cudaError_t launch_gemm_t(const GemmOperands &op, const AdjEpiArgs &ea,
     dim3 grid((op.N + BN - 1) / BN, (op.M + S::BM - 1) / S::BM);
     const uint32_t idesc = umma::idesc_f16(S::BM, BN, op.bf16);
     return launch_dependent(kern, grid, dim3(192), S::SMEM, s, tA, tB, tA2, tB2, g,
-                            ea, idesc);
+                            idesc);
 }
 
 bool gemm_operands_ok(const GemmOperands &op) {
@@ -319,7 +316,7 @@ bool gemm_operands_ok(const GemmOperands &op) {
     return true;
 }
 
-static int sm_count_of_current_device() {
+int sm_count_of_current_device() {
     static int cache[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
@@ -381,34 +378,16 @@ cudaError_t launch_umma_gemm(const GemmOperands &op, unsigned *status,
         }
         return cudaSuccess;
     }
-    AdjEpiArgs ea{};
     const GemmPlan plan = gemm_plan(op.M, op.N, op.tiles, sm_count_of_current_device(),
                                     op.bf16 ? 0 : op.split ? 2 : 1, op.bn);
     if (plan.tiling == CGH_GEMM_PAIRS) return launch_umma_pair(op, plan.bn, status, s);
     const int bn = plan.bn;
     if (op.split)
-        return bn == 112 ? launch_gemm_t<112, true, 3, 0>(op, ea, status, s)
-                         : launch_gemm_t<128, true, 3, 0>(op, ea, status, s);
-    return bn == 112 ? launch_gemm_t<112, false, 6, 0>(op, ea, status, s)
-                     : launch_gemm_t<128, false, 6, 0>(op, ea, status, s);
+        return bn == 112 ? launch_gemm_t<112, true, 3>(op, status, s)
+                         : launch_gemm_t<128, true, 3>(op, status, s);
+    return bn == 112 ? launch_gemm_t<112, false, 6>(op, status, s)
+                     : launch_gemm_t<128, false, 6>(op, status, s);
 }
-
-cudaError_t launch_umma_adjoint(const GemmOperands &op, const PointRec *rec,
-                                const float *points, int npoints, int npad,
-                                int axis, float *part, unsigned *status,
-                                cudaStream_t s, int *tile_n) {
-    if (!gemm_operands_ok(op) || !op.split || (op.M & 1)) return cudaErrorInvalidValue;
-    AdjEpiArgs ea{rec, points, npoints, npad, axis, part};
-    const bool pairs = op.tiles == CGH_GEMM_PAIRS ||
-                       (op.tiles == CGH_GEMM_AUTO && op.M > 128);
-    if (pairs)
-        return launch_umma_pair_adjoint(op, ea, sm_count_of_current_device(), status, s,
-                                        tile_n);
-    *tile_n = 128;
-    return launch_gemm_t<128, true, 3, 1>(op, ea, status, s);
-}
-
-int umma_tile_n() { return 128; }
 
 // ------------------------------------------------------ grouped (batch)
 // Persistent grouped split GEMM: work items (problem, m tile, n tile) are
