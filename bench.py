@@ -46,7 +46,8 @@ FP32_PER_CLK_PER_SM = 128    # FP32 lanes of the FMA pipe per SM per clock
 # updates per clock per SM.  (Issue slots do not bind: packed FP32x2
 # instructions do two of these operations per slot.)
 MIXED_PP_PER_CLK_PER_SM = 16.0 * 14.0 / 9.0
-# The direct adjoint per update: hardware path = angle add, argument scale,
+# A direct adjoint with a sincos per update (the bound the angle-addition
+# adjoint no longer has): hardware path = angle add, argument scale,
 # sin + cos (2 MUFU), 3 accumulations (G cos, the column's and the row's
 # G sin: 5 FP32 ops); polynomial path = add, fold, square, 5 + 5 FMA (cos
 # and sin), times u, 3 accumulations (17 FP32 ops, no MUFU).  FMA-pipe
@@ -490,11 +491,9 @@ def alu_recipe(kernel, tile=None):
                 "update at 16/clk/SM (7 issue slots per update allow 18.3)",
                 lambda m, f: m, 1.0)
     if kernel == "bwd_direct":
-        return (ADJ_MIXED_PP_PER_CLK_PER_SM,
-                "FMA-pipe (128 FP32 ops/clk/SM) and MUFU (16 ops/clk/SM) limits of "
-                "the adjoint recipe: 5 FP32 ops + 2 MUFU (sin, cos) per hardware "
-                "update, 17 FP32 ops per polynomial update, best mix 11/28 -> 13.2 "
-                "updates/clk/SM", lambda m, f: (f + 6.0 * m) / 17.0, 2.0)
+        return (BWD_SIMT_PP_PER_CLK_PER_SM,
+                "FMA-pipe limit of the angle-addition adjoint: 4 FP32 "
+                "multiply-adds per update, 128 per clk/SM", lambda m, f: f / 4.0, 0.0)
     return (MIXED_PP_PER_CLK_PER_SM,
             "FMA-pipe (128 FP32 ops/clk/SM) and MUFU (16 cosines/clk/SM) limits "
             "of the direct recipe: 3 FP32 ops + 1 MUFU per MUFU-cosine update, "

@@ -20,7 +20,8 @@
 //      behind those, the tables U', V' with their point records;
 //   2. G to FP16 hi and lo in both orientations;
 //   3. both products, one grid;
-//   4. the partial sums added in FP64 in a fixed order, per-point factors.
+//   4. the partial sums added in a fixed order, per-point factors
+//      (backward.cu).
 // Points are taken in chunks whose tables stay within TABLE_BYTES.
 #include <cuda_fp16.h>
 #include <math.h>
@@ -165,7 +166,8 @@ adj32_convert_kernel(const float *__restrict__ G, int Nx, int Ny, const float *_
     const float s = m > 0.0f && isfinite(m)
                         ? scalbnf(1.0f, S32_EXP - 1 - (ilogbf(m) < -110 ? -110 : ilogbf(m)))
                         : 1.0f;
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *gscale = s;
+    // (the products' other factor is scaled by S32_R_SCALE)
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *gscale = s * S32_R_SCALE;
     const int bx = blockIdx.x * GC_T, by = blockIdx.y * GC_T;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -198,57 +200,6 @@ adj32_convert_kernel(const float *__restrict__ G, int Nx, int Ny, const float *_
         }
     }
     pdl_trigger();
-}
-
-// The partial sums of one chunk: one block per R32_PTS points, its slices of
-// threads take every R32_SL-th partial (FP64), slice 0 adds the slices in
-// order: deterministic.
-constexpr int R32_PTS = 32, R32_SL = 8;
-
-__global__ void __launch_bounds__(R32_PTS * R32_SL)
-adj32_sum_kernel(PointSource src, int npad, const float *__restrict__ part_x, int Tx,
-                 const float *__restrict__ part_y, int Ty, const float *__restrict__ gscale,
-                 float *__restrict__ gpts, float *__restrict__ gA, float *__restrict__ gz) {
-    __shared__ double part[R32_SL][5][R32_PTS];
-    const int lj = threadIdx.x % R32_PTS, sl = threadIdx.x / R32_PTS;
-    const int j = blockIdx.x * R32_PTS + lj;
-    pdl_wait();  // the partial sums come from the kernel before
-    double v[5] = {0, 0, 0, 0, 0};
-    if (j < src.N) {
-        for (int t = sl; t < Tx; t += R32_SL) {
-            const float *p = part_x + ((size_t)t * npad + j) * 3;
-            v[0] += p[0];
-            v[1] += p[1];
-            v[2] += p[2];
-        }
-        for (int t = sl; t < Ty; t += R32_SL) {
-            const float *p = part_y + ((size_t)t * npad + j) * 3;
-            v[3] += p[1];
-            v[4] += p[2];
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < 5; ++k) part[sl][k][lj] = v[k];
-    __syncthreads();
-    if (sl != 0 || j >= src.N) return;
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-        v[k] = 0;
-#pragma unroll
-        for (int q = 0; q < R32_SL; ++q) v[k] += part[q][k][lj];
-    }
-    const PointRec r =
-        make_point_rec(src.points, src.A, src.z, src.N, j, src.K, (unsigned *)nullptr);
-    const bool ok = r.Q32 > 0.0f;
-    const double inv = 1.0 / ((double)*gscale * S32_R_SCALE);
-    const double P = 6.283185307179586 * (double)r.Q32;
-    const double a = (double)r.A;
-    if (gA) gA[j] = ok ? (float)(v[0] * inv) : 0.0f;
-    if (gpts) {
-        gpts[2 * j] = ok ? (float)(2.0 * P * a * v[1] * inv) : 0.0f;
-        gpts[2 * j + 1] = ok ? (float)(2.0 * P * a * v[3] * inv) : 0.0f;
-    }
-    if (gz) gz[j] = ok ? (float)(P * a / (double)src.z[j] * (v[2] + v[4]) * inv) : 0.0f;
 }
 
 }  // namespace cgh
@@ -358,11 +309,11 @@ cgh_status cgh_ctx::backward_sep32(const float *points, const float *A, const fl
         {
             TimedLaunch tl(this, CGH_K_BWD_REDUCE, s);
             const int ix = axis[0] == 0 ? 0 : 1, iy = 1 - ix;
-            cudaError_t e = launch_dependent(
-                adj32_sum_kernel, dim3((n + R32_PTS - 1) / R32_PTS), dim3(R32_PTS * R32_SL), 0, s,
-                src, npad, (const float *)part[ix], T[ix], (const float *)part[iy], T[iy],
-                (const float *)gscale, gpts ? gpts + 2 * (size_t)j0 : nullptr,
-                gA ? gA + j0 : nullptr, gz ? gz + j0 : nullptr);
+            const AdjointParts pp{part[ix], part[iy] + npad, T[ix],       T[iy],
+                                  3 * (size_t)npad, (size_t)npad};
+            cudaError_t e = launch_adjoint_sum(src, pp, gscale,
+                                               gpts ? gpts + 2 * (size_t)j0 : nullptr,
+                                               gA ? gA + j0 : nullptr, gz ? gz + j0 : nullptr, s);
             if (e != cudaSuccess) return cuda_fail(e, "adjoint reduce launch");
             tl.done();
         }

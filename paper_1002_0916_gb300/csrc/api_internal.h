@@ -87,12 +87,6 @@ struct cgh_ctx {
     int direct_schedule = CGH_SCHED_AUTO;         // cgh_set_direct_schedule
     int gemm_tiles = CGH_GEMM_AUTO;               // cgh_set_gemm_tiles
     int gemm_bn = 0;                              // cgh_set_gemm_plan width (0: heuristic)
-    // polynomial (FMA-pipe) sin/cos columns of the direct adjoint's 16-column
-    // strips: 0, 4 (default) or 6; CGH_BWD_POLY at cgh_create
-    int bwd_poly = 4;
-    // direct adjoint: G staged through shared memory by TMA where its layout
-    // allows (1) or read row by row from global memory (0); CGH_BWD_STAGED
-    int bwd_staged = 1;
     // direct forward: the tables kernel builds the point records itself (1)
     // or reads them from a prologue launch (0); CGH_DIRECT_FUSED_TABLES
     int direct_fused_tables = 1;

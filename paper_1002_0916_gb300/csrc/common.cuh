@@ -228,6 +228,18 @@ struct PointSource {
     unsigned *status;
     int y0 = 0;  // origin of the pixel rows (see make_point_rec)
 };
+// Partial sums of the adjoint (backward.cu): Tx tiles of (sum G cos, G sin
+// dx, G sin dx^2) at x + tile * stride + field * npad + point, and Ty tiles of
+// (G sin dy, G sin dy^2) at y.
+struct AdjointParts {
+    const float *x, *y;
+    int Tx, Ty;
+    size_t stride, npad;
+};
+// Adds them in a fixed order, divides by *scale (nullptr: 1) and applies the
+// per-point factors; any of the three outputs may be null.
+cudaError_t launch_adjoint_sum(const PointSource &src, const AdjointParts &pp, const float *scale,
+                               float *gpts, float *gA, float *gz, cudaStream_t s);
 // The same tables with the records built inside the kernel (no prologue).
 cudaError_t launch_direct_tables_fused(const PointSource &src, int Npad, int Nx,
                                        int Ny, const DirectTile &t, float *phx,

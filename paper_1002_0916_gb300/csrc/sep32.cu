@@ -316,10 +316,10 @@ __device__ __forceinline__ void adj32_reduce(const Adj32Prod &pr, const Adj32Arg
     S1 += __shfl_xor_sync(0xffffffffu, S1, 1);
     S2 += __shfl_xor_sync(0xffffffffu, S2, 1);
     if (valid && !odd) {
-        float *p = pr.part + ((size_t)t * ga.npad + j) * 3;
+        float *p = pr.part + (size_t)t * 3 * ga.npad + j;
         p[0] = C;
-        p[1] = S1;
-        p[2] = S2;
+        p[ga.npad] = S1;
+        p[2 * ga.npad] = S2;
     }
 }
 

@@ -52,7 +52,7 @@ struct Adj32Prod {
     int S;        // K slices
     int KB;       // K blocks of 64
     int axis;     // the columns' axis: 0 x, 1 y
-    float *part;  // [(slice, column tile, half)][npad][3]
+    float *part;  // [(slice, column tile, half)][3][npad]
 };
 
 struct Adj32Args {
