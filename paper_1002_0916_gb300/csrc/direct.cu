@@ -27,72 +27,23 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "direct_table.cuh"
 #include "direct_tile.cuh"
 #include "point_rec.cuh"
 
 namespace cgh {
 
 // ------------------------------------------------------------ tables
-// One block per DT_POINTS points (grid x) and 256 pixel columns or rows
-// (grid y: the x range, then the y range): the records are staged in shared
-// memory once; each thread then writes its coordinate for every point, or,
-// in a rotation table, four coordinates of a group for one point at a time.
+// One block per DT_POINTS points (grid x) and DT_SPAN pixel columns or rows
+// (grid y: the x range, then the y range); see direct_table.cuh.
 // FUSE: the block builds its DT_POINTS records itself from the caller's
 // points (step A1, as in prologue.cu) instead of reading them from `rec`;
 // each record is then built once per block row of grid y, a few FP64
 // operations each, which costs less than a separate kernel in the chain.
-constexpr int DT_POINTS = 16;
-
-// One coordinate w (column or row, axis 0 = x, 1 = y) of a tile's angle
-// table for the npts points of srec: dst[q * stride] = its angle for point q.
-__device__ __forceinline__ void angle_column(const PointRec *srec, int npts, int w, int axis,
-                                             float *dst, int stride) {
-    for (int q = 0; q < npts; ++q) {
-        const PointRec &r = srec[q];
-        const uint64_t b = axis ? r.by : r.bx, a = axis ? r.ay : r.ax;
-        dst[(size_t)q * stride] = (float)phase_hi(axis_phase(r.c, b, a, w)) * RAD_PER_U32;
-    }
-}
-
-// Four coordinates g0 + k0 .. g0 + k0 + 3 (k0 = 4 h) of one rotation group
-// of gs coordinates along an axis (0 = x, 1 = y), for one point: slots k0 ..
-// k0 + 3 (cosines of the offsets; slot 0 is the angle at g0) and gs + k0 ..
-// gs + k0 + 3 (sines; slot gs is 0), one 16-byte store each into the
-// point's row of the table (ng groups per tile).  The offsets are exact in
-// fixed point: Phi(g0 + k) - Phi(g0) = k (c (2 g0 + k) - b) for the first,
-// then each next one adds the first difference c (2 u + 1) - b, which grows
-// by 2 c per coordinate (Eq. 2 on the axis).
-__device__ __forceinline__ void rotation_quarter(const PointRec &r, int axis, int g0, int g,
-                                                 int h, int gs, int ng, float *row) {
-    const uint64_t c = r.c, b = axis ? r.by : r.bx, a = axis ? r.ay : r.ax;
-    const int k0 = 4 * h;
-    uint64_t d = (uint64_t)k0 * (c * (uint64_t)(2 * g0 + k0) - b);
-    uint64_t step = c * (uint64_t)(2 * (g0 + k0) + 1) - b;
-    float co[4], si[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        if (k0 + i == 0) {
-            co[i] = (float)phase_hi(axis_phase(c, b, a, g0)) * RAD_PER_U32;
-            si[i] = 0.0f;
-        } else {
-            sincospif(2.0f * ((float)phase_hi(d) * TURN_PER_U32), &si[i], &co[i]);
-        }
-        d += step;
-        step += 2 * c;
-    }
-    *reinterpret_cast<float4 *>(row + rotation_pos(g, k0, ng)) =
-        make_float4(co[0], co[1], co[2], co[3]);
-    *reinterpret_cast<float4 *>(row + rotation_pos(g, gs + k0, ng)) =
-        make_float4(si[0], si[1], si[2], si[3]);
-}
-
 template <bool FUSE>
-__global__ void direct_tables_kernel(const PointRec *__restrict__ rec,
-                                     PointSource src, int Npad, int TX, int TY, int XG,
-                                     int YG, int nxt, int nyt, float *__restrict__ phx,
-                                     float *__restrict__ phy,
-                                     float *__restrict__ amp,
-                                     unsigned *__restrict__ zero, int nzero) {
+__global__ void __launch_bounds__(DT_SPAN)
+direct_tables_kernel(const PointRec *__restrict__ rec, PointSource src, DirectTables dt,
+                     unsigned *__restrict__ zero, int nzero) {
     __shared__ PointRec srec[DT_POINTS];
     pdl_wait();  // the records (or the caller's points) come from the kernel before
     pdl_trigger();
@@ -103,7 +54,7 @@ __global__ void direct_tables_kernel(const PointRec *__restrict__ rec,
              k += gridDim.y * blockDim.x)
             zero[k] = 0u;
     const int j0 = blockIdx.x * DT_POINTS;
-    if (threadIdx.x < DT_POINTS && j0 + (int)threadIdx.x < Npad) {
+    if (threadIdx.x < DT_POINTS && j0 + (int)threadIdx.x < dt.Npad) {
         if constexpr (FUSE)
             srec[threadIdx.x] =
                 make_point_rec(src.points, src.A, src.z, src.N, j0 + threadIdx.x,
@@ -112,30 +63,8 @@ __global__ void direct_tables_kernel(const PointRec *__restrict__ rec,
             srec[threadIdx.x] = rec[j0 + threadIdx.x];
     }
     __syncthreads();
-    // grid y: the x coordinates in blocks of 256, then the y coordinates
-    const int nx = nxt * TX, ny = nyt * TY, nbx = (nx + 255) / 256;
-    const int axis = (int)blockIdx.y >= nbx ? 1 : 0;
-    const int w0 = ((int)blockIdx.y - axis * nbx) * 256;  // the block's first coordinate
-    const int n = axis ? ny : nx, T = axis ? TY : TX, gs = axis ? YG : XG;
-    float *tab = axis ? phy : phx;
-    const int npts = Npad - j0 < DT_POINTS ? Npad - j0 : DT_POINTS;
-    if (gs) {
-        // a rotation table: one thread per four coordinates and point
-        for (int it = threadIdx.x; it < 64 * npts; it += blockDim.x) {
-            const int w = w0 + 4 * (it & 63), q = it >> 6;
-            if (w >= n) continue;
-            const int t = w / T, i = w - t * T, g = i / gs, h = (i - g * gs) >> 2;
-            rotation_quarter(srec[q], axis, w - 4 * h, g, h, gs, T / gs,
-                             tab + ((size_t)t * Npad + j0 + q) * T * 2);
-        }
-    } else {
-        const int u = w0 + threadIdx.x;
-        if (u < n) {
-            const int t = u / T, i = u - t * T;
-            angle_column(srec, npts, u, axis, tab + ((size_t)t * Npad + j0) * T + i, T);
-        }
-    }
-    if (blockIdx.y == 0 && threadIdx.x < npts) amp[j0 + threadIdx.x] = srec[threadIdx.x].A;
+    const int npts = dt.Npad - j0 < DT_POINTS ? dt.Npad - j0 : DT_POINTS;
+    direct_table_block(dt, srec, j0, npts, blockIdx.y);
 }
 
 // ------------------------------------------------------- direct kernel
@@ -272,18 +201,14 @@ static cudaError_t launch_tables(const PointRec *rec, const PointSource *src,
                                  int Npad, int Nx, int Ny, const DirectTile &t,
                                  float *phx, float *phy, float *amp,
                                  unsigned *zero, int nzero, cudaStream_t s) {
-    int nxt = (Nx + t.tx - 1) / t.tx, nyt = (Ny + t.ty - 1) / t.ty;
-    // grid y: the x coordinates, then the y coordinates, in blocks of 256
-    const int nby = (nxt * t.tx + 255) / 256 + (nyt * t.ty + 255) / 256;
-    dim3 grid((Npad + DT_POINTS - 1) / DT_POINTS, nby);
-    const int xg = direct_xg(t), yg = direct_yg(t);
+    const DirectTables dt{Npad, t.tx, t.ty, direct_xg(t), direct_yg(t), (Nx + t.tx - 1) / t.tx,
+                          (Ny + t.ty - 1) / t.ty, phx, phy, amp};
+    dim3 grid((Npad + DT_POINTS - 1) / DT_POINTS, dt.spans());
     if (src)  // (builds the records itself: the call's first kernel)
-        return launch_kernel(false, direct_tables_kernel<true>, grid, dim3(256), 0, s,
-                             (const PointRec *)nullptr, *src, Npad, t.tx, t.ty, xg, yg, nxt,
-                             nyt, phx, phy, amp, zero, nzero);
-    return launch_dependent(direct_tables_kernel<false>, grid, dim3(256), 0, s, rec,
-                            PointSource{}, Npad, t.tx, t.ty, xg, yg, nxt, nyt, phx, phy,
-                            amp, zero, nzero);
+        return launch_kernel(false, direct_tables_kernel<true>, grid, dim3(DT_SPAN), 0, s,
+                             (const PointRec *)nullptr, *src, dt, zero, nzero);
+    return launch_dependent(direct_tables_kernel<false>, grid, dim3(DT_SPAN), 0, s, rec,
+                            PointSource{}, dt, zero, nzero);
 }
 
 cudaError_t launch_direct_tables(const PointRec *rec, int Npad, int Nx, int Ny,

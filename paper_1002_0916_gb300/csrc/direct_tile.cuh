@@ -75,82 +75,14 @@ namespace cgh {
 // group share 2 gs slots: 0: the angle at g0; k = 1 .. gs - 1: cos of the
 // exact phase offset of coordinate g0 + k from g0; gs: 0 (the sine of
 // coordinate g0's zero offset); gs + k: sin of the offset of g0 + k.  The
-// offsets are exact in fixed point; their sines and cosines are accurate
-// (sincospi of the offset in turns).
-__device__ __forceinline__ float rotation_entry(uint64_t c, uint64_t b, uint64_t a, int g0,
-                                                int gs, int slot) {
-    if (slot == 0) return (float)phase_hi(axis_phase(c, b, a, g0)) * RAD_PER_U32;
-    if (slot == gs) return 0.0f;
-    const int k = slot < gs ? slot : slot - gs;
-    const uint64_t d = axis_phase(c, b, a, g0 + k) - axis_phase(c, b, a, g0);
-    float s, co;
-    sincospif(2.0f * ((float)phase_hi(d) * TURN_PER_U32), &s, &co);
-    return slot < gs ? co : s;
-}
-
+// offsets are exact in fixed point; their sines and cosines are taken to FP32
+// rounding (direct_table.cuh).
 // Position of slot `slot` of group g within one point's row of a tile's
 // rotation table with ng groups: the slots go in fours, and the k-th four
 // of every group sit side by side (so a warp's 16-byte loads of the same
 // four of neighbouring groups hit distinct banks).
 __host__ __device__ constexpr int rotation_pos(int g, int slot, int ng) {
     return (slot >> 2) * ng * 4 + g * 4 + (slot & 3);
-}
-
-// The inverse: the (group, slot) of position pos of a row with ng groups.
-__device__ __forceinline__ void rotation_slot(int pos, int ng, int &g, int &slot) {
-    const int j = pos / (ng * 4), r = pos - j * ng * 4;
-    g = r >> 2;
-    slot = j * 4 + (r & 3);
-}
-
-// Entries of the per-axis tables of one problem: x values laid out
-// [x tile][point][x in tile] (xg ? 2 : 1 floats per column, rotation groups
-// of xg columns), then y values [y tile][point][y in tile] (likewise with
-// yg), then the amplitudes [point].
-__device__ __forceinline__ long long direct_table_entries(int Npad, int TX, int TY, int nxt,
-                                                          int nyt, int xg, int yg) {
-    return (long long)nxt * Npad * TX * (xg ? 2 : 1) +
-           (long long)nyt * Npad * TY * (yg ? 2 : 1) + Npad;
-}
-
-__device__ __forceinline__ float axis_table_entry(uint64_t c, uint64_t b, uint64_t a,
-                                                  int T, int gs, int t, int i) {
-    if (gs) {
-        int g, slot;
-        rotation_slot(i, T / gs, g, slot);
-        return rotation_entry(c, b, a, t * T + g * gs, gs, slot);
-    }
-    return (float)phase_hi(axis_phase(c, b, a, t * T + i)) * RAD_PER_U32;
-}
-
-__device__ __forceinline__ void direct_table_entry(
-    const PointRec *__restrict__ rec, int Npad, int TX, int TY, int nxt,
-    int nyt, int xg, int yg, long long e, float *__restrict__ phx,
-    float *__restrict__ phy, float *__restrict__ amp) {
-    const int rx = TX * (xg ? 2 : 1), ry = TY * (yg ? 2 : 1);
-    const long long nx_e = (long long)nxt * Npad * rx;
-    const long long ny_e = (long long)nyt * Npad * ry;
-    if (e < nx_e) {
-        const long long per = (long long)Npad * rx;
-        const int t = (int)(e / per);
-        const long long rem = e - (long long)t * per;
-        const int j = (int)(rem / rx);
-        const int i = (int)(rem - (long long)j * rx);
-        const PointRec &r = rec[j];
-        phx[e] = axis_table_entry(r.c, r.bx, r.ax, TX, xg, t, i);
-    } else if (e < nx_e + ny_e) {
-        const long long f = e - nx_e;
-        const long long per = (long long)Npad * ry;
-        const int t = (int)(f / per);
-        const long long rem = f - (long long)t * per;
-        const int j = (int)(rem / ry);
-        const int i = (int)(rem - (long long)j * ry);
-        const PointRec &r = rec[j];
-        phy[f] = axis_table_entry(r.c, r.by, r.ay, TY, yg, t, i);
-    } else {
-        const int j = (int)(e - nx_e - ny_e);
-        amp[j] = rec[j].A;
-    }
 }
 
 template <int N>
