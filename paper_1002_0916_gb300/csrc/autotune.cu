@@ -31,12 +31,16 @@ std::string size_bucket(int method, int N, int Nx, int Ny) {
 }
 
 double direct_tile_cost(int i, int N, int Nx, int Ny, int sm_count) {
-    (void)N;
     const DirectTile t = direct_tile_get(i);
-    // CTAs are handed to SMs as earlier ones finish, so an SM's share is
-    // about ceil(CTAs / SMs) CTAs of equal work
+    // CTAs are handed to SMs as earlier ones finish: whole tiles per SM, and
+    // the rest cut into chunks of points (direct_split_plan) where a tile has
+    // points enough, else a last wave of whole tiles.  (Counting that wave
+    // whole took 32x32 tiles at 1366x768x777: 105 us against 92 with 64x32.)
     long long ctas = (long long)((Nx + t.tx - 1) / t.tx) * ((Ny + t.ty - 1) / t.ty);
-    const double waves = (double)((ctas + sm_count - 1) / sm_count);
+    const long long rem = ctas % sm_count;
+    const bool split = rem > 0 && N >= 4 * t.pt;
+    const double waves = split ? (double)ctas / sm_count + 0.1
+                               : (double)((ctas + sm_count - 1) / sm_count);
     // Per-update cost model (in MUFU-cosine units), from the measured
     // rates: a quarter of the cosines on the FMA pipe saves about a
     // sixth, packed FP32x2 arithmetic a further 7-9%, shared-memory loads
@@ -57,6 +61,9 @@ double direct_tile_cost(int i, int N, int Nx, int Ny, int sm_count) {
         // measured 0.58 of the pipe's rate
         const double f = 2.0 + 3.0 / t.vx;
         per_pp = f / 8.0 / 0.58;
+        // packed: measured 0.89 of the scalar form's time with 16x4 blocks at
+        // 3840x2160x4096 (2.60 against 2.91 ms), 0.92 with 8x4
+        if (t.pk == 8) per_pp *= t.vx >= 16 ? 0.89 : 0.92;
     }
     return waves * t.tx * t.ty * per_pp;
 }

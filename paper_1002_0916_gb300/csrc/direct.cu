@@ -15,11 +15,17 @@
 //    (cp.async.bulk, mbarrier completion), NST stages deep -- the paper's
 //    shared-memory staging of 256 points per barrier (Section 2.1).
 //  * Work per thread.  Each thread owns a VX x VY block of pixels (the
-//    paper's float8 "eight pixels per item", Section 2.1); per point it reads
-//    VX x-angles, VY y-angles and A_j (broadcast) from shared memory and does
-//    VX*VY of: add, hardware cosine (the paper's native cos), FMA.
-//  * Bound.  One MUFU cosine per point-pixel update; everything else is
-//    2 FP32 ops, so the kernel is bound by the MUFU issue rate.
+//    paper's float8 "eight pixels per item", Section 2.1).  The rotation
+//    tiles (the heuristic's choice) take one hardware sincos per thread and
+//    point and reach the block's other pixels by angle addition with the
+//    tables' cosines and sines; the others a cosine per pixel (the paper's
+//    native cos).
+//  * Bound.  The rotation tiles: the FMA pipe (2 multiply-adds per update) and
+//    the shared-memory reads beside it.  With packed 16x4 blocks the pipe is
+//    73% and the shared-memory data path 76% busy (3840x2160x2048): 41.5
+//    updates per clock and SM of 58.5.  1920x1024x1024 204 -> 167 us,
+//    3840x2160x16384 11.13 -> 10.30 ms against scalar 16x4 blocks with the
+//    groups' sums stored in place.  Cosine-per-pixel tiles: the MUFU.
 //
 // Accuracy: angle rounding about 2^-22 rad per axis, __cosf absolute error
 // about 2^-21 on |x| <= pi, FP32 accumulation: far inside
@@ -124,6 +130,35 @@ direct_fwd_kernel(const float *__restrict__ phx, const float *__restrict__ phy,
         return;
     }
     // publish this chunk's partial tile, then count in
+    if constexpr (L::QUADS) {
+        float4 v[L::NQ];
+        L::reduce_quads(acc, smem, v);
+        float4 *dst = reinterpret_cast<float4 *>(part + (size_t)q * TX * TY);
+#pragma unroll
+        for (int i = 0; i < L::NQ; ++i) dst[threadIdx.x + i * S::THREADS] = v[i];
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0)
+            s_last = atomicAdd(&count[tile - tail], 1u) == (unsigned)(m - 1);
+        __syncthreads();
+        if (!s_last) return;
+        __threadfence();
+        const float4 *src =
+            reinterpret_cast<const float4 *>(part + (size_t)(tile - tail) * m * TX * TY);
+#pragma unroll
+        for (int i = 0; i < L::NQ; ++i) v[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        for (int k = 0; k < m; ++k, src += TX * TY / 4)
+#pragma unroll
+            for (int i = 0; i < L::NQ; ++i) {
+                const float4 p = __ldcg(src + threadIdx.x + i * S::THREADS);
+                v[i].x += p.x;
+                v[i].y += p.y;
+                v[i].z += p.z;
+                v[i].w += p.w;
+            }
+        L::write_quads(v, xt, yt, Nx, Ny, out, vec_store);
+        return;
+    }
     L::reduce_groups(acc, smem);
     const int lt = threadIdx.x % S::GT, grp = threadIdx.x / S::GT;
     const int tx = lt % S::NTX, ty = lt / S::NTX;
