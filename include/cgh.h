@@ -362,9 +362,8 @@ cgh_status cgh_set_direct_schedule(cgh_handle h, int schedule);
  *                    cgh_batch takes CGH_GEMM_PAIRS then);
  *   CGH_GEMM_AUTO:   the handle's tuned plan for the size (cgh_tune), else
  *                    CTA pairs for single holograms of more
- *                    than 128 rows, one-CTA tiles otherwise and for
- *                    cgh_batch (whose persistent work list balances better
- *                    with the smaller items).
+ *                    than 128 rows and for cgh_batch, one-CTA tiles
+ *                    otherwise.
  * Every mode computes the same products with FP32 accumulation; results
  * agree to rounding.  The adjoint has one tiling of its own (CTA pairs) and
  * does not depend on this setting. */

@@ -178,6 +178,9 @@ def _check(h, status: int, what: str):
 
 
 def _method(m) -> int:
+    v = METHODS.get(m) if isinstance(m, str) else None
+    if v is not None:
+        return v
     if isinstance(m, str):
         if m not in METHODS:
             raise ValueError(f"unknown method {m!r}; one of {sorted(METHODS)}")
@@ -185,20 +188,36 @@ def _method(m) -> int:
     return int(m)
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 def _stream_ptr(stream) -> Optional[int]:
     torch = _torch()
     if stream is None:
+        # the current stream of the current device; without the Stream object
+        # torch.cuda.current_stream() makes for it (3 us of a call's 23) where
+        # PyTorch has its CUDA state already
+        if torch.cuda.is_initialized():
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
         stream = torch.cuda.current_stream()
     return int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def _dev_f32(t, name: str, numel: Optional[int] = None):
     torch = _torch()
+    if isinstance(t, torch.Tensor) and t.is_cuda and t.dtype is torch.float32 and \
+            t.is_contiguous():
+        n = t.numel()
+        if numel is None or n == numel:
+            return t.data_ptr() if n else None
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
     if t.dtype != torch.float32 or not t.is_contiguous():
@@ -597,8 +616,7 @@ def _make_function():
             pts, A_, z_ = ctx.saved_tensors
             lam, p, Nx, Ny, bm = ctx.args
             need = ctx.needs_input_grad[:3]
-            gp, gA, gz = cgh_backward(pts, A_, z_, lam, p, Nx, Ny,
-                                      grad_out.contiguous(), method=bm,
+            gp, gA, gz = cgh_backward(pts, A_, z_, lam, p, Nx, Ny, grad_out, method=bm,
                                       need=(need[0], need[1], need[2]))
             return gp, gA, gz, None, None, None, None, None, None
 
@@ -611,6 +629,7 @@ class _LazyFunction:
     def __getattr__(self, name):
         if _LazyFunction._fn is None:
             _LazyFunction._fn = _make_function()
+            self.apply = _LazyFunction._fn.apply  # (found without this detour from now on)
         return getattr(_LazyFunction._fn, name)
 
 

@@ -106,8 +106,10 @@ cgh_status cgh_ctx::check_problem(const float *points, const float *A,
 // ------------------------------------------------------------ tiles
 int cgh_ctx::pick_direct_tile(int N, int Nx, int Ny) {
     if (forced_tile >= 0) return forced_tile;
-    auto it = tuned.find(size_bucket(CGH_DIRECT_FP32, N, Nx, Ny));
-    if (it != tuned.end()) return it->second;
+    if (!tuned.empty()) {
+        auto it = tuned.find(size_bucket(CGH_DIRECT_FP32, N, Nx, Ny));
+        if (it != tuned.end()) return it->second;
+    }
     return default_direct_tile(N, Nx, Ny, sm_count);
 }
 

@@ -596,11 +596,11 @@ bool cgh_ctx::batch_sep_pairs(const cgh_problem *probs, int count, bool *tuned_o
         if (tuned_out) *tuned_out = true;
         return it->second / 1000 == CGH_GEMM_PAIRS;
     }
-    // one-CTA items (128 x 128) unless CTA pairs were asked for: pair items
-    // (256 x 128) halve the number of work items, and on the 64-hologram
-    // batch the coarser balance cost more (4.55 ms) than the halved operand
-    // bytes per SM saved (one-CTA items: 4.24 ms)
-    return false;
+    // CTA-pair items (256 x 128): batches of 64, 16 and 8 holograms of 512 to
+    // 2048 pixels a side took 4.05, 1.00 and 0.50 ms with them, 4.16, 1.20 and
+    // 0.58 with one-CTA items (128 x 128), which read twice the operand bytes
+    // per SM
+    return true;
 }
 
 cgh_status cgh_ctx::batch_separable(const cgh_problem *probs, int count,

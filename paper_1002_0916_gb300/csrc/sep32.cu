@@ -27,14 +27,16 @@
 // alternate between the MMAs and the epilogue.  Eight epilogue warps hold
 // the CTA's 128 x BNP sums, each thread one row and half of the columns (at
 // most 128 registers).  What bounds it is the MMA rate (12 steps per K
-// block): at 256 columns a K block takes 0.81 us, the same with the promotion
-// as without it; at 112 to 160 columns it takes 0.64 to 0.69 us against 0.60,
-// or 0.52 with no loads.  The epilogue's barrier waits are at CTA scope and
-// its arrivals relaxed (tensor memory is ordered by the tcgen05 fences, and no
-// generic memory is handed over): with cluster-scope acquire and release a
-// block took 1.1 to 1.4 us.
+// block): a K block takes 0.81 us at 256 columns and 0.37 at 112 (one pair
+// alone), 139 and 63 SM cycles a step.  Two things cost more than the MMAs
+// before: issued from one lane's branch instead of an elected lane of a
+// converged warp, a step took 105 to 120 cycles at any width below 192 (see
+// elect_one); and with cluster-scope acquire and release on the epilogue's
+// barriers a block took 1.1 to 1.4 us (the waits are at CTA scope and the
+// arrivals relaxed: tensor memory is ordered by the tcgen05 fences, and no
+// generic memory is handed over).
 // Measured, whole call, against an FP32 product on the FMA pipe (0.70 of its
-// bound): 1920x1024x3584 543 -> 84 us, 3840x2160x16384 9.85 -> 1.12 ms;
+// bound): 1920x1024x3584 543 -> 73 us, 3840x2160x16384 9.85 -> 1.04 ms;
 // relative RMS error against FP64 6.8e-7 -> 1.9e-7 and 1.6e-6 -> 2.3e-7.
 //
 // Long products on few tiles are cut along K into S slices: each slice's
@@ -151,7 +153,13 @@ sep32_tables_kernel(PointSource src, int Npad, int Nx, int Ny, int Kp,
 
 // ------------------------------------------------------------------ GEMM
 constexpr int S32_EPI_WARPS = 8;
-constexpr int S32_THREADS = 64 + 32 * S32_EPI_WARPS;
+// One warpgroup with the producer and the MMA issuer, two of epilogue warps.
+// 384 threads get 168 registers each at launch; the first group gives up all
+// but 56, the others take 224 (56 + 2 x 224 = 3 x 168), which holds a
+// thread's 128 sums and two tensor-memory loads without spills (at 168: 5 to
+// 10% slower).
+constexpr int S32_THREADS = 128 + 32 * S32_EPI_WARPS;
+constexpr int S32_ROLE_REGS = 56, S32_EPI_REGS = 224;
 
 struct Sep32Args {
     int units, tiles_m, tiles_n, KB;  // forward: tiles, K blocks; units of either
@@ -224,7 +232,7 @@ __device__ __forceinline__ void sep32_store(const Sep32Args &g, bool ok, int mt,
         }
         __threadfence();
         asm volatile("bar.sync 1, %0;" ::"n"(32 * S32_EPI_WARPS) : "memory");
-        if (threadIdx.x == 64)
+        if (threadIdx.x == 128)
             *s_last = atomicAdd(&g.count[tile * 2 + rank], 1u) == (unsigned)(g.S - 1);
         asm volatile("bar.sync 1, %0;" ::"n"(32 * S32_EPI_WARPS) : "memory");
         store = ok && *(volatile int *)s_last;
@@ -383,7 +391,7 @@ sep32_pair_kernel(const __grid_constant__ Sep32Maps maps0,
 
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const uint32_t rank = umma2::cluster_rank();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = umma::warp_index(), lane = threadIdx.x & 31;
     const int cl = blockIdx.x >> 1, ncl = gridDim.x >> 1;
 
     if (threadIdx.x == 0) {
@@ -412,51 +420,59 @@ sep32_pair_kernel(const __grid_constant__ Sep32Maps maps0,
     const uint32_t tmem = tmem_base;
     pdl_wait();  // the tables and factors come from the kernel before
 
-    if (warp == 0 && lane == 0) {
-        // ------------------------------------------ producer (both CTAs)
-        unsigned n = 0;  // K blocks issued
-        for (int r = 0; r * ncl < g.units && !abort_flag; ++r) {
-            const int u = sep32_unit_index(r, cl, ncl);
-            if (u >= g.units) break;
-            const Sep32Unit w = sep32_unit<ADJ>(u, g, ga);
-            const Sep32Maps *maps = w.which ? &maps1 : &maps0;
-            const int m0 = w.mt * 2 * S::BM + (int)rank * S::BM;  // this CTA's rows
-            const int nb = w.nt * BNP + (int)rank * S::BNH;       // its B rows
-            for (int i = 0; i < w.nkb; ++i, ++n) {
-                const int s = (int)(n % STAGES);
-                if (n >= STAGES &&
-                    !mbar_wait_bounded(&empty[s], ((n / STAGES) - 1) & 1)) {
-                    abort_flag = 1;
-                    set_status(g.status, DEV_TIMEOUT);
+    if (warp < 4) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(S32_ROLE_REGS));
+        if (warp == 0) {
+            // -------------------------------------- producer (both CTAs)
+            unsigned n = 0;  // K blocks issued
+            bool ok = true;
+            for (int r = 0; r * ncl < g.units && ok; ++r) {
+                const int u = sep32_unit_index(r, cl, ncl);
+                if (u >= g.units) break;
+                const Sep32Unit w = sep32_unit<ADJ>(u, g, ga);
+                const Sep32Maps *maps = w.which ? &maps1 : &maps0;
+                const int m0 = w.mt * 2 * S::BM + (int)rank * S::BM;  // this CTA's rows
+                const int nb = w.nt * BNP + (int)rank * S::BNH;       // its B rows
+                for (int i = 0; i < w.nkb; ++i, ++n) {
+                    const int s = (int)(n % STAGES);
+                    if (n >= STAGES && !mbar_wait_bounded(&empty[s], ((n / STAGES) - 1) & 1)) {
+                        abort_flag = 1;
+                        set_status(g.status, DEV_TIMEOUT);
+                    }
+                    ok = __all_sync(0xffffffffu, !abort_flag);
+                    if (!ok) break;
+                    uint8_t *st = smem + (size_t)s * S::STAGE_BYTES;
+                    const uint32_t bar = umma2::map_to_rank(&full[s], 0);
+                    const int k = (w.kb0 + i) * S::BK;
+                    if (umma::elect_one()) {
+                        // the even CTA's barrier counts the bytes of both CTAs' loads
+                        if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * S::STAGE_BYTES);
+                        umma2::tma_load_2d_pair(st, &maps->A, k, m0, bar);
+                        umma2::tma_load_2d_pair(st + S::A_BYTES, &maps->B, k, nb, bar);
+                        umma2::tma_load_2d_pair(st + S::A_BYTES + S::B_BYTES, &maps->A2, k, m0,
+                                                bar);
+                        umma2::tma_load_2d_pair(st + 2 * S::A_BYTES + S::B_BYTES, &maps->B2, k,
+                                                nb, bar);
+                    }
                 }
-                if (abort_flag) break;
-                uint8_t *st = smem + (size_t)s * S::STAGE_BYTES;
-                // the even CTA's barrier counts the bytes of both CTAs' loads
-                if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * S::STAGE_BYTES);
-                const uint32_t bar = umma2::map_to_rank(&full[s], 0);
-                const int k = (w.kb0 + i) * S::BK;
-                umma2::tma_load_2d_pair(st, &maps->A, k, m0, bar);
-                umma2::tma_load_2d_pair(st + S::A_BYTES, &maps->B, k, nb, bar);
-                umma2::tma_load_2d_pair(st + S::A_BYTES + S::B_BYTES, &maps->A2, k, m0, bar);
-                umma2::tma_load_2d_pair(st + 2 * S::A_BYTES + S::B_BYTES, &maps->B2, k, nb, bar);
             }
-        }
-        const unsigned lo = n > STAGES ? n - STAGES : 0;
-        if (abort_flag && rank == 0) {
-            // let the stages' copies land before shared memory goes (the odd
-            // CTA leaves only after the closing cluster barrier)
-            for (unsigned i = lo; i < n; ++i) mbar_wait_bounded(&full[i % STAGES], (i / STAGES) & 1);
-        } else if (!abort_flag) {
-            // wait (bounded) for the commits of the last stages, so that no
-            // arrive is in flight when the CTA's shared memory passes on
-            for (unsigned i = lo; i < n; ++i)
-                mbar_wait_bounded(&empty[i % STAGES], (i / STAGES) & 1);
-        }
-    } else if (warp == 1 && lane == 0) {
-        if (rank == 0) {
+            const unsigned lo = n > STAGES ? n - STAGES : 0;
+            if (!ok && rank == 0) {
+                // let the stages' copies land before shared memory goes (the odd
+                // CTA leaves only after the closing cluster barrier)
+                for (unsigned i = lo; i < n; ++i)
+                    mbar_wait_bounded(&full[i % STAGES], (i / STAGES) & 1);
+            } else if (ok) {
+                // wait (bounded) for the commits of the last stages, so that no
+                // arrive is in flight when the CTA's shared memory passes on
+                for (unsigned i = lo; i < n; ++i)
+                    mbar_wait_bounded(&empty[i % STAGES], (i / STAGES) & 1);
+            }
+        } else if (warp == 1 && rank == 0) {
             // ---------------------------------------- MMA issuer (even CTA)
             unsigned n = 0;
-            for (int r = 0; r * ncl < g.units && !abort_flag; ++r) {
+            bool ok = true;
+            for (int r = 0; r * ncl < g.units && ok; ++r) {
                 const int u = sep32_unit_index(r, cl, ncl);
                 if (u >= g.units) break;
                 const int nkb = sep32_unit<ADJ>(u, g, ga).nkb;
@@ -467,7 +483,8 @@ sep32_pair_kernel(const __grid_constant__ Sep32Maps maps0,
                         abort_flag = 1;
                         set_status(g.status, DEV_TIMEOUT);
                     }
-                    if (abort_flag) break;
+                    ok = __all_sync(0xffffffffu, !abort_flag);
+                    if (!ok) break;
                     umma::fence_after_sync();
                     const uint32_t a = smem_u32(smem + (size_t)s * S::STAGE_BYTES);
                     const uint32_t bb = a + S::A_BYTES;
@@ -477,26 +494,30 @@ sep32_pair_kernel(const __grid_constant__ Sep32Maps maps0,
                     const uint64_t ad2 = umma::sw128_kmajor_desc(a2);
                     const uint64_t bd2 = umma::sw128_kmajor_desc(b2);
                     const uint32_t d = tmem + (uint32_t)b * C::STRIDE;
-                    // the small cross products first: the sum's low bits are
-                    // dropped only by the four hi*hi steps
+                    if (umma::elect_one()) {
+                        // the small cross products first: the sum's low bits are
+                        // dropped only by the four hi*hi steps
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        umma2::mma2_f16(d, ad + 2 * kk, bd2 + 2 * kk, idesc, kk != 0);
+                        for (int kk = 0; kk < 4; ++kk)
+                            umma2::mma2_f16(d, ad + 2 * kk, bd2 + 2 * kk, idesc, kk != 0);
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        umma2::mma2_f16(d, ad2 + 2 * kk, bd + 2 * kk, idesc, 1);
+                        for (int kk = 0; kk < 4; ++kk)
+                            umma2::mma2_f16(d, ad2 + 2 * kk, bd + 2 * kk, idesc, 1);
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        umma2::mma2_f16(d, ad + 2 * kk, bd + 2 * kk, idesc, 1);
-                    umma2::commit2(&empty[s], 0x3);
-                    umma2::commit2(&acc_full[b], 0x3);
+                        for (int kk = 0; kk < 4; ++kk)
+                            umma2::mma2_f16(d, ad + 2 * kk, bd + 2 * kk, idesc, 1);
+                        umma2::commit2(&empty[s], 0x3);
+                        umma2::commit2(&acc_full[b], 0x3);
+                    }
+                    __syncwarp();
                 }
             }
         }
-    } else if (warp >= 2) {
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(S32_EPI_REGS));
         // --------------------------------------- epilogue (both CTAs)
         const int q = warp & 3;               // the 32-lane quarter of TMEM
-        const int half = (warp - 2) >> 2;     // the columns' half
+        const int half = (warp - 4) >> 2;     // the columns' half
         const int nu = half ? C::U1 : C::U0;  // its units of 16 columns
         const int c0 = half * C::U0 * 16;
         const int lrow = q * 32 + lane;
@@ -519,9 +540,11 @@ sep32_pair_kernel(const __grid_constant__ Sep32Maps maps0,
                 ok = __all_sync(0xffffffffu,
                                 mbar_wait_bounded(&acc_full[b], (n / C::NBUF) & 1));
                 umma::fence_after_sync();
-                if (!ok) set_status(g.status, DEV_TIMEOUT);
-                ok = __all_sync(0xffffffffu, ok && !abort_flag);
-                if (!ok) break;
+                if (!ok || abort_flag) {
+                    if (!ok) set_status(g.status, DEV_TIMEOUT);
+                    ok = false;
+                    break;
+                }
                 sep32_promote<C::U0>(t0 + (uint32_t)b * C::STRIDE, nu, f, acc);
                 umma::fence_before_sync();
                 __syncwarp();
@@ -553,28 +576,26 @@ struct Sep32Plan {
     int bn, S;
 };
 
-static const int kSep32BN[] = {112, 128, 160, 192, 256};
+static const int kSep32BN[] = {112, 128, 144, 160, 192, 224, 256};
 constexpr int S32_MAX_SPLIT = 64;
 
 // The tile width and the number of K slices with the least modelled time:
 // waves of the SM pairs times (K blocks of a slice + fill and epilogue), plus
 // the partial tiles of a split.  The constants are fits in microseconds to a
 // sweep of every width and 1 to 64 slices over 13 frames (128 x 128 to
-// 3840 x 2160, 64 to 16,384 points): a K block takes 0.69 us at 112 columns
-// and 0.87 at 256 -- below 160 columns the MMA steps stop getting shorter
-// (90 SM cycles each, for operand reads) -- so the narrow tiles only serve to
-// fill the SMs, and a small frame is better cut along K: 128x128x16384 36 us
-// in 32 slices against 327 in one, 640x480x2000 22.7 us in 6 against 49.
+// 3840 x 2160, 64 to 16,384 points): a K block takes 0.44 us at 112 columns
+// and 0.87 at 256, and a small frame is better cut along K: 128x128x16384 31 us
+// in 24 slices against 187 in one, 640x480x2000 21 us in 5 against 39.
 static Sep32Plan sep32_plan(int M, int N, int KB, int sms) {
     Sep32Plan best{256, 1};
     double best_cost = 1e300;
     const int pairs = sms / 2 > 0 ? sms / 2 : 1;
     for (int bn : kSep32BN) {
         const long long tiles = (long long)((M + 255) / 256) * ((N + bn - 1) / bn);
-        for (int S = 1; S <= S32_MAX_SPLIT && S <= KB; ++S) {
+        for (int S = 1; S <= S32_MAX_SPLIT && S <= KB && (S == 1 || tiles * S <= 2 * pairs); ++S) {
             const long long waves = (tiles * S + pairs - 1) / pairs;
             const double cost =
-                (double)waves * (((KB + S - 1) / S) * (0.55 + 0.00125 * bn) + 2.0 + 0.012 * bn) +
+                (double)waves * (((KB + S - 1) / S) * (0.10 + 0.0030 * bn) + 2.0 + 0.012 * bn) +
                 (S > 1 ? 4.0 + 0.0065 * bn * S : 0.0);
             if (cost < best_cost) {
                 best_cost = cost;
@@ -625,8 +646,10 @@ static cudaError_t launch_sep32(int bn, const Sep32Operands &op, const Sep32Args
     switch (bn) {
     case 112: return launch_sep32_t<112, 4>(op, g, s);
     case 128: return launch_sep32_t<128, 4>(op, g, s);
+    case 144: return launch_sep32_t<144, 4>(op, g, s);
     case 160: return launch_sep32_t<160, 4>(op, g, s);
     case 192: return launch_sep32_t<192, 4>(op, g, s);
+    case 224: return launch_sep32_t<224, 3>(op, g, s);
     case 256: return launch_sep32_t<256, 3>(op, g, s);
     }
     return cudaErrorInvalidValue;
@@ -638,10 +661,10 @@ static const int kAdj32BN[] = {192, 224, 256};
 // The width and slices with the least modelled time (the constants of
 // sep32_plan): units of both products on the SM pairs, longest first, so the
 // total spread over the pairs plus part of a unit, or the longest unit alone.
-// A unit's epilogue adds 1.8 us at 192 columns to 2.9 at 256 that the next
-// unit's MMAs do not cover (1920x1080x4096: 142 us at 224 columns, 149 at 256,
-// 159 at 192); a K slice costs nothing else, since the epilogue is linear in D
-// and every slice writes its own partial sums.
+// A unit's epilogue adds about 2.9 us that the next unit's MMAs do not cover
+// (1920x1080x4096: 128 us at 224 columns, 134 at 192, 141 at 256); a K slice
+// costs nothing else, since the epilogue is linear in D and every slice writes
+// its own partial sums.
 Adj32Plan adj32_plan(int n, int Nx, int Ny, int sms) {
     Adj32Plan best{256, {1, 1}};
     double best_cost = 1e300;
@@ -650,11 +673,14 @@ Adj32Plan adj32_plan(int n, int Nx, int Ny, int sms) {
     const int N[2] = {Nx <= Ny ? Nx : Ny, Nx <= Ny ? Ny : Nx};  // columns; K = the other
     const int KB[2] = {(N[1] + 63) / 64, (N[0] + 63) / 64};
     for (int bn : kAdj32BN) {
-        const double tkb = 1.1 * (0.55 + 0.00125 * bn), epi = 0.011 * bn;
-        for (int S0 = 1; S0 <= 16 && S0 <= KB[0]; ++S0)
-            for (int S1 = 1; S1 <= 16 && S1 <= KB[1]; ++S1) {
-                const double n0 = (double)(mt * ((N[0] + bn - 1) / bn) * S0);
-                const double n1 = (double)(mt * ((N[1] + bn - 1) / bn) * S1);
+        const double tkb = 1.1 * (0.10 + 0.0030 * bn), epi = 2.9;
+        // (slices only where the tiles alone leave pairs idle)
+        const long long t0 = mt * ((N[0] + bn - 1) / bn), t1 = mt * ((N[1] + bn - 1) / bn);
+        const int most = t0 + t1 >= 4 * pairs ? 1 : 16;
+        for (int S0 = 1; S0 <= most && S0 <= KB[0]; ++S0)
+            for (int S1 = 1; S1 <= most && S1 <= KB[1]; ++S1) {
+                if (S0 + S1 > 2 && t0 * S0 + t1 * S1 > 2 * pairs) break;
+                const double n0 = (double)(t0 * S0), n1 = (double)(t1 * S1);
                 const double u0 = ((KB[0] + S0 - 1) / S0) * tkb + epi;
                 const double u1 = ((KB[1] + S1 - 1) / S1) * tkb + epi;
                 const double longest = u0 > u1 ? u0 : u1;

@@ -97,7 +97,7 @@ cgh_ctx::GemmPlanChoice cgh_ctx::sep_plan(int method, int N, int Nx, int Ny) {
                                      forced_plan % 1000);
         return GemmPlanChoice{p.tiling, p.bn, false};
     }
-    if (gemm_tiles == CGH_GEMM_AUTO) {
+    if (gemm_tiles == CGH_GEMM_AUTO && !tuned_gemm.empty()) {
         auto it = tuned_gemm.find(size_bucket(method, N, Nx, Ny));
         if (it != tuned_gemm.end()) {
             const GemmPlan p = gemm_plan(Ny, Nx, it->second / 1000, sm_count, kind,

@@ -71,7 +71,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tA,
     __shared__ volatile int abort_flag;
 
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = umma::warp_index(), lane = threadIdx.x & 31;
     const int n0 = blockIdx.x * BN, m0 = blockIdx.y * S::BM;
     const int KB = (g.K + S::BK - 1) / S::BK;
 
@@ -100,8 +100,9 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tA,
     umma::fence_after_sync();
     const uint32_t tmem = tmem_base;
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
         // ---------------------------------------------------- producer
+        bool ok = true;
         int issued = 0;
         for (int kb = 0; kb < KB; ++kb) {
             const int s = kb % STAGES;
@@ -110,20 +111,23 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tA,
                 abort_flag = 1;
                 set_status(g.status, DEV_TIMEOUT);
             }
-            if (abort_flag) break;
+            ok = __all_sync(0xffffffffu, !abort_flag);
+            if (!ok) break;
             uint8_t *st = smem + (size_t)s * S::STAGE_BYTES;
-            mbar_arrive_expect_tx(&full[s], S::STAGE_BYTES);
-            umma::tma_load_2d(st, &tA, kb * S::BK, m0, &full[s]);
-            umma::tma_load_2d(st + S::A_BYTES, &tB, kb * S::BK, n0, &full[s]);
-            if (SPLIT) {
-                umma::tma_load_2d(st + S::A_BYTES + S::B_BYTES, &tA2, kb * S::BK,
-                                  m0, &full[s]);
-                umma::tma_load_2d(st + 2 * S::A_BYTES + S::B_BYTES, &tB2,
-                                  kb * S::BK, n0, &full[s]);
+            if (umma::elect_one()) {
+                mbar_arrive_expect_tx(&full[s], S::STAGE_BYTES);
+                umma::tma_load_2d(st, &tA, kb * S::BK, m0, &full[s]);
+                umma::tma_load_2d(st + S::A_BYTES, &tB, kb * S::BK, n0, &full[s]);
+                if (SPLIT) {
+                    umma::tma_load_2d(st + S::A_BYTES + S::B_BYTES, &tA2, kb * S::BK,
+                                      m0, &full[s]);
+                    umma::tma_load_2d(st + 2 * S::A_BYTES + S::B_BYTES, &tB2,
+                                      kb * S::BK, n0, &full[s]);
+                }
             }
             ++issued;
         }
-        if (abort_flag) {
+        if (!ok) {
             // let this CTA's own copies land before its shared memory goes
             for (int kb = issued - STAGES < 0 ? 0 : issued - STAGES; kb < issued; ++kb)
                 mbar_wait_bounded(&full[kb % STAGES], (uint32_t)((kb / STAGES) & 1));
@@ -136,7 +140,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tA,
             for (int kb = KB - STAGES < 0 ? 0 : KB - STAGES; kb < KB; ++kb)
                 mbar_wait_bounded(&empty[kb % STAGES], (uint32_t)((kb / STAGES) & 1));
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         // --------------------------------------------------- MMA issuer
         for (int kb = 0; kb < KB; ++kb) {
             const int s = kb % STAGES;
@@ -144,31 +148,34 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tA,
                 abort_flag = 1;
                 set_status(g.status, DEV_TIMEOUT);
             }
-            if (abort_flag) break;
+            if (!__all_sync(0xffffffffu, !abort_flag)) break;
             umma::fence_after_sync();
             const uint32_t a = smem_u32(smem + (size_t)s * S::STAGE_BYTES);
             const uint32_t b = a + S::A_BYTES;
+            const uint32_t a2 = b + S::B_BYTES, b2 = a2 + S::A_BYTES;
             const uint64_t ad = umma::sw128_kmajor_desc(a);
             const uint64_t bd = umma::sw128_kmajor_desc(b);
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-                umma::mma_f16(tmem, ad + 2 * kk, bd + 2 * kk, idesc,
-                              (kb | kk) != 0);
-            if (SPLIT) {
-                const uint32_t a2 = b + S::B_BYTES, b2 = a2 + S::A_BYTES;
-                const uint64_t ad2 = umma::sw128_kmajor_desc(a2);
-                const uint64_t bd2 = umma::sw128_kmajor_desc(b2);
+            const uint64_t ad2 = umma::sw128_kmajor_desc(a2);
+            const uint64_t bd2 = umma::sw128_kmajor_desc(b2);
+            if (umma::elect_one()) {
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)
-                    umma::mma_f16(tmem + S::ACC1, ad + 2 * kk, bd2 + 2 * kk, idesc,
-                                  (kb | kk) != 0);
+                    umma::mma_f16(tmem, ad + 2 * kk, bd + 2 * kk, idesc, (kb | kk) != 0);
+                if (SPLIT) {
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    umma::mma_f16(tmem + S::ACC1, ad2 + 2 * kk, bd + 2 * kk, idesc, 1);
+                    for (int kk = 0; kk < 4; ++kk)
+                        umma::mma_f16(tmem + S::ACC1, ad + 2 * kk, bd2 + 2 * kk, idesc,
+                                      (kb | kk) != 0);
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk)
+                        umma::mma_f16(tmem + S::ACC1, ad2 + 2 * kk, bd + 2 * kk, idesc, 1);
+                }
+                umma::mma_commit(&empty[s]);
             }
-            umma::mma_commit(&empty[s]);
+            __syncwarp();
         }
-        umma::mma_commit(&accum_bar);  // fires once every issued MMA is done
+        // fires once every issued MMA is done
+        if (umma::elect_one()) umma::mma_commit(&accum_bar);
     } else if (warp >= 2) {
         // ----------------------------------------------------- epilogue
         const int q = warp & 3;  // the 32-lane quarter of TMEM this warp reads
@@ -398,7 +405,7 @@ umma_grouped_kernel(const GroupProb *__restrict__ probs,
     __shared__ volatile int abort_flag;
 
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = umma::warp_index(), lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
@@ -421,10 +428,11 @@ umma_grouped_kernel(const GroupProb *__restrict__ probs,
     umma::fence_after_sync();
     const uint32_t tmem = tmem_base;
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
         // ---------------------------------------------------- producer
+        bool ok = true;
         unsigned g = 0, issued_from = 0;
-        for (int it = blockIdx.x; it < nitems && !abort_flag; it += gridDim.x) {
+        for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x) {
             const uint2 w = items[it];
             const GroupProb *gp = probs + w.x;
             const int m0 = (int)(w.y & 0xffffu) * S::BM, n0 = (int)(w.y >> 16) * BN;
@@ -436,19 +444,22 @@ umma_grouped_kernel(const GroupProb *__restrict__ probs,
                     abort_flag = 1;
                     set_status(status, DEV_TIMEOUT);
                 }
-                if (abort_flag) break;
+                ok = __all_sync(0xffffffffu, !abort_flag);
+                if (!ok) break;
                 uint8_t *st = smem + (size_t)s * S::STAGE_BYTES;
-                mbar_arrive_expect_tx(&full[s], S::STAGE_BYTES);
-                umma::tma_load_2d(st, &gp->tA, kb * S::BK, m0, &full[s]);
-                umma::tma_load_2d(st + S::A_BYTES, &gp->tB, kb * S::BK, n0, &full[s]);
-                umma::tma_load_2d(st + S::A_BYTES + S::B_BYTES, &gp->tA2, kb * S::BK,
-                                  m0, &full[s]);
-                umma::tma_load_2d(st + 2 * S::A_BYTES + S::B_BYTES, &gp->tB2,
-                                  kb * S::BK, n0, &full[s]);
+                if (umma::elect_one()) {
+                    mbar_arrive_expect_tx(&full[s], S::STAGE_BYTES);
+                    umma::tma_load_2d(st, &gp->tA, kb * S::BK, m0, &full[s]);
+                    umma::tma_load_2d(st + S::A_BYTES, &gp->tB, kb * S::BK, n0, &full[s]);
+                    umma::tma_load_2d(st + S::A_BYTES + S::B_BYTES, &gp->tA2, kb * S::BK,
+                                      m0, &full[s]);
+                    umma::tma_load_2d(st + 2 * S::A_BYTES + S::B_BYTES, &gp->tB2,
+                                      kb * S::BK, n0, &full[s]);
+                }
                 issued_from = g + 1;
             }
         }
-        if (abort_flag) {
+        if (!ok) {
             unsigned lo = issued_from > STAGES ? issued_from - STAGES : 0;
             for (unsigned u = lo; u < issued_from; ++u)
                 mbar_wait_bounded(&full[u % STAGES], (uint32_t)((u / STAGES) & 1));
@@ -462,18 +473,20 @@ umma_grouped_kernel(const GroupProb *__restrict__ probs,
             for (unsigned u = lo; u < g; ++u)
                 mbar_wait_bounded(&empty[u % STAGES], (uint32_t)((u / STAGES) & 1));
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         // --------------------------------------------------- MMA issuer
         const uint32_t idesc = umma::idesc_f16(S::BM, BN, false);
         unsigned g = 0;
         int n = 0;
-        for (int it = blockIdx.x; it < nitems && !abort_flag; it += gridDim.x, ++n) {
+        bool ok = true;
+        for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x, ++n) {
             const int b = n & 1;
             if (!mbar_wait_bounded(&acc_empty[b], (uint32_t)(((n >> 1) & 1) ^ 1))) {
                 abort_flag = 1;
                 set_status(status, DEV_TIMEOUT);
-                break;
             }
+            ok = __all_sync(0xffffffffu, !abort_flag);
+            if (!ok) break;
             umma::fence_after_sync();
             const uint32_t d0 = tmem + (uint32_t)b * ACC_COLS, d1 = d0 + BN;
             const GroupProb *gp = probs + items[it].x;
@@ -483,8 +496,9 @@ umma_grouped_kernel(const GroupProb *__restrict__ probs,
                 if (!mbar_wait_bounded(&full[s], (uint32_t)((g / STAGES) & 1))) {
                     abort_flag = 1;
                     set_status(status, DEV_TIMEOUT);
-                    break;
                 }
+                ok = __all_sync(0xffffffffu, !abort_flag);
+                if (!ok) break;
                 umma::fence_after_sync();
                 const uint32_t a = smem_u32(smem + (size_t)s * S::STAGE_BYTES);
                 const uint32_t bb = a + S::A_BYTES;
@@ -493,18 +507,22 @@ umma_grouped_kernel(const GroupProb *__restrict__ probs,
                 const uint64_t bd = umma::sw128_kmajor_desc(bb);
                 const uint64_t ad2 = umma::sw128_kmajor_desc(a2);
                 const uint64_t bd2 = umma::sw128_kmajor_desc(b2);
+                if (umma::elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    umma::mma_f16(d0, ad + 2 * kk, bd + 2 * kk, idesc, (kb | kk) != 0);
+                    for (int kk = 0; kk < 4; ++kk)
+                        umma::mma_f16(d0, ad + 2 * kk, bd + 2 * kk, idesc, (kb | kk) != 0);
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    umma::mma_f16(d1, ad + 2 * kk, bd2 + 2 * kk, idesc, (kb | kk) != 0);
+                    for (int kk = 0; kk < 4; ++kk)
+                        umma::mma_f16(d1, ad + 2 * kk, bd2 + 2 * kk, idesc, (kb | kk) != 0);
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    umma::mma_f16(d1, ad2 + 2 * kk, bd + 2 * kk, idesc, 1);
-                umma::mma_commit(&empty[s]);
+                    for (int kk = 0; kk < 4; ++kk)
+                        umma::mma_f16(d1, ad2 + 2 * kk, bd + 2 * kk, idesc, 1);
+                    umma::mma_commit(&empty[s]);
+                }
+                __syncwarp();
             }
-            umma::mma_commit(&acc_full[b]);
+            if (umma::elect_one()) umma::mma_commit(&acc_full[b]);
+            __syncwarp();
         }
     } else if (warp >= 2) {
         // ----------------------------------------------------- epilogue

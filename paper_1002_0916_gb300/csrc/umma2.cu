@@ -52,7 +52,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tA,
 
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const uint32_t rank = umma2::cluster_rank();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = umma::warp_index(), lane = threadIdx.x & 31;
     const int m0 = blockIdx.y * 2 * S::BM + (int)rank * S::BM;  // this CTA's rows
     const int np0 = (blockIdx.x >> 1) * BNP;                     // the pair's columns
     const int nb = np0 + (int)rank * S::BNH;                     // this CTA's B rows
@@ -83,8 +83,9 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tA,
     const uint32_t tmem = tmem_base;
     pdl_wait();  // operands come from (and D may be read by) the kernel before
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
         // ------------------------------------------ producer (both CTAs)
+        bool ok = true;
         int issued = 0;
         for (int kb = 0; kb < KB; ++kb) {
             const int s = kb % STAGES;
@@ -93,28 +94,31 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tA,
                 abort_flag = 1;
                 set_status(g.status, DEV_TIMEOUT);
             }
-            if (abort_flag) break;
+            ok = __all_sync(0xffffffffu, !abort_flag);
+            if (!ok) break;
             uint8_t *st = smem + (size_t)s * S::STAGE_BYTES;
-            // the even CTA's barrier counts the bytes of both CTAs' loads
-            if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * S::STAGE_BYTES);
             const uint32_t bar = umma2::map_to_rank(&full[s], 0);
-            umma2::tma_load_2d_pair(st, &tA, kb * S::BK, m0, bar);
-            umma2::tma_load_2d_pair(st + S::A_BYTES, &tB, kb * S::BK, nb, bar);
-            if (SPLIT) {
-                umma2::tma_load_2d_pair(st + S::A_BYTES + S::B_BYTES, &tA2, kb * S::BK,
-                                        m0, bar);
-                umma2::tma_load_2d_pair(st + 2 * S::A_BYTES + S::B_BYTES, &tB2,
-                                        kb * S::BK, nb, bar);
+            if (umma::elect_one()) {
+                // the even CTA's barrier counts the bytes of both CTAs' loads
+                if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * S::STAGE_BYTES);
+                umma2::tma_load_2d_pair(st, &tA, kb * S::BK, m0, bar);
+                umma2::tma_load_2d_pair(st + S::A_BYTES, &tB, kb * S::BK, nb, bar);
+                if (SPLIT) {
+                    umma2::tma_load_2d_pair(st + S::A_BYTES + S::B_BYTES, &tA2, kb * S::BK,
+                                            m0, bar);
+                    umma2::tma_load_2d_pair(st + 2 * S::A_BYTES + S::B_BYTES, &tB2,
+                                            kb * S::BK, nb, bar);
+                }
             }
             ++issued;
         }
-        if (abort_flag && rank == 0) {
+        if (!ok && rank == 0) {
             // let the stages' copies land before shared memory goes: their
             // barriers are here (the odd CTA cannot see its own loads'
             // completion; it leaves only after the closing cluster barrier)
             for (int kb = issued - STAGES < 0 ? 0 : issued - STAGES; kb < issued; ++kb)
                 mbar_wait_bounded(&full[kb % STAGES], (uint32_t)((kb / STAGES) & 1));
-        } else if (!abort_flag) {
+        } else if (ok) {
             // The MMA issuer's commits of the last stages arrive on this
             // CTA's empty barriers asynchronously (multicast to both CTAs),
             // and nothing else waits for them: wait here (bounded), so that
@@ -123,51 +127,55 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tA,
             for (int kb = KB - STAGES < 0 ? 0 : KB - STAGES; kb < KB; ++kb)
                 mbar_wait_bounded(&empty[kb % STAGES], (uint32_t)((kb / STAGES) & 1));
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         if (rank == 0) {
             // ---------------------------------------- MMA issuer (even CTA)
             int done = 0;
             for (int kb = 0; kb < KB; ++kb) {
                 const int s = kb % STAGES;
                 const uint32_t par = (uint32_t)((kb / STAGES) & 1);
-                if (!umma2::wait_cluster_bounded(&full[s], par)) {
+                if (!mbar_wait_bounded(&full[s], par)) {
                     abort_flag = 1;
                     set_status(g.status, DEV_TIMEOUT);
                 }
-                if (abort_flag) break;
+                if (!__all_sync(0xffffffffu, !abort_flag)) break;
                 umma::fence_after_sync();
                 const uint32_t a = smem_u32(smem + (size_t)s * S::STAGE_BYTES);
                 const uint32_t b = a + S::A_BYTES;
+                const uint32_t a2 = b + S::B_BYTES, b2 = a2 + S::A_BYTES;
                 const uint64_t ad = umma::sw128_kmajor_desc(a);
                 const uint64_t bd = umma::sw128_kmajor_desc(b);
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    umma2::mma2_f16(tmem, ad + 2 * kk, bd + 2 * kk, idesc, (kb | kk) != 0);
-                if (SPLIT) {
-                    const uint32_t a2 = b + S::B_BYTES, b2 = a2 + S::A_BYTES;
-                    const uint64_t ad2 = umma::sw128_kmajor_desc(a2);
-                    const uint64_t bd2 = umma::sw128_kmajor_desc(b2);
+                const uint64_t ad2 = umma::sw128_kmajor_desc(a2);
+                const uint64_t bd2 = umma::sw128_kmajor_desc(b2);
+                if (umma::elect_one()) {
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk)
-                        umma2::mma2_f16(tmem + S::ACC1, ad + 2 * kk, bd2 + 2 * kk, idesc,
-                                        (kb | kk) != 0);
+                        umma2::mma2_f16(tmem, ad + 2 * kk, bd + 2 * kk, idesc, (kb | kk) != 0);
+                    if (SPLIT) {
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        umma2::mma2_f16(tmem + S::ACC1, ad2 + 2 * kk, bd + 2 * kk, idesc, 1);
+                        for (int kk = 0; kk < 4; ++kk)
+                            umma2::mma2_f16(tmem + S::ACC1, ad + 2 * kk, bd2 + 2 * kk, idesc,
+                                            (kb | kk) != 0);
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk)
+                            umma2::mma2_f16(tmem + S::ACC1, ad2 + 2 * kk, bd + 2 * kk, idesc,
+                                            1);
+                    }
+                    umma2::commit2(&empty[s], 0x3);
                 }
-                umma2::commit2(&empty[s], 0x3);
+                __syncwarp();
                 ++done;
             }
             // both CTAs' accumulators are complete -- or, after a timeout,
             // only this CTA learns that its MMAs in flight have finished (the
             // odd CTA's epilogue wait then runs out and skips its store)
-            umma2::commit2(&accum_bar, done == KB ? 0x3 : 0x1);
+            if (umma::elect_one()) umma2::commit2(&accum_bar, done == KB ? 0x3 : 0x1);
         }
     } else if (warp >= 2) {
         // --------------------------------------- epilogue (both CTAs)
         const int q = warp & 3;  // the 32-lane quarter of TMEM this warp reads
         const int row = m0 + q * 32 + lane;
-        const bool ok = __all_sync(0xffffffffu, umma2::wait_cluster_bounded(&accum_bar, 0));
+        const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&accum_bar, 0));
         umma::fence_after_sync();
         pdl_trigger();  // only the epilogue is left
         if (!ok) set_status(g.status, DEV_TIMEOUT);
@@ -333,7 +341,7 @@ umma_grouped_pair_kernel(const GroupProb *__restrict__ probs,
 
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const uint32_t rank = umma2::cluster_rank();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = umma::warp_index(), lane = threadIdx.x & 31;
     const int cl = blockIdx.x >> 1, ncl = gridDim.x >> 1;
 
     if (threadIdx.x == 0) {
@@ -357,10 +365,11 @@ umma_grouped_pair_kernel(const GroupProb *__restrict__ probs,
     umma::fence_after_sync();
     const uint32_t tmem = tmem_base;
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
         // ------------------------------------------ producer (both CTAs)
+        bool ok = true;
         unsigned g = 0, issued_from = 0;
-        for (int it = cl; it < nitems && !abort_flag; it += ncl) {
+        for (int it = cl; it < nitems && ok; it += ncl) {
             const uint2 w = items[it];
             const GroupProb *gp = probs + w.x;
             const int m0 = (int)(w.y & 0xffffu) * 2 * S::BM + (int)rank * S::BM;
@@ -373,24 +382,27 @@ umma_grouped_pair_kernel(const GroupProb *__restrict__ probs,
                     abort_flag = 1;
                     set_status(status, DEV_TIMEOUT);
                 }
-                if (abort_flag) break;
+                ok = __all_sync(0xffffffffu, !abort_flag);
+                if (!ok) break;
                 uint8_t *st = smem + (size_t)s * S::STAGE_BYTES;
-                if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * S::STAGE_BYTES);
                 const uint32_t bar = umma2::map_to_rank(&full[s], 0);
-                umma2::tma_load_2d_pair(st, &gp->tA, kb * S::BK, m0, bar);
-                umma2::tma_load_2d_pair(st + S::A_BYTES, &gp->tB, kb * S::BK, nb, bar);
-                umma2::tma_load_2d_pair(st + S::A_BYTES + S::B_BYTES, &gp->tA2,
-                                        kb * S::BK, m0, bar);
-                umma2::tma_load_2d_pair(st + 2 * S::A_BYTES + S::B_BYTES, &gp->tB2,
-                                        kb * S::BK, nb, bar);
+                if (umma::elect_one()) {
+                    if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * S::STAGE_BYTES);
+                    umma2::tma_load_2d_pair(st, &gp->tA, kb * S::BK, m0, bar);
+                    umma2::tma_load_2d_pair(st + S::A_BYTES, &gp->tB, kb * S::BK, nb, bar);
+                    umma2::tma_load_2d_pair(st + S::A_BYTES + S::B_BYTES, &gp->tA2,
+                                            kb * S::BK, m0, bar);
+                    umma2::tma_load_2d_pair(st + 2 * S::A_BYTES + S::B_BYTES, &gp->tB2,
+                                            kb * S::BK, nb, bar);
+                }
                 issued_from = g + 1;
             }
         }
-        if (abort_flag && rank == 0) {
+        if (!ok && rank == 0) {
             const unsigned lo = issued_from > STAGES ? issued_from - STAGES : 0;
             for (unsigned u = lo; u < issued_from; ++u)
                 mbar_wait_bounded(&full[u % STAGES], (uint32_t)((u / STAGES) & 1));
-        } else if (!abort_flag) {
+        } else if (ok) {
             // The MMA issuer's commits of the last stages arrive on this
             // CTA's empty barriers asynchronously (multicast to both CTAs),
             // and nothing else waits for them: wait here (bounded), so that
@@ -400,32 +412,33 @@ umma_grouped_pair_kernel(const GroupProb *__restrict__ probs,
             for (unsigned u = lo; u < g; ++u)
                 mbar_wait_bounded(&empty[u % STAGES], (uint32_t)((u / STAGES) & 1));
         }
-    } else if (warp == 1 && lane == 0 && rank == 0) {
+    } else if (warp == 1 && rank == 0) {
         // ---------------------------------------- MMA issuer (even CTA)
         const uint32_t idesc = umma::idesc_f16(2 * S::BM, GP_BN, false);
         unsigned g = 0;
         int n = 0;
-        for (int it = cl; it < nitems && !abort_flag; it += ncl, ++n) {
+        bool ok = true;
+        for (int it = cl; it < nitems && ok; it += ncl, ++n) {
             const int b = n & 1;
-            if (!umma2::wait_cluster_bounded(&acc_empty[b],
+            if (!mbar_wait_bounded(&acc_empty[b],
                                              (uint32_t)(((n >> 1) & 1) ^ 1))) {
                 abort_flag = 1;
                 set_status(status, DEV_TIMEOUT);
-                break;
             }
+            ok = __all_sync(0xffffffffu, !abort_flag);
+            if (!ok) break;
             umma::fence_after_sync();
             const uint32_t d0 = tmem + (uint32_t)b * ACC_COLS, d1 = d0 + GP_BN;
             const GroupProb *gp = probs + items[it].x;
             const int KB = (gp->K + S::BK - 1) / S::BK;
-            bool ok = true;
             for (int kb = 0; kb < KB; ++kb, ++g) {
                 const int s = (int)(g % STAGES);
-                if (!umma2::wait_cluster_bounded(&full[s], (uint32_t)((g / STAGES) & 1))) {
+                if (!mbar_wait_bounded(&full[s], (uint32_t)((g / STAGES) & 1))) {
                     abort_flag = 1;
                     set_status(status, DEV_TIMEOUT);
-                    ok = false;
-                    break;
                 }
+                ok = __all_sync(0xffffffffu, !abort_flag);
+                if (!ok) break;
                 umma::fence_after_sync();
                 const uint32_t a = smem_u32(smem + (size_t)s * S::STAGE_BYTES);
                 const uint32_t bb = a + S::A_BYTES;
@@ -434,20 +447,24 @@ umma_grouped_pair_kernel(const GroupProb *__restrict__ probs,
                 const uint64_t bd = umma::sw128_kmajor_desc(bb);
                 const uint64_t ad2 = umma::sw128_kmajor_desc(a2);
                 const uint64_t bd2 = umma::sw128_kmajor_desc(b2);
+                if (umma::elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    umma2::mma2_f16(d0, ad + 2 * kk, bd + 2 * kk, idesc, (kb | kk) != 0);
+                    for (int kk = 0; kk < 4; ++kk)
+                        umma2::mma2_f16(d0, ad + 2 * kk, bd + 2 * kk, idesc, (kb | kk) != 0);
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    umma2::mma2_f16(d1, ad + 2 * kk, bd2 + 2 * kk, idesc, (kb | kk) != 0);
+                    for (int kk = 0; kk < 4; ++kk)
+                        umma2::mma2_f16(d1, ad + 2 * kk, bd2 + 2 * kk, idesc, (kb | kk) != 0);
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    umma2::mma2_f16(d1, ad2 + 2 * kk, bd + 2 * kk, idesc, 1);
-                umma2::commit2(&empty[s], 0x3);
+                    for (int kk = 0; kk < 4; ++kk)
+                        umma2::mma2_f16(d1, ad2 + 2 * kk, bd + 2 * kk, idesc, 1);
+                    umma2::commit2(&empty[s], 0x3);
+                }
+                __syncwarp();
             }
             // a timed-out item is not handed to the odd CTA's epilogue (its
             // wait runs out); this CTA's epilogue learns that its MMAs ended
-            umma2::commit2(&acc_full[b], ok ? 0x3 : 0x1);
+            if (umma::elect_one()) umma2::commit2(&acc_full[b], ok ? 0x3 : 0x1);
+            __syncwarp();
         }
     } else if (warp >= 2) {
         // --------------------------------------- epilogue (both CTAs)
@@ -458,7 +475,7 @@ umma_grouped_pair_kernel(const GroupProb *__restrict__ probs,
             const int b = n & 1;
             const bool ok = __all_sync(
                 0xffffffffu,
-                umma2::wait_cluster_bounded(&acc_full[b], (uint32_t)((n >> 1) & 1)));
+                mbar_wait_bounded(&acc_full[b], (uint32_t)((n >> 1) & 1)));
             umma::fence_after_sync();
             if (!ok || abort_flag) {
                 if (!ok) set_status(status, DEV_TIMEOUT);
@@ -502,7 +519,7 @@ umma_grouped_pair_kernel(const GroupProb *__restrict__ probs,
             }
             umma::fence_before_sync();
             __syncwarp();
-            if (lane == 0) umma2::remote_arrive(lead_empty0 + (uint32_t)b * 8u);
+            if (lane == 0) umma2::arrive_pair(lead_empty0 + (uint32_t)b * 8u);
         }
     }
     umma::fence_before_sync();
