@@ -51,6 +51,7 @@
 #include "sep32.cuh"
 #include "sep_table.cuh"
 #include "umma.cuh"
+#include "umma_epi.cuh"
 #include "umma_pair.cuh"
 
 namespace cgh {
@@ -170,7 +171,7 @@ struct Sep32Args {
     float *part;         // [unit][cta rank][column / 4][row][4] partial tiles (S > 1)
     unsigned *count;     // [tile][cta rank] arrival counters, zero at launch (S > 1)
     int S;               // K slices
-    int vec;             // stores of 4 consecutive columns are 16-byte aligned
+    int vec;             // store_width(D, ldd)
     unsigned *status;
 };
 
@@ -214,7 +215,8 @@ __device__ __forceinline__ void sep32_promote(uint32_t taddr, int nu, float f,
 template <int BNP>
 __device__ __forceinline__ void sep32_store(const Sep32Args &g, bool ok, int mt, int nt, int slice,
                                             int rank, int half, int lrow, int m0, int np0,
-                                            int *s_last, float (&acc)[Sep32Cols<BNP>::U0 * 16]) {
+                                            int *s_last, float *stage,
+                                            float (&acc)[Sep32Cols<BNP>::U0 * 16]) {
     using C = Sep32Cols<BNP>;
     constexpr int BM = 128;
     const int nu = half ? C::U1 : C::U0, c0 = half * C::U0 * 16;
@@ -256,18 +258,32 @@ __device__ __forceinline__ void sep32_store(const Sep32Args &g, bool ok, int mt,
         }
     }
     const int row = m0 + lrow;
-    if (!store || row >= g.M) return;
+    if (!store) return;  // (the same in every lane)
+    if (!g.vec) {
+        const int lane = lrow & 31, row0 = row - lane;
+#pragma unroll
+        for (int u = 0; u < C::U0; ++u)
+            if (u < nu)
+                epilogue_store_odd(stage, acc + u * 16, g.D + (long long)row0 * g.ldd, g.ldd,
+                                   g.M - row0, np0 + c0 + u * 16, g.N, false, lane);
+        return;
+    }
+    if (row >= g.M) return;
     float *drow = g.D + (long long)row * g.ldd;
 #pragma unroll
-    for (int c = 0; c < C::U0 * 16; c += 4) {
+    for (int c = 0; c < C::U0 * 16; c += 8) {
         const int col = np0 + c0 + c;
         if (c >= nu * 16 || col >= g.N) break;
-        if (g.vec && col + 4 <= g.N) {
+        if (g.vec == 2 && col + 8 <= g.N) {
+            store8(drow + col, acc + c);
+        } else if (col + 8 <= g.N) {
             *reinterpret_cast<float4 *>(drow + col) =
                 make_float4(acc[c], acc[c + 1], acc[c + 2], acc[c + 3]);
+            *reinterpret_cast<float4 *>(drow + col + 4) =
+                make_float4(acc[c + 4], acc[c + 5], acc[c + 6], acc[c + 7]);
         } else {
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
+            for (int e = 0; e < 8; ++e)
                 if (col + e < g.N) drow[col + e] = acc[c + e];
         }
     }
@@ -523,6 +539,8 @@ sep32_pair_kernel(const __grid_constant__ Sep32Maps maps0,
         const int lrow = q * 32 + lane;
         const uint32_t t0 = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0;
         const uint32_t lead_empty = umma2::map_to_rank(&acc_empty[0], 0);
+        float *stage = reinterpret_cast<float *>(smem + (size_t)STAGES * S::STAGE_BYTES) +
+                       (warp - 4) * EPI_WARP_FLOATS;  // (forward only)
         bool ok = true;
         unsigned n = 0;
         for (int r = 0; r * ncl < g.units; ++r) {
@@ -559,7 +577,7 @@ sep32_pair_kernel(const __grid_constant__ Sep32Maps maps0,
             } else {
                 // (every warp, also after a timeout: it meets at barriers)
                 sep32_store<BNP>(g, ok, w.mt, w.nt, w.slice, (int)rank, half, lrow, m0,
-                                 w.nt * BNP, &s_last, acc);
+                                 w.nt * BNP, &s_last, stage, acc);
             }
         }
     }
@@ -618,19 +636,21 @@ template <int BNP, int STAGES, bool ADJ>
 static cudaError_t launch_sep32_kernel(const Sep32Maps &m0, const Sep32Maps &m1,
                                        const Sep32Args &g, const Adj32Args &ga, cudaStream_t s) {
     using S = PairShape<BNP, true, STAGES>;
+    constexpr size_t SMEM = ADJ ? S::RING : S::SMEM;
+    static_assert(SMEM <= 232448 - 1024, "shared memory");
     auto kern = sep32_pair_kernel<BNP, STAGES, ADJ>;
     static bool attr_set[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64 || !attr_set[dev]) {
         cudaError_t e = cudaFuncSetAttribute(
-            kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+            kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
     }
     const int pairs = sm_count_of_current_device() / 2;
     const int clusters = g.units < pairs ? g.units : pairs > 0 ? pairs : 1;
-    return launch_dependent(kern, dim3(2 * clusters), dim3(S32_THREADS), S::SMEM, s, m0, m1, g, ga,
+    return launch_dependent(kern, dim3(2 * clusters), dim3(S32_THREADS), SMEM, s, m0, m1, g, ga,
                             umma::idesc_f16(2 * S::BM, BNP, false));
 }
 
@@ -648,7 +668,7 @@ static cudaError_t launch_sep32(int bn, const Sep32Operands &op, const Sep32Args
     case 128: return launch_sep32_t<128, 4>(op, g, s);
     case 144: return launch_sep32_t<144, 4>(op, g, s);
     case 160: return launch_sep32_t<160, 4>(op, g, s);
-    case 192: return launch_sep32_t<192, 4>(op, g, s);
+    case 192: return launch_sep32_t<192, 3>(op, g, s);
     case 224: return launch_sep32_t<224, 3>(op, g, s);
     case 256: return launch_sep32_t<256, 3>(op, g, s);
     }
@@ -773,7 +793,7 @@ cgh_status cgh_ctx::forward_sep32(const float *points, const float *A, const flo
         g.part = part;
         g.count = count;
         g.S = plan.S;
-        g.vec = (Nx % 4 == 0) && (((uintptr_t)out & 15) == 0);
+        g.vec = store_width(out, Nx);
         g.status = d_status;
         cudaError_t e = launch_sep32(plan.bn, Sep32Operands{Rhi, Rlo, Lhi, Llo, Kp, Kp}, g, s);
         if (e != cudaSuccess) return cuda_fail(e, "FP32 separable product launch");

@@ -189,7 +189,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tA,
         if (ok && !abort_flag) {
             const uint32_t t_row = tmem + ((uint32_t)(q * 32) << 16);
             float *drow = g.D + (long long)row * g.ldd;
-            const bool vec = ((g.ldd & 3) == 0) && ((((uintptr_t)g.D) & 15) == 0);
+            const int vec = store_width(g.D, g.ldd);
             constexpr int CH = S::CH;
 #pragma unroll 1
             for (int c = 0; c < BN; c += CH) {
@@ -545,7 +545,7 @@ umma_grouped_kernel(const GroupProb *__restrict__ probs,
             const long long ldd = gp->ldd;
             const float los = gp->lo_scale;
             float *drow = gp->D + (long long)row * ldd;
-            const bool vec = ((ldd & 3) == 0) && ((((uintptr_t)gp->D) & 15) == 0);
+            const int vec = store_width(gp->D, ldd);
             const uint32_t t_row =
                 tmem + (uint32_t)b * ACC_COLS + ((uint32_t)(q * 32) << 16);
 #pragma unroll 1
@@ -560,7 +560,10 @@ umma_grouped_kernel(const GroupProb *__restrict__ probs,
                     v[i] = fmaf(los, __uint_as_float(r2[i]), __uint_as_float(r[i]));
                 if (row < M) {
                     const int col = n0 + c;
-                    if (vec && col + 32 <= Ncols) {
+                    if (vec == 2 && col + 32 <= Ncols) {
+#pragma unroll
+                        for (int i = 0; i < 32; i += 8) store8(drow + col + i, v + i);
+                    } else if (vec && col + 32 <= Ncols) {
 #pragma unroll
                         for (int i = 0; i < 32; i += 4)
                             *reinterpret_cast<float4 *>(drow + col + i) =

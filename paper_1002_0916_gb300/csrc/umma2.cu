@@ -35,8 +35,12 @@ namespace cgh {
 
 // Grid: x = 2 x (column blocks of BNP), y = row blocks of 256; clusters of
 // two CTAs along x.
+// Eight epilogue warps: the epilogue is latency (tensor-memory loads, then
+// stores), 2.9 us at 112 columns with four.
+constexpr int PAIR_THREADS = 64 + 32 * 8;
+
 template <int BNP, bool SPLIT, int STAGES>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PAIR_THREADS, 1)
 umma_pair_kernel(const __grid_constant__ CUtensorMap tA,
                  const __grid_constant__ CUtensorMap tB,
                  const __grid_constant__ CUtensorMap tA2,
@@ -182,10 +186,13 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tA,
         if (ok && !abort_flag) {
             const uint32_t t_row = tmem + ((uint32_t)(q * 32) << 16);
             float *drow = g.D + (long long)row * g.ldd;
-            const bool vec = ((g.ldd & 3) == 0) && ((((uintptr_t)g.D) & 15) == 0);
+            const int vec = store_width(g.D, g.ldd);
+            float *stage = reinterpret_cast<float *>(smem + (size_t)STAGES * S::STAGE_BYTES) +
+                           (warp - 2) * EPI_WARP_FLOATS;
             constexpr int CH = S::CH;
+            // the two warps of a quarter take every other chunk of columns
 #pragma unroll 1
-            for (int c = 0; c < BNP; c += CH) {
+            for (int c = ((warp - 2) >> 2) * CH; c < BNP; c += 2 * CH) {
                 uint32_t r[CH];
                 float v[CH];
                 if constexpr (CH == 32) umma::tmem_ld32(t_row + c, r);
@@ -204,7 +211,15 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tA,
 #pragma unroll
                     for (int i = 0; i < CH; ++i) v[i] = __uint_as_float(r[i]);
                 }
-                if (row < g.M) epilogue_store_row<CH>(drow, np0 + c, v, g, vec);
+                if (vec) {
+                    if (row < g.M) epilogue_store_row<CH>(drow, np0 + c, v, g, vec);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < CH; i += EPI_COLS)
+                        epilogue_store_odd(stage, v + i, drow - (long long)lane * g.ldd, g.ldd,
+                                           g.M - (row - lane), np0 + c + i, g.N, g.accumulate,
+                                           lane);
+                }
             }
         }
     }
@@ -224,6 +239,7 @@ template <int BNP, bool SPLIT, int STAGES>
 static cudaError_t launch_pair_t(const GemmOperands &op, unsigned *status,
                                  cudaStream_t s) {
     using S = PairShape<BNP, SPLIT, STAGES>;
+    static_assert(S::SMEM <= 232448 - 1024, "shared memory");
     CUtensorMap tA, tB, tA2, tB2;
     if (!make_gemm_map(&tA, op.A_hi, op.K, op.M, op.lda, S::BM, op.bf16) ||
         !make_gemm_map(&tB, op.B_hi, op.K, op.N, op.ldb, S::BNH, op.bf16))
@@ -249,7 +265,7 @@ static cudaError_t launch_pair_t(const GemmOperands &op, unsigned *status,
     GemmArgs g{op.M, op.N, op.K, op.D, op.ldd, op.lo_scale, status, op.accumulate};
     dim3 grid(2 * ((op.N + BNP - 1) / BNP), (op.M + 2 * S::BM - 1) / (2 * S::BM));
     const uint32_t idesc = umma::idesc_f16(2 * S::BM, BNP, op.bf16);
-    return launch_dependent(kern, grid, dim3(192), S::SMEM, s, tA, tB, tA2, tB2, g,
+    return launch_dependent(kern, grid, dim3(PAIR_THREADS), S::SMEM, s, tA, tB, tA2, tB2, g,
                             idesc);
 }
 
@@ -305,8 +321,8 @@ cudaError_t launch_umma_pair(const GemmOperands &op, int bnp, unsigned *status,
         case 112: return launch_pair_t<112, false, 9>(op, status, s);
         case 144: return launch_pair_t<144, false, 8>(op, status, s);
         case 160: return launch_pair_t<160, false, 8>(op, status, s);
-        case 224: return launch_pair_t<224, false, 7>(op, status, s);
-        case 256: return launch_pair_t<256, false, 7>(op, status, s);
+        case 224: return launch_pair_t<224, false, 6>(op, status, s);
+        case 256: return launch_pair_t<256, false, 6>(op, status, s);
         }
     }
     return cudaErrorInvalidValue;
@@ -490,7 +506,7 @@ umma_grouped_pair_kernel(const GroupProb *__restrict__ probs,
             const long long ldd = gp->ldd;
             const float los = gp->lo_scale;
             float *drow = gp->D + (long long)row * ldd;
-            const bool vec = ((ldd & 3) == 0) && ((((uintptr_t)gp->D) & 15) == 0);
+            const int vec = store_width(gp->D, ldd);
             const uint32_t t_row =
                 tmem + (uint32_t)b * ACC_COLS + ((uint32_t)(q * 32) << 16);
 #pragma unroll 1
@@ -505,7 +521,10 @@ umma_grouped_pair_kernel(const GroupProb *__restrict__ probs,
                     v[i] = fmaf(los, __uint_as_float(r2[i]), __uint_as_float(r[i]));
                 if (row < M) {
                     const int col = n0 + c;
-                    if (vec && col + 32 <= Ncols) {
+                    if (vec == 2 && col + 32 <= Ncols) {
+#pragma unroll
+                        for (int i = 0; i < 32; i += 8) store8(drow + col + i, v + i);
+                    } else if (vec && col + 32 <= Ncols) {
 #pragma unroll
                         for (int i = 0; i < 32; i += 4)
                             *reinterpret_cast<float4 *>(drow + col + i) =
@@ -538,7 +557,7 @@ cudaError_t prepare_umma_grouped_pair() {
     if (dev >= 0 && dev < 64 && attr_set[dev]) return cudaSuccess;
     cudaError_t e = cudaFuncSetAttribute(umma_grouped_pair_kernel<GP_STAGES>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)S::SMEM);
+                                         (int)S::RING);
     if (e == cudaSuccess && dev >= 0 && dev < 64) attr_set[dev] = true;
     return e;
 }
@@ -550,7 +569,7 @@ cudaError_t launch_umma_grouped_pair(const GroupProb *probs, const uint2 *items,
     if (nitems <= 0) return cudaSuccess;
     const int clusters = nitems < sm_count / 2 ? nitems : sm_count / 2;
     umma_grouped_pair_kernel<GP_STAGES><<<2 * (clusters > 0 ? clusters : 1), 192,
-                                          S::SMEM, s>>>(probs, items, nitems, status);
+                                          S::RING, s>>>(probs, items, nitems, status);
     return cudaGetLastError();
 }
 

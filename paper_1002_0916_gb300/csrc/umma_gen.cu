@@ -303,13 +303,13 @@ static cudaError_t launch_gen_t(const GenArgs &ga, const GemmArgs &g, cudaStream
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64 || !attr_set[dev]) {
         cudaError_t e = cudaFuncSetAttribute(
-            kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+            kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::RING);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
     }
     dim3 grid(2 * ((g.N + BNP - 1) / BNP), (g.M + 2 * S::BM - 1) / (2 * S::BM));
     const uint32_t idesc = umma::idesc_f16(2 * S::BM, BNP, KIND == 0);
-    return launch_dependent(kern, grid, dim3(GEN_THREADS), S::SMEM, s, ga, g, idesc);
+    return launch_dependent(kern, grid, dim3(GEN_THREADS), S::RING, s, ga, g, idesc);
 }
 
 static cudaError_t launch_gen_one(const GenArgs &ga, const GemmArgs &g, int kind, int bnp,

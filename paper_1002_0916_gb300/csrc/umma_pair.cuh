@@ -6,6 +6,7 @@
 
 #include "common.cuh"
 #include "umma.cuh"
+#include "umma_epi.cuh"
 
 namespace cgh {
 namespace umma2 {
@@ -149,11 +150,13 @@ struct PairShape {
         ACC_COLS <= 32 ? 32 : ACC_COLS <= 64 ? 64 : ACC_COLS <= 128 ? 128
         : ACC_COLS <= 256 ? 256 : 512;
     static constexpr int CH = BNP % 32 == 0 ? 32 : 16;
-    static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024;
+    static constexpr size_t RING = (size_t)STAGES * STAGE_BYTES + 1024;
+    // with the epilogue warps' staging of odd rows (umma_epi.cuh)
+    static constexpr size_t SMEM = RING + 8 * EPI_WARP_FLOATS * sizeof(float);
     static_assert(BNH % 8 == 0, "each B half is whole 8-row swizzle atoms");
     static_assert(BNP % 16 == 0 && BNP >= 32 && BNP <= 256, "UMMA N at M = 256");
     static_assert(ACC_COLS <= 512, "TMEM");
-    static_assert(SMEM <= 232448, "shared memory");
+    static_assert(RING <= 232448, "shared memory");
 };
 
 }  // namespace cgh
