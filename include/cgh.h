@@ -225,14 +225,15 @@ typedef struct {
     float *out;
 } cgh_problem;
 
-/* Many holograms of uneven size, N and wavelength in one persistent launch
+/* Many holograms of uneven size, N and wavelength in one launch
  * (after one prologue launch).  Each problem is one evaluation of Eq. 1
  * (Section 1) with its own points, constants and frame; the paper's
  * Table 1 runs the same 1,920 x 1,024 frame once per point count, and this
  * call runs many such frames (of any size) as one piece of device work.  probs: host array of `count` problems
  * (1 <= count <= 4096).  The work list of (problem, tile) items is built on
- * the host, sorted longest-first, and pulled by the persistent CTAs from an
- * atomic counter.  method: CGH_DIRECT_FP32 or CGH_SEP_FP16X3.
+ * the host, sorted longest-first; the direct method runs one CTA per item in
+ * that order, the tensor-core method persistent CTAs that pull the items from
+ * an atomic counter.  method: CGH_DIRECT_FP32 or CGH_SEP_FP16X3.
  * The launches are captured once per batch geometry (problem count, sizes,
  * constants and buffer addresses) into a CUDA graph that later calls of the
  * same geometry replay; the graph reads the buffers' current contents.
@@ -290,7 +291,7 @@ cgh_status cgh_forward_noalloc(const float *points, const float *A,
                                const float *z, int N, double lambda, double p,
                                int Nx, int Ny, float *out, void *stream);
 
-/* Tile shape of the direct kernel (also used by the persistent batch). */
+/* Tile shape of the direct kernel (also used by the batch). */
 typedef struct {
     int tile_x;            /* pixels per CTA along x           */
     int tile_y;            /* pixels per CTA along y           */
@@ -326,14 +327,16 @@ typedef struct {
  *   CGH_SCHED_GRID:  one CTA per pixel tile.  When the tile count is not a
  *                    multiple of the SM count the last wave leaves SMs idle.
  *   CGH_SCHED_SPLIT: one CTA per pixel tile, except for the last
- *                    (tiles mod SMs) tiles: their points are cut into chunks
- *                    of point stages, one CTA per chunk, run at the end of
- *                    the grid; each such tile is the sum of its chunks'
+ *                    (tiles mod SMs) tiles, or all of a few: where that is
+ *                    done sooner, their points are cut into chunks of point
+ *                    stages, one CTA per chunk, run at the end of the grid;
+ *                    each such tile is the sum of its chunks'
  *                    partial tiles added in chunk order (deterministic; the
  *                    rounding differs from GRID's by the summation order
  *                    only).
  *   CGH_SCHED_AUTO:  SPLIT (the default).
- * The batch entry point (cgh_batch) has its own persistent schedule. */
+ * The batch entry point (cgh_batch) has its own schedule: whole tiles, the
+ * problems with the most points first. */
 typedef enum {
     CGH_SCHED_AUTO = 0,
     CGH_SCHED_GRID = 1,

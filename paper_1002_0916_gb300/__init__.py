@@ -394,7 +394,7 @@ def _problems(problems):
 
 def cgh_batch(problems: Sequence[dict], *, method="direct", handle=None,
               stream=None):
-    """Many holograms in one persistent launch.  Each problem is a dict with
+    """Many holograms in one launch.  Each problem is a dict with
     points, A, z (CUDA tensors), lam, p, Nx, Ny and out (CUDA tensor)."""
     arr, n = _problems(problems)
     dev = problems[0]["A"].device.index if n else None
@@ -469,8 +469,8 @@ SCHEDULES = {"auto": 0, "grid": 1, "split": 2}
 
 def cgh_set_direct_schedule(h, schedule="auto"):
     """How the direct kernel spreads pixel tiles over the SMs: "grid" (one
-    CTA per tile), "split" (persistent CTAs with equal runs of (tile, point
-    stage) units, split tiles summed in a fixed order) or "auto"."""
+    CTA per tile), "split" (the tiles that do not share out evenly cut
+    into chunks of points, summed in a fixed order) or "auto"."""
     st = _L().cgh_set_direct_schedule(h, SCHEDULES[schedule])
     _check(h, st, "cgh_set_direct_schedule")
 

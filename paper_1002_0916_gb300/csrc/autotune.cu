@@ -30,17 +30,8 @@ std::string size_bucket(int method, int N, int Nx, int Ny) {
     return buf;
 }
 
-double direct_tile_cost(int i, int N, int Nx, int Ny, int sm_count) {
+double direct_update_cost(int i) {
     const DirectTile t = direct_tile_get(i);
-    // CTAs are handed to SMs as earlier ones finish: whole tiles per SM, and
-    // the rest cut into chunks of points (direct_split_plan) where a tile has
-    // points enough, else a last wave of whole tiles.  (Counting that wave
-    // whole took 32x32 tiles at 1366x768x777: 105 us against 92 with 64x32.)
-    long long ctas = (long long)((Nx + t.tx - 1) / t.tx) * ((Ny + t.ty - 1) / t.ty);
-    const long long rem = ctas % sm_count;
-    const bool split = rem > 0 && N >= 4 * t.pt;
-    const double waves = split ? (double)ctas / sm_count + 0.1
-                               : (double)((ctas + sm_count - 1) / sm_count);
     // Per-update cost model (in MUFU-cosine units), from the measured
     // rates: a quarter of the cosines on the FMA pipe saves about a
     // sixth, packed FP32x2 arithmetic a further 7-9%, shared-memory loads
@@ -65,15 +56,30 @@ double direct_tile_cost(int i, int N, int Nx, int Ny, int sm_count) {
         // 3840x2160x4096 (2.60 against 2.91 ms), 0.92 with 8x4
         if (t.pk == 8) per_pp *= t.vx >= 16 ? 0.89 : 0.92;
     }
-    return waves * t.tx * t.ty * per_pp;
+    return per_pp;
 }
 
+double direct_tile_cost(int i, int N, int Nx, int Ny, int sm_count) {
+    const DirectTile t = direct_tile_get(i);
+    // a tile's start and store take about as long as 10^5 updates of the
+    // fastest forms
+    const int Npad = pad_to(N > 0 ? N : 1, t.pt);
+    const DirectSplit d = direct_split_plan(i, sm_count, Npad, Nx, Ny, true);
+    return d.points / Npad * ((double)t.tx * t.ty * (N > 0 ? N : 1) * direct_update_cost(i) + 4e4);
+}
+
+// Of the two-axis rotation forms with eight point groups: the most accurate
+// (the FP32 chain of a pixel is N / 8 points long).  Of 19 frames of 256 to
+// 3840 pixels a side and 64 to 5000 points the choice is within 5% of the
+// fastest of all shapes in 18, 11% behind in one.
 int default_direct_tile(int N, int Nx, int Ny, int sm_count) {
     double best = 1e300;
     int best_i = 0;
     for (int i = 0; i < direct_tile_count(); ++i) {
+        const DirectTile t = direct_tile_get(i);
+        if (t.pk < 7 || t.g < 8) continue;
         const double cost = direct_tile_cost(i, N, Nx, Ny, sm_count);
-        if (cost < best - 1e-9) {
+        if (cost < best * (1.0 - 1e-9)) {
             best = cost;
             best_i = i;
         }

@@ -1,17 +1,19 @@
 // batch.cu -- many holograms of uneven size, point count and wavelength in
-// one persistent launch (step A9).
+// one launch (step A9).
 //
 // Direct FP32 batch:
 //   1. one prologue launch builds the point records of every problem
 //      (grid y = problem);
 //   2. one launch writes every problem's per-axis angle tables;
-//   3. one persistent launch (as many CTAs as fit on the SMs at once) pulls
-//      work items -- (problem, pixel tile) -- from an atomic counter, in the
-//      order of a host-built list sorted longest-first (by point count); each
-//      item runs the same staged point loop as the single-hologram kernel,
-//      with the shared-memory ring and its mbarriers carried from item to
-//      item.
-// The counter reset, the zero-fill of problems without points and the three
+//   3. one launch of a CTA per work item -- (problem, pixel tile) -- in the
+//      order of a host-built list sorted longest-first (by point count),
+//      which is the order the CTAs start in; each runs the same staged point
+//      loop as the single-hologram kernel.  (Persistent CTAs pulling the
+//      items from an atomic counter carried more state through the point
+//      loop than its registers hold: with the spills, 16 holograms of 512 to
+//      2048 pixels a side and up to 8192 points took 11.86 ms against 11.04
+//      with the same 64x32 tile.)
+// The zero-fill of problems without points and the three
 // launches are captured once per batch geometry into a CUDA graph on a
 // private stream and replayed on the caller's stream.  If the caller's
 // stream is itself being captured, the same nodes are enqueued on it instead.
@@ -40,7 +42,7 @@ struct BatchPrep {  // per problem: inputs and where its tables go
     DirectTables dt;
 };
 
-struct BatchTile {  // per problem: what the persistent kernel reads
+struct BatchTile {  // per problem: what the point loop reads
     const float *phx, *phy, *amp;
     float *out;
     int Npad, Nx, Ny, vec_store;
@@ -80,81 +82,57 @@ template <int TX, int TY, int VX, int VY, int PT, int NST, int NP, int G, int PK
 __global__ void __launch_bounds__(DirectTileLoop<TX, TY, VX, VY, PT, NST, NP, G, PK>::S::THREADS,
                                     DirectTileLoop<TX, TY, VX, VY, PT, NST, NP, G, PK>::MIN_CTAS)
 direct_batch_kernel(const BatchTile *__restrict__ probs,
-                    const uint2 *__restrict__ items, int nitems,
-                    unsigned *counter, unsigned *status) {
+                    const uint2 *__restrict__ items, unsigned *status) {
     using L = DirectTileLoop<TX, TY, VX, VY, PT, NST, NP, G, PK>;
     extern __shared__ __align__(128) float smem[];
     __shared__ __align__(8) uint64_t full[NST];
     __shared__ volatile int abort_flag;
-    __shared__ int s_item;
     if (threadIdx.x == 0) {
         abort_flag = 0;
         for (int s = 0; s < NST; ++s) mbar_init(&full[s], 1);
         mbar_fence_init();
     }
-    unsigned g = 0;  // stage loads this CTA has issued so far
-    for (;;) {
-        if (threadIdx.x == 0) s_item = (int)atomicAdd(counter, 1u);
-        __syncthreads();
-        const int it = s_item;
-        __syncthreads();
-        if (it >= nitems) break;
-        const uint2 w = items[it];
-        const BatchTile bt = probs[w.x];
-        const int xt = (int)(w.y & 0xffffu), yt = (int)(w.y >> 16);
-        const int ntile = bt.Npad / PT;
-        typename L::Acc acc;
-        acc.zero();
-        if (!L::accumulate(smem, full, &abort_flag,
-                           bt.phx + (size_t)xt * bt.Npad * TX * L::XF,
-                           bt.phy + (size_t)yt * bt.Npad * TY * L::YF, bt.amp, ntile, g,
-                           acc,
-                           status))
-            return;
-        g += (unsigned)ntile;
-        L::store(acc, smem, xt, yt, bt.Nx, bt.Ny, bt.out, bt.vec_store);
-    }
+    __syncthreads();
+    const uint2 w = items[blockIdx.x];
+    const int xt = (int)(w.y & 0xffffu), yt = (int)(w.y >> 16);
+    const BatchTile &bt = probs[w.x];
+    typename L::Acc acc;
+    acc.zero();
+    if (!L::accumulate(smem, full, &abort_flag, bt.phx + (size_t)xt * bt.Npad * TX * L::XF,
+                       bt.phy + (size_t)yt * bt.Npad * TY * L::YF, bt.amp, bt.Npad / PT, acc, status))
+        return;
+    L::store(acc, smem, xt, yt, bt.Nx, bt.Ny, bt.out, bt.vec_store);
 }
 
 template <int TX, int TY, int VX, int VY, int PT, int NST, int NP, int G, int PK>
 static cudaError_t launch_batch_t(const BatchTile *probs, const uint2 *items,
-                                  int nitems, unsigned *counter, unsigned *status,
-                                  int sm_count, cudaStream_t s) {
-    // probs == nullptr: only set the kernel's attributes and cache its
-    // occupancy (done before any capture)
+                                  int nitems, unsigned *status, cudaStream_t s) {
+    // probs == nullptr: only set the kernel's attribute (done before any
+    // capture; once per device)
     using S = typename DirectTileLoop<TX, TY, VX, VY, PT, NST, NP, G, PK>::S;
     auto kern = direct_batch_kernel<TX, TY, VX, VY, PT, NST, NP, G, PK>;
-    // attribute and occupancy once per device (no such calls inside a capture
-    // of a geometry that has run before)
-    static int per_sm_cache[64] = {};
+    static bool attr_set[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
-    int per_sm = (dev >= 0 && dev < 64) ? per_sm_cache[dev] : 0;
-    if (per_sm == 0) {
+    if (dev < 0 || dev >= 64 || !attr_set[dev]) {
         cudaError_t e = cudaFuncSetAttribute(
             kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
         if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, S::THREADS,
-                                                          S::SMEM);
-        if (e != cudaSuccess) return e;
-        per_sm = std::max(1, per_sm);
-        if (dev >= 0 && dev < 64) per_sm_cache[dev] = per_sm;
+        if (dev >= 0 && dev < 64) attr_set[dev] = true;
     }
     if (!probs) return cudaSuccess;
-    int grid = per_sm * sm_count;
-    if (grid > nitems) grid = nitems;
-    kern<<<grid, S::THREADS, S::SMEM, s>>>(probs, items, nitems, counter, status);
+    kern<<<nitems, S::THREADS, S::SMEM, s>>>(probs, items, status);
     return cudaGetLastError();
 }
 
 static cudaError_t launch_batch(int tile_index, const BatchTile *probs,
-                                const uint2 *items, int nitems, unsigned *counter,
-                                unsigned *status, int sm_count, cudaStream_t s) {
+                                const uint2 *items, int nitems, unsigned *status,
+                                cudaStream_t s) {
     int i = 0;
 #define X(tx, ty, vx, vy, pt, ns, np, g, pk)                                    \
     if (tile_index == i)                                                        \
         return launch_batch_t<tx, ty, vx, vy, pt, ns, np, g, pk>(                \
-            probs, items, nitems, counter, status, sm_count, s);                \
+            probs, items, nitems, status, s);                                   \
     ++i;
     CGH_DIRECT_TILES(X)
 #undef X
@@ -336,21 +314,19 @@ cgh_status cgh_ctx::batch_direct(const cgh_problem *probs, int count,
             for (int xt = 0; xt < prep[k].dt.nxt; ++xt)
                 items.push_back(make_uint2((unsigned)k, (unsigned)xt | ((unsigned)yt << 16)));
     const int nitems = (int)items.size();
-    // ---- metadata: counter | prep | tiles | items
-    const size_t c_b = 256;
+    // ---- metadata: prep | tiles | items
     const size_t prep_b = align256(prep.size() * sizeof(BatchPrep));
     const size_t tile_b = align256(tiles.size() * sizeof(BatchTile));
     const size_t item_b = align256(items.size() * sizeof(uint2));
-    const size_t meta_b = c_b + prep_b + tile_b + item_b;
+    const size_t meta_b = std::max<size_t>(prep_b + tile_b + item_b, 256);
     st = ensure(meta, meta_b, s, "batch metadata");
     if (st) return st;
     st = ensure_host_stage(meta_b);
     if (st) return st;
     char *mb = (char *)meta.ptr;
-    unsigned *counter = (unsigned *)mb;
-    BatchPrep *d_prep = (BatchPrep *)(mb + c_b);
-    BatchTile *d_tiles = (BatchTile *)(mb + c_b + prep_b);
-    uint2 *d_items = (uint2 *)(mb + c_b + prep_b + tile_b);
+    BatchPrep *d_prep = (BatchPrep *)mb;
+    BatchTile *d_tiles = (BatchTile *)(mb + prep_b);
+    uint2 *d_items = (uint2 *)(mb + prep_b + tile_b);
 
     uint64_t key = 1469598103934665603ull;
     const int method = CGH_DIRECT_FP32;
@@ -367,16 +343,15 @@ cgh_status cgh_ctx::batch_direct(const cgh_problem *probs, int count,
                                               ((bp.dt.Npad + DT_POINTS - 1) / DT_POINTS));
     }
     const int np = (int)prep.size();
-    cudaError_t e = launch_batch(tile_index, nullptr, nullptr, 0, nullptr, nullptr,
-                                 sm_count, s);
+    cudaError_t e = launch_batch(tile_index, nullptr, nullptr, 0, nullptr, s);
     if (e != cudaSuccess) return cuda_fail(e, "batch kernel set-up");
     auto fill = [&](char *hb) {
-        memcpy(hb + c_b, prep.data(), prep.size() * sizeof(BatchPrep));
-        memcpy(hb + c_b + prep_b, tiles.data(), tiles.size() * sizeof(BatchTile));
-        memcpy(hb + c_b + prep_b + tile_b, items.data(), items.size() * sizeof(uint2));
+        memcpy(hb, prep.data(), prep.size() * sizeof(BatchPrep));
+        memcpy(hb + prep_b, tiles.data(), tiles.size() * sizeof(BatchTile));
+        memcpy(hb + prep_b + tile_b, items.data(), items.size() * sizeof(uint2));
     };
     auto enqueue = [&](cudaStream_t q) -> cudaError_t {
-        cudaError_t r = cudaMemsetAsync(counter, 0, sizeof(unsigned), q);
+        cudaError_t r = cudaSuccess;
         for (int i = 0; i < count && r == cudaSuccess; ++i)
             if (probs[i].N == 0)
                 r = cudaMemsetAsync(probs[i].out, 0,
@@ -390,8 +365,7 @@ cgh_status cgh_ctx::batch_direct(const cgh_problem *probs, int count,
         batch_tables_kernel<<<g2, DT_SPAN, 0, q>>>(d_prep);
         r = cudaGetLastError();
         if (r != cudaSuccess) return r;
-        return launch_batch(tile_index, d_tiles, d_items, nitems, counter, d_status,
-                            sm_count, q);
+        return launch_batch(tile_index, d_tiles, d_items, nitems, d_status, q);
     };
     return run_batch_graph(key, meta_b, np ? 3 : 0, fill, enqueue, s, CGH_K_BATCH);
 }
@@ -429,15 +403,33 @@ cgh_status cgh_ctx::batch(const cgh_problem *probs, int count, int method,
                 "batch method must be CGH_DIRECT_FP32 or CGH_SEP_FP16X3");
 }
 
-// Untuned: the heuristic's shape for the problem with the most work
-// (persistent CTAs balance the rest).
+// Untuned: the shape of the least work over the batch (of every k-th problem
+// of a batch of more than 64): the tiles' updates per SM at the shape's rate,
+// and a last wave of the problem with the fewest points, whose tiles run last.
 int cgh_ctx::default_batch_tile(const cgh_problem *probs, int count) {
-    int big = 0;
-    for (int i = 1; i < count; ++i)
-        if ((double)probs[i].N * probs[i].Nx * probs[i].Ny >
-            (double)probs[big].N * probs[big].Nx * probs[big].Ny)
-            big = i;
-    return default_direct_tile(probs[big].N, probs[big].Nx, probs[big].Ny, sm_count);
+    const int step = (count + 63) / 64;
+    double best = 1e300;
+    int best_i = 0;
+    for (int i = 0; i < direct_tile_count(); ++i) {
+        const DirectTile t = direct_tile_get(i);
+        if (t.pk < 7 || t.g < 8) continue;  // as default_direct_tile
+        double work = 0.0;
+        int least = 0;
+        for (int k = 0; k < count; k += step) {
+            const cgh_problem &p = probs[k];
+            if (p.N <= 0) continue;
+            const int Npad = pad_to(p.N, t.pt);
+            if (!least || Npad < least) least = Npad;
+            work += (double)((p.Nx + t.tx - 1) / t.tx) * ((p.Ny + t.ty - 1) / t.ty) * Npad;
+        }
+        const double cost = (work * step / sm_count + (double)least * direct_tile_ctas(i)) *
+                            t.tx * t.ty * direct_update_cost(i);
+        if (cost < best * (1.0 - 1e-9)) {
+            best = cost;
+            best_i = i;
+        }
+    }
+    return best_i;
 }
 
 std::string batch_bucket(const cgh_problem *probs, int count) {

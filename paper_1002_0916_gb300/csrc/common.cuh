@@ -209,6 +209,7 @@ cudaError_t launch_prologue(const float *points, const float *A,
 int direct_tile_count();
 DirectTile direct_tile_get(int i);
 int direct_tile_index(const DirectTile &t);
+int direct_tile_ctas(int i);  // CTAs that an SM holds at once
 size_t direct_phase_table_floats(const DirectTile &t, int Npad, int Nx, int Ny);
 // (zero, nzero): words the tables kernel sets to zero (the split
 // schedule's arrival counters), or (nullptr, 0)
@@ -246,13 +247,15 @@ cudaError_t launch_direct_tables_fused(const PointSource &src, int Npad, int Nx,
                                        float *phy, float *amp, unsigned *zero,
                                        int nzero, cudaStream_t s);
 // Tail split of the direct kernel: `tiles` pixel tiles, those from `tail`
-// on each cut into m chunks of point stages (tail == tiles: none).
+// on each cut into m chunks of point stages (tail == tiles: none); points:
+// those of the busiest SM's tiles.
 struct DirectSplit {
     int tiles, tail, m;
+    double points;
     int chunks() const { return (tiles - tail) * m; }
 };
 DirectSplit direct_split_plan(int tile_index, int sm_count, int Npad, int Nx,
-                              int Ny, bool split);
+                              int Ny, bool split, bool full = true);
 // part: chunks() partial tiles; count: tiles - tail words, zero at launch
 cudaError_t launch_direct_forward(int tile_index, const float *phx,
                                   const float *phy, const float *amp, int Npad,

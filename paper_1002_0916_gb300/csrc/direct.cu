@@ -24,7 +24,7 @@
 //    the shared-memory reads beside it.  With packed 16x4 blocks the pipe is
 //    73% and the shared-memory data path 76% busy (3840x2160x2048): 41.5
 //    updates per clock and SM of 58.5.  1920x1024x1024 204 -> 167 us,
-//    3840x2160x16384 11.13 -> 10.30 ms against scalar 16x4 blocks with the
+//    3840x2160x16384 11.13 -> 10.28 ms against scalar 16x4 blocks with the
 //    groups' sums stored in place.  Cosine-per-pixel tiles: the MUFU.
 //
 // Accuracy: angle rounding about 2^-22 rad per axis, __cosf absolute error
@@ -51,8 +51,10 @@ __global__ void __launch_bounds__(DT_SPAN)
 direct_tables_kernel(const PointRec *__restrict__ rec, PointSource src, DirectTables dt,
                      unsigned *__restrict__ zero, int nzero) {
     __shared__ PointRec srec[DT_POINTS];
+    // No early trigger for the direct kernel: placed while this kernel still
+    // runs, its CTAs would double up on the SMs that are free first
+    // (640x480x300: 26 us against 18; nothing gained elsewhere).
     pdl_wait();  // the records (or the caller's points) come from the kernel before
-    pdl_trigger();
     // the split schedule's per-tile arrival counters start at zero (every
     // earlier kernel on the stream has finished: pdl_wait above)
     if (blockIdx.x == 0)
@@ -121,7 +123,7 @@ direct_fwd_kernel(const float *__restrict__ phx, const float *__restrict__ phy,
     if (!L::accumulate(smem, full, &abort_flag,
                        phx + (size_t)xt * Npad * TX * L::XF + (size_t)s0 * S::SX,
                        phy + (size_t)yt * Npad * TY * L::YF + (size_t)s0 * S::SY,
-                       amp + (size_t)s0 * PT, s1 - s0, 0u, acc, status))
+                       amp + (size_t)s0 * PT, s1 - s0, acc, status))
         return;
     // only the stores are left: the next kernel of the stream may launch
     pdl_trigger();
@@ -260,23 +262,58 @@ cudaError_t launch_direct_tables_fused(const PointSource &src, int Npad, int Nx,
     return launch_tables(nullptr, &src, Npad, Nx, Ny, t, phx, phy, amp, zero, nzero, s);
 }
 
+static const int kTileCtas[] = {
+#define X(tx, ty, vx, vy, pt, ns, np, g, pk) \
+    DirectTileLoop<tx, ty, vx, vy, pt, ns, np, g, pk>::SM_CTAS,
+    CGH_DIRECT_TILES(X)
+#undef X
+};
+
+int direct_tile_ctas(int i) { return kTileCtas[i]; }
+
+// Which tiles to cut, and into how many chunks.  An SM gets through its CTAs
+// at about the same rate however many it holds (one alone 7% slower), so the
+// whole tiles are as many as share out evenly, and the others are cut so that
+// the busiest SM has the fewest points left, a chunk counted 20 points more
+// than its share, the cutting itself 60, and the sum of a tile's chunks the
+// time of 34000 updates (0.4 us) each.  All tiles
+// are cut where the whole ones would fill some of an SM's places only: 800x600
+// x2000 (247 tiles) 96 us against 110 with one whole tile per SM.  Kernel
+// times by the count of chunks follow this: 1023x767x1999, 80 tiles to cut,
+// 138 us in 11 chunks, 143 in 4 (always two chunks per SM, the former rule),
+// 156 in 2 or whole; 300x200x5000, 35 tiles, 41 us in 8, 51 in 9; 1920x1080
+// x4096, 108 tiles, 660 us in 4, 684 in 3; 1500x900x200 39 whole, 42 cut.
+// full: up to 8 chunks per SM, else 2 (less scratch).
 DirectSplit direct_split_plan(int tile_index, int sm_count, int Npad, int Nx,
-                              int Ny, bool split) {
+                              int Ny, bool split, bool full) {
     const DirectTile &t = kTiles[tile_index];
     DirectSplit d;
     d.tiles = ((Nx + t.tx - 1) / t.tx) * ((Ny + t.ty - 1) / t.ty);
     d.tail = d.tiles;
     d.m = 1;
     const int nst = Npad / t.pt;
-    const int rem = sm_count > 0 ? d.tiles % sm_count : 0;
-    if (!split || rem == 0 || nst < 2) return d;
-    // the last `rem` tiles, each cut into about 2 SMs' worth / rem chunks
-    d.tail = d.tiles - rem;
-    d.m = (2 * sm_count + rem - 1) / rem;
-    if (d.m > nst) d.m = nst;
-    if (d.m < 2) {
-        d.tail = d.tiles;
-        d.m = 1;
+    d.points = sm_count > 0 ? (double)((d.tiles + sm_count - 1) / sm_count) * Npad : 0.0;
+    if (!split || sm_count < 1 || nst < 2 || d.tiles % sm_count == 0) return d;
+    const int slots = sm_count * kTileCtas[tile_index];
+    const int most = (full ? 8 : 2) * sm_count;
+    const int even = d.tiles - d.tiles % sm_count;
+    for (int tail = even; tail >= 0; tail -= even > 0 ? even : 1) {
+        const int rest = d.tiles - tail;
+        for (int m = 2; m <= nst && rest * m <= most; ++m) {
+            const int ctas = tail + rest * m;
+            if (tail > 0 && tail < slots && ctas > slots) break;
+            const int rounds = (rest * m + sm_count - 1) / sm_count;
+            double points = (double)tail / sm_count * Npad +
+                            rounds * (double)((nst + m - 1) / m * t.pt + 20) + 60.0 +
+                            m * 34000.0 / (t.tx * t.ty);
+            if (ctas <= sm_count) points *= 1.07;
+            if (points < d.points) {
+                d.points = points;
+                d.tail = tail;
+                d.m = m;
+            }
+        }
+        if (even >= slots) break;
     }
     return d;
 }

@@ -1,6 +1,6 @@
 // direct_tile.cuh -- the staged point loop of the direct kernel for one
 // pixel tile, shared by the single-hologram kernel (direct.cu) and the
-// persistent batch kernel (batch.cu).  Internal to libcgh.
+// batch kernel (batch.cu).  Internal to libcgh.
 #pragma once
 
 #include "common.cuh"
@@ -221,10 +221,8 @@ struct DirectShape {
                   "partial sums of the extra groups fit in the stage ring");
 };
 
-// Per-CTA driver of the staged loop.  Point tile t of a pixel tile is the
-// (g0 + t)-th stage load of the CTA, so a persistent CTA can run many pixel
-// tiles back to back on the same NST-slot ring and mbarriers: slot
-// (g0 + t) % NST, barrier parity ((g0 + t) / NST) & 1.
+// The staged loop of one CTA: stage t is loaded into slot t % NST of the
+// ring, barrier parity (t / NST) & 1.
 template <int TX, int TY, int VX, int VY, int PT, int NST, int NP, int G,
           int PKV>
 struct DirectTileLoop {
@@ -253,6 +251,11 @@ struct DirectTileLoop {
     // rotation forms, two with 64-pixel blocks (at most 128 registers a
     // thread), three with 32-pixel blocks (at most 85)
     static constexpr int MIN_CTAS = PKV < 7 ? 1 : VX * VY >= 64 ? 2 : 3;
+    // CTAs that an SM holds at once: by their registers (two of the other
+    // forms), and by their shared memory with its 1 KB of the system's
+    static constexpr int REG_CTAS = PKV < 7 ? 2 : MIN_CTAS;
+    static constexpr int SMEM_CTAS = (int)(228 * 1024 / (S::SMEM + 1280));
+    static constexpr int SM_CTAS = SMEM_CTAS < REG_CTAS ? SMEM_CTAS : REG_CTAS;
     // (the two-axis rotation form updates its pixels one by one)
     using Acc = DirectAcc<VY, VX, PK && PKV != 7>;
     static_assert(PKV != 8 || VX % 4 == 0, "the packed two-axis form: column groups of 4 or 8");
@@ -387,8 +390,13 @@ struct DirectTileLoop {
             // order decides the FMA rate through the register operands.  Bare
             // rank-2 updates of a 16x4 block run at 52.5 pixels per clock and
             // SM in this order packed, 50.5 row by row, 47.1 scalar (8x8: 49.6,
-            // 46.6, 43.7); with the loads, 41.1 against 38.1 row by row and
-            // 38.0 scalar at 3840x2160x4096.
+            // 46.6, 43.7); with the loads, 41.5 against 38.1 row by row and
+            // 38.0 scalar at 3840x2160x4096.  What is left is the shared-
+            // memory path, 128 bytes per clock into the registers: 10 16-byte
+            // loads per point for 64 pixels keep it 84% busy.  (16x6 blocks
+            // in four point groups, 168 registers and 12 warps per SM, reach
+            // 43.7, but their FP32 chains are twice as long: 6.5e-7 from FP64
+            // at 2048 points against 5.3e-7; in two halves, 42.7.)
 #pragma unroll
             for (int k = 0; k < VX / 2; ++k) {
 #pragma unroll
@@ -484,13 +492,12 @@ struct DirectTileLoop {
     __device__ static bool accumulate(float *smem, uint64_t *full,
                                       volatile int *abort_flag, const float *gx,
                                       const float *gy, const float *amp,
-                                      int ntile, unsigned g0, Acc &acc,
+                                      int ntile, Acc &acc,
                                       unsigned *status) {
         int issued = 0;  // meaningful in thread 0 only
         if (threadIdx.x == 0) {
-            fence_proxy_async_smem();  // the ring may hold partial sums
             for (int s = 0; s < NST && s < ntile; ++s) {
-                issue(smem, full, gx, gy, amp, s, (int)((g0 + s) % NST));
+                issue(smem, full, gx, gy, amp, s, s);
                 ++issued;
             }
         }
@@ -498,9 +505,8 @@ struct DirectTileLoop {
         const int tx = lt % S::NTX, ty = lt / S::NTX;
         int t = 0;
         for (; t < ntile; ++t) {
-            const unsigned g = g0 + (unsigned)t;
-            const int s = (int)(g % NST);
-            const uint32_t par = (uint32_t)((g / NST) & 1);
+            const int s = t % NST;
+            const uint32_t par = (uint32_t)((t / NST) & 1);
             bool ok = mbar_wait_bounded(&full[s], par);
             if (!ok) {
                 *abort_flag = 1;
@@ -520,10 +526,8 @@ struct DirectTileLoop {
             // let the copies still in flight land before the shared memory
             // goes away (each wait bounded again)
             if (threadIdx.x == 0) {
-                for (int u = t; u < issued; ++u) {
-                    const unsigned g = g0 + (unsigned)u;
-                    mbar_wait_bounded(&full[g % NST], (uint32_t)((g / NST) & 1));
-                }
+                for (int u = t; u < issued; ++u)
+                    mbar_wait_bounded(&full[u % NST], (uint32_t)((u / NST) & 1));
             }
             return false;
         }
@@ -651,8 +655,7 @@ struct DirectTileLoop {
         }
     }
 
-    // Store the pixels of pixel tile (xt, yt).  Ends with the ring free for
-    // the next copies of a persistent CTA.
+    // Store the pixels of pixel tile (xt, yt).
     __device__ static void store(Acc &acc, float *smem, int xt, int yt, int Nx,
                                  int Ny, float *out, int vec_store) {
         if constexpr (QUADS) {
@@ -663,7 +666,6 @@ struct DirectTileLoop {
             reduce_groups(acc, smem);
             write_out(acc, xt, yt, Nx, Ny, out, vec_store);
         }
-        if (G > 1) __syncthreads();
     }
 };
 

@@ -199,14 +199,15 @@ extern "C" cgh_status cgh_forward_noalloc(const float *points, const float *A,
     if (tile_index < 0) return CGH_ERR_UNSUPPORTED;  // no tile's tables fit the array
     const DirectTile t = direct_tile_get(tile_index);
     const int Npad = pad_to(N > 0 ? N : 1, t.pt);
-    DirectSplit d = direct_split_plan(tile_index, sms, Npad, Nx, Ny, true);
-    ScratchPlan sp = plan_scratch(t, Npad, Nx, Ny, d);
-    if (N > 0 && sp.total > (size_t)CGH_NOALLOC_SCRATCH_BYTES) {
-        d = direct_split_plan(tile_index, sms, Npad, Nx, Ny, false);
+    DirectSplit d;
+    ScratchPlan sp;
+    for (int k = 0; k < 3; ++k) {  // split, split less, not split
+        d = direct_split_plan(tile_index, sms, Npad, Nx, Ny, k < 2, k == 0);
         sp = plan_scratch(t, Npad, Nx, Ny, d);
-        if (sp.total > (size_t)CGH_NOALLOC_SCRATCH_BYTES)
-            return CGH_ERR_UNSUPPORTED;  // this frame needs more scratch than exists
+        if (N == 0 || sp.total <= (size_t)CGH_NOALLOC_SCRATCH_BYTES) break;
     }
+    if (N > 0 && sp.total > (size_t)CGH_NOALLOC_SCRATCH_BYTES)
+        return CGH_ERR_UNSUPPORTED;  // this frame needs more scratch than exists
 
     void *base = nullptr;
     if (scratch_address(dev, &base) != cudaSuccess) {
