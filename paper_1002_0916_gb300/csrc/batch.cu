@@ -499,10 +499,10 @@ extern "C" cgh_status cgh_tune_batch(cgh_handle h, const cgh_problem *probs,
     if (prev != h->device) cudaSetDevice(h->device);
     cudaStream_t s = (cudaStream_t)stream;
     if (method == CGH_SEP_FP16X3) {
-        // the grouped split-FP16 GEMM's two item shapes: one-CTA items (the
-        // default) and CTA-pair items, each timed on its captured graph
+        // the grouped split-FP16 GEMM's two kinds of items: one-CTA items and
+        // CTA-pair items (the default), each timed on its captured graph
         int best_pairs = -1;
-        cgh_status st = tune_pick(h, 2, 0, TUNE_KEEP, s,
+        cgh_status st = tune_pick(h, 2, 1, TUNE_KEEP, s,
                                   [&](int pairs) {
                                       return h->batch(probs, count, method, s, -1, pairs);
                                   },
@@ -591,8 +591,15 @@ bool cgh_ctx::batch_sep_pairs(const cgh_problem *probs, int count, bool *tuned_o
     // CTA-pair items (256 x 128): batches of 64, 16 and 8 holograms of 512 to
     // 2048 pixels a side took 4.05, 1.00 and 0.50 ms with them, 4.16, 1.20 and
     // 0.58 with one-CTA items (128 x 128), which read twice the operand bytes
-    // per SM
+    // per SM (64 holograms over and over, at the power cap: 4.4 ms with either)
     return true;
+}
+
+// Columns per CTA-pair item of a problem of Nx columns: equal whole
+// thirty-twos, at most group_pair_tile_n().
+static int pair_item_columns(int Nx) {
+    const int bn = group_pair_tile_n(), nt = (Nx + bn - 1) / bn;
+    return pad_to((Nx + nt - 1) / nt, 32);
 }
 
 cgh_status cgh_ctx::batch_separable(const cgh_problem *probs, int count,
@@ -624,9 +631,8 @@ cgh_status cgh_ctx::batch_separable(const cgh_problem *probs, int count,
     if (st) return st;
     const bool pairs = pairs_override >= 0 ? pairs_override != 0
                                            : batch_sep_pairs(probs, count, nullptr);
-    const int TM = pairs ? group_pair_tile_m() : 128;
-    const int BN = pairs ? group_pair_tile_n() : group_tile_n();
-    const int b_box = pairs ? group_pair_box_b() : group_tile_n();
+    const int TM = pairs ? 256 : 128;
+    const int b_box = pairs ? group_pair_tile_n() / 2 : group_tile_n();
     cudaError_t e = pairs ? prepare_umma_grouped_pair() : prepare_umma_grouped();
     if (e != cudaSuccess) return cuda_fail(e, "grouped GEMM set-up");
     std::vector<GroupProb> gps(prep.size());
@@ -664,6 +670,7 @@ cgh_status cgh_ctx::batch_separable(const cgh_problem *probs, int count,
         ops[k] = op;
         if (!encode_group_prob(&gps[k], op, b_box))
             return fail(CGH_ERR_CUDA, "problem %d: tensor map encoding failed", pidx[k]);
+        gps[k].bw = pairs ? pair_item_columns(sp.Nx) : group_tile_n();
     }
     // items: (problem, m tile, n tile), largest K first
     std::vector<int> order(prep.size());
@@ -679,7 +686,7 @@ cgh_status cgh_ctx::batch_separable(const cgh_problem *probs, int count,
     for (int k : order)
         if (prep[k].Kp <= gemm_k_chunk(true))
         for (int mt = 0; mt < (prep[k].Ny + TM - 1) / TM; ++mt)
-            for (int nt = 0; nt < (prep[k].Nx + BN - 1) / BN; ++nt)
+            for (int nt = 0; nt * gps[k].bw < prep[k].Nx; ++nt)
                 items.push_back(make_uint2((unsigned)k, (unsigned)mt | ((unsigned)nt << 16)));
     const int nitems = (int)items.size();
     const size_t prep_b = align256(prep.size() * sizeof(SepPrep));

@@ -385,15 +385,8 @@ __device__ __forceinline__ Sep32Unit sep32_unit(int u, const Sep32Args &g, const
     return w;
 }
 
-// The r-th unit of cluster c of n: round by round, every other round in
-// reverse order, so that units sorted longest first spread evenly; units or
-// more: none in this round.
-__device__ __forceinline__ int sep32_unit_index(int r, int c, int n) {
-    return r * n + ((r & 1) ? n - 1 - c : c);
-}
-
 // Persistent: clusters of two CTAs (one per SM) take the units in
-// sep32_unit_index order; loads and MMAs run ahead into the next unit while
+// group_item_index order; loads and MMAs run ahead into the next unit while
 // the epilogue of the last one finishes.  ADJ: both products of the adjoint
 // in one list, the longer K first.
 template <int BNP, int STAGES, bool ADJ>
@@ -450,7 +443,7 @@ sep32_pair_kernel(const __grid_constant__ Sep32Maps maps0,
             unsigned n = 0;  // K blocks issued
             bool ok = true;
             for (int r = 0; r * ncl < g.units && ok; ++r) {
-                const int u = sep32_unit_index(r, cl, ncl);
+                const int u = group_item_index(r, cl, ncl);
                 if (u >= g.units) break;
                 const Sep32Unit w = sep32_unit<ADJ>(u, g, ga);
                 const Sep32Maps *maps = w.which ? &maps1 : &maps0;
@@ -496,7 +489,7 @@ sep32_pair_kernel(const __grid_constant__ Sep32Maps maps0,
             unsigned n = 0;
             bool ok = true;
             for (int r = 0; r * ncl < g.units && ok; ++r) {
-                const int u = sep32_unit_index(r, cl, ncl);
+                const int u = group_item_index(r, cl, ncl);
                 if (u >= g.units) break;
                 const int nkb = sep32_unit<ADJ>(u, g, ga).nkb;
                 for (int i = 0; i < nkb; ++i, ++n) {
@@ -551,7 +544,7 @@ sep32_pair_kernel(const __grid_constant__ Sep32Maps maps0,
         bool ok = true;
         unsigned n = 0;
         for (int r = 0; r * ncl < g.units; ++r) {
-            const int u = sep32_unit_index(r, cl, ncl);
+            const int u = group_item_index(r, cl, ncl);
             if (u >= g.units) break;
             const Sep32Unit w = sep32_unit<ADJ>(u, g, ga);
             float acc[C::U0 * 16];

@@ -168,6 +168,7 @@ struct alignas(alignof(CUtensorMap)) GroupProb {
     float *D;
     long long ldd;
     int M, N, K;
+    int bw;  // columns per CTA-pair item
     float lo_scale;
 };
 
@@ -181,14 +182,19 @@ cudaError_t launch_umma_grouped(const GroupProb *probs, const uint2 *items,
                                 cudaStream_t s);
 cudaError_t prepare_umma_grouped();
 int group_tile_n();
-// umma2.cu: the same on CTA pairs; items are (problem, 256-row tile,
-// group_pair_tile_n()-column tile)
+// umma2.cu: the same on CTA pairs; items are (problem, 256-row tile, column
+// tile of the problem's bw columns), bw at most group_pair_tile_n()
 cudaError_t launch_umma_grouped_pair(const GroupProb *probs, const uint2 *items,
                                      int nitems, unsigned *status, int sm_count,
                                      cudaStream_t s);
 cudaError_t prepare_umma_grouped_pair();
-int group_pair_tile_m();
 int group_pair_tile_n();
-int group_pair_box_b();
+
+// The r-th unit of cluster c of n: round by round, every other round in
+// reverse order, so that units sorted longest first spread evenly; the number
+// of units or more: none in this round.
+__device__ __forceinline__ int group_item_index(int r, int c, int n) {
+    return r * n + ((r & 1) ? n - 1 - c : c);
+}
 
 }  // namespace cgh

@@ -330,28 +330,43 @@ cudaError_t launch_umma_pair(const GemmOperands &op, int bnp, unsigned *status,
 
 // ------------------------------------------------ grouped (batch), pairs
 // The persistent grouped split GEMM of the batch on CTA pairs: clusters of
-// two CTAs take work items (problem, 256-row tile, 128-column tile) round
-// robin; per SM 128 rows of A and 64 rows of B per stage.  Two TMEM
-// accumulator buffers (hi*hi and cross terms, 256 columns each) let the
-// epilogue of one item overlap the MMAs of the next.  The even CTA's
-// `acc_empty` barrier collects one arrival from each of the 8 epilogue warps
-// of the pair (the odd CTA's arrive remotely) before that buffer is reused.
+// two CTAs take work items (problem, 256-row tile, column tile) in
+// group_item_index order; per SM 128 rows of A and 64 rows of B per stage.  An
+// item's columns are the problem's GroupProb::bw, at most 128, and fewer (whole
+// thirty-twos) at the frame's edge: the MMA's N.  Two TMEM accumulator buffers
+// (hi*hi and cross terms, 256 columns each) let the epilogue of one item
+// overlap the MMAs of the next.  The even CTA's `acc_empty` barrier collects
+// one arrival from each of the 16 epilogue warps of the pair (the odd CTA's
+// arrive remotely) before that buffer is reused.
+// Bound: the MMAs, 1.77 PFLOP/s with the rows that 256-row tiles pad (64
+// holograms, 3.38 ms with items dealt round robin in 128-column tiles, 3.23
+// in this order); over seconds the power cap.  Items of 256 columns, one
+// buffer: 3.44 ms.
 constexpr int GP_BN = 128, GP_STAGES = 4;
+constexpr int GP_EPI_WARPS = 8;
+constexpr int GP_THREADS = 64 + 32 * GP_EPI_WARPS;
+
+// The columns of an item at n0 (whole thirty-twos).
+__device__ __forceinline__ int group_item_columns(const GroupProb *gp, int n0) {
+    const int left = (gp->N - n0 + 31) & ~31;
+    return left < gp->bw ? left : gp->bw;
+}
 
 template <int STAGES>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GP_THREADS, 1)
 umma_grouped_pair_kernel(const GroupProb *__restrict__ probs,
                          const uint2 *__restrict__ items, int nitems,
                          unsigned *status) {
     using S = PairShape<GP_BN, true, STAGES>;
-    constexpr uint32_t ACC_COLS = 2 * GP_BN;        // hi*hi and cross terms
-    constexpr uint32_t TMEM_COLS = 2 * ACC_COLS;    // two buffers
+    constexpr int NBUF = 2;
+    constexpr uint32_t ACC_COLS = 2 * GP_BN;  // hi*hi and cross terms
+    constexpr uint32_t TMEM_COLS = NBUF * ACC_COLS;
     static_assert(TMEM_COLS <= 512, "TMEM");
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full[STAGES];
     __shared__ __align__(8) uint64_t empty[STAGES];
-    __shared__ __align__(8) uint64_t acc_full[2];
-    __shared__ __align__(8) uint64_t acc_empty[2];
+    __shared__ __align__(8) uint64_t acc_full[NBUF];
+    __shared__ __align__(8) uint64_t acc_empty[NBUF];
     __shared__ uint32_t tmem_base;
     __shared__ volatile int abort_flag;
 
@@ -366,9 +381,9 @@ umma_grouped_pair_kernel(const GroupProb *__restrict__ probs,
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < NBUF; ++b) {
             mbar_init(&acc_full[b], 1);
-            mbar_init(&acc_empty[b], 8);  // 4 epilogue warps in each CTA
+            mbar_init(&acc_empty[b], 2 * GP_EPI_WARPS);
         }
         mbar_fence_init();
     }
@@ -385,11 +400,14 @@ umma_grouped_pair_kernel(const GroupProb *__restrict__ probs,
         // ------------------------------------------ producer (both CTAs)
         bool ok = true;
         unsigned g = 0, issued_from = 0;
-        for (int it = cl; it < nitems && ok; it += ncl) {
+        for (int r = 0; r * ncl < nitems && ok; ++r) {
+            const int it = group_item_index(r, cl, ncl);
+            if (it >= nitems) break;
             const uint2 w = items[it];
             const GroupProb *gp = probs + w.x;
             const int m0 = (int)(w.y & 0xffffu) * 2 * S::BM + (int)rank * S::BM;
-            const int nb = (int)(w.y >> 16) * GP_BN + (int)rank * S::BNH;
+            const int n0 = (int)(w.y >> 16) * gp->bw;
+            const int nb = n0 + (int)rank * (group_item_columns(gp, n0) / 2);
             const int KB = (gp->K + S::BK - 1) / S::BK;
             for (int kb = 0; kb < KB; ++kb, ++g) {
                 const int s = (int)(g % STAGES);
@@ -430,14 +448,12 @@ umma_grouped_pair_kernel(const GroupProb *__restrict__ probs,
         }
     } else if (warp == 1 && rank == 0) {
         // ---------------------------------------- MMA issuer (even CTA)
-        const uint32_t idesc = umma::idesc_f16(2 * S::BM, GP_BN, false);
         unsigned g = 0;
-        int n = 0;
         bool ok = true;
-        for (int it = cl; it < nitems && ok; it += ncl, ++n) {
-            const int b = n & 1;
-            if (!mbar_wait_bounded(&acc_empty[b],
-                                             (uint32_t)(((n >> 1) & 1) ^ 1))) {
+        for (int n = 0; n * ncl < nitems && ok; ++n) {
+            const int it = group_item_index(n, cl, ncl), b = n % NBUF;
+            if (it >= nitems) break;
+            if (!mbar_wait_bounded(&acc_empty[b], (uint32_t)(((n / NBUF) & 1) ^ 1))) {
                 abort_flag = 1;
                 set_status(status, DEV_TIMEOUT);
             }
@@ -445,7 +461,10 @@ umma_grouped_pair_kernel(const GroupProb *__restrict__ probs,
             if (!ok) break;
             umma::fence_after_sync();
             const uint32_t d0 = tmem + (uint32_t)b * ACC_COLS, d1 = d0 + GP_BN;
-            const GroupProb *gp = probs + items[it].x;
+            const uint2 w = items[it];
+            const GroupProb *gp = probs + w.x;
+            const uint32_t idesc = umma::idesc_f16(
+                2 * S::BM, group_item_columns(gp, (int)(w.y >> 16) * gp->bw), false);
             const int KB = (gp->K + S::BK - 1) / S::BK;
             for (int kb = 0; kb < KB; ++kb, ++g) {
                 const int s = (int)(g % STAGES);
@@ -486,12 +505,12 @@ umma_grouped_pair_kernel(const GroupProb *__restrict__ probs,
         // --------------------------------------- epilogue (both CTAs)
         const int q = warp & 3;
         const uint32_t lead_empty0 = umma2::map_to_rank(&acc_empty[0], 0);
-        int n = 0;
-        for (int it = cl; it < nitems; it += ncl, ++n) {
-            const int b = n & 1;
+        for (int n = 0; n * ncl < nitems; ++n) {
+            const int it = group_item_index(n, cl, ncl), b = n % NBUF;
+            if (it >= nitems) break;
             const bool ok = __all_sync(
                 0xffffffffu,
-                mbar_wait_bounded(&acc_full[b], (uint32_t)((n >> 1) & 1)));
+                mbar_wait_bounded(&acc_full[b], (uint32_t)((n / NBUF) & 1)));
             umma::fence_after_sync();
             if (!ok || abort_flag) {
                 if (!ok) set_status(status, DEV_TIMEOUT);
@@ -500,7 +519,7 @@ umma_grouped_pair_kernel(const GroupProb *__restrict__ probs,
             const uint2 w = items[it];
             const GroupProb *gp = probs + w.x;
             const int m0 = (int)(w.y & 0xffffu) * 2 * S::BM + (int)rank * S::BM;
-            const int n0 = (int)(w.y >> 16) * GP_BN;
+            const int n0 = (int)(w.y >> 16) * gp->bw, cols = group_item_columns(gp, n0);
             const int row = m0 + q * 32 + lane;
             const int M = gp->M, Ncols = gp->N;
             const long long ldd = gp->ldd;
@@ -509,8 +528,9 @@ umma_grouped_pair_kernel(const GroupProb *__restrict__ probs,
             const int vec = store_width(gp->D, ldd);
             const uint32_t t_row =
                 tmem + (uint32_t)b * ACC_COLS + ((uint32_t)(q * 32) << 16);
+            // (the two warps of a quarter take every other 32 columns)
 #pragma unroll 1
-            for (int c = 0; c < GP_BN; c += 32) {
+            for (int c = (warp - 2) / 4 * 32; c < cols; c += 64) {
                 uint32_t r[32], r2[32];
                 umma::tmem_ld32(t_row + c, r);
                 umma::tmem_ld32(t_row + GP_BN + c, r2);
@@ -568,13 +588,11 @@ cudaError_t launch_umma_grouped_pair(const GroupProb *probs, const uint2 *items,
     using S = PairShape<GP_BN, true, GP_STAGES>;
     if (nitems <= 0) return cudaSuccess;
     const int clusters = nitems < sm_count / 2 ? nitems : sm_count / 2;
-    umma_grouped_pair_kernel<GP_STAGES><<<2 * (clusters > 0 ? clusters : 1), 192,
+    umma_grouped_pair_kernel<GP_STAGES><<<2 * (clusters > 0 ? clusters : 1), GP_THREADS,
                                           S::RING, s>>>(probs, items, nitems, status);
     return cudaGetLastError();
 }
 
-int group_pair_tile_m() { return 2 * 128; }
 int group_pair_tile_n() { return GP_BN; }
-int group_pair_box_b() { return GP_BN / 2; }
 
 }  // namespace cgh
