@@ -334,7 +334,7 @@ cudaError_t launch_umma_gemm(const GemmOperands &op, unsigned *status,
 // separable.cu: U / V tables of the separable form, the point records
 // built inside the kernel from the caller's points.
 cudaError_t launch_sep_tables(const PointSource &src, int Npad, int Nx, int Ny, int Kp,
-                              int kind, void *Lhi, void *Llo, void *Rhi, void *Rlo,
+                              int kind, int sms, void *Lhi, void *Llo, void *Rhi, void *Rlo,
                               cudaStream_t s);
 
 }  // namespace cgh

@@ -34,19 +34,19 @@
 
 namespace cgh {
 
-// Grid: x over blocks of ST_POINTS points, y over runs of ST_BLOCK_ROWS
+// Grid: x over blocks of ST_POINTS points, y over ST_RUNS runs of run_rows
 // consecutive table rows (x rows, then y rows).  The block first builds the
 // records of its points in shared memory (step A1 in FP64, as prologue.cu;
 // each record is built once per row block, which costs less than a
 // separate prologue launch in the chain), then each warp writes one run of
-// ST_ROWS rows for 32 point pairs (sep_table_rows): a warp's stores are
+// run_rows rows for 32 point pairs (sep_table_rows): a warp's stores are
 // contiguous 256-byte pieces of a table row.
 constexpr int ST_POINTS = 64;
-constexpr int ST_BLOCK_ROWS = 8 * ST_ROWS;
+constexpr int ST_RUNS = 8;  // runs per block
 
 template <int KIND>
 __global__ void __launch_bounds__(256)
-sep_tables_kernel(PointSource src, int Npad, int Nx, int Ny, int Kp,
+sep_tables_kernel(PointSource src, int Npad, int Nx, int Ny, int Kp, int run_rows,
                   void *__restrict__ Lhi, void *__restrict__ Llo,
                   void *__restrict__ Rhi, void *__restrict__ Rlo) {
     __shared__ PointRec srec[ST_POINTS];
@@ -61,29 +61,34 @@ sep_tables_kernel(PointSource src, int Npad, int Nx, int Ny, int Kp,
     const int pair = threadIdx.x & 31, run = threadIdx.x >> 5;
     const int jj = j0 + 2 * pair;  // even; Npad is even, so jj + 1 < Npad too
     if (jj >= Npad) return;
-    const int r0 = blockIdx.y * ST_BLOCK_ROWS + run * ST_ROWS;
+    const int r0 = (blockIdx.y * ST_RUNS + run) * run_rows;
     const int rows = Nx + Ny;
     if (r0 >= rows) return;
-    const int r1 = r0 + ST_ROWS < rows ? r0 + ST_ROWS : rows;
+    const int r1 = r0 + run_rows < rows ? r0 + run_rows : rows;
     const bool v0 = jj < src.N, v1 = jj + 1 < src.N;
     sep_table_rows<KIND>(srec[2 * pair], srec[2 * pair + 1], v0, v1, Nx, Kp, jj, r0,
                          r1, Lhi, Llo, Rhi, Rlo);
 }
 
 cudaError_t launch_sep_tables(const PointSource &src, int Npad, int Nx, int Ny, int Kp,
-                              int kind, void *Lhi, void *Llo, void *Rhi, void *Rlo,
-                              cudaStream_t s) {
-    const int rows = Nx + Ny;  // <= 65536: grid y stays below its limit
-    dim3 grid((Npad + ST_POINTS - 1) / ST_POINTS, (rows + ST_BLOCK_ROWS - 1) / ST_BLOCK_ROWS);
+                              int kind, int sms, void *Lhi, void *Llo, void *Rhi,
+                              void *Rlo, cudaStream_t s) {
+    // Rows per run: ST_ROWS, or with one plane up to 64 while that leaves 16
+    // blocks per SM.  Each run evaluates its first phases, and each block its
+    // records, anew: 3840x2160x16384 in BF16 74 us with runs of 16, 62 of 32,
+    // 59 of 64 (writing 393 MB).  Two planes are bound by their stores (107 us
+    // with 16, 110 with 64).
+    const int rows = Nx + Ny, bx = (Npad + ST_POINTS - 1) / ST_POINTS;  // rows <= 65536
+    int run = ST_ROWS;
+    while (kind != 2 && run < 64 &&
+           (long long)bx * ((rows + 2 * run * ST_RUNS - 1) / (2 * run * ST_RUNS)) >= 16LL * sms)
+        run *= 2;
+    const dim3 grid(bx, (rows + run * ST_RUNS - 1) / (run * ST_RUNS));
     // (builds the records itself: the call's first kernel, an ordinary launch)
-    if (kind == 0)
-        return launch_kernel(false, sep_tables_kernel<0>, grid, dim3(256), 0, s, src, Npad,
-                             Nx, Ny, Kp, Lhi, Llo, Rhi, Rlo);
-    if (kind == 1)
-        return launch_kernel(false, sep_tables_kernel<1>, grid, dim3(256), 0, s, src, Npad,
-                             Nx, Ny, Kp, Lhi, Llo, Rhi, Rlo);
-    return launch_kernel(false, sep_tables_kernel<2>, grid, dim3(256), 0, s, src, Npad, Nx,
-                         Ny, Kp, Lhi, Llo, Rhi, Rlo);
+    auto kern = kind == 0 ? sep_tables_kernel<0> : kind == 1 ? sep_tables_kernel<1>
+                                                             : sep_tables_kernel<2>;
+    return launch_kernel(false, kern, grid, dim3(32 * ST_RUNS), 0, s, src, Npad, Nx, Ny, Kp, run,
+                         Lhi, Llo, Rhi, Rlo);
 }
 
 }  // namespace cgh
@@ -154,7 +159,7 @@ cgh_status cgh_ctx::forward_separable(const float *points, const float *A,
         TimedLaunch tl(this, CGH_K_SEP_TABLES, s);
         cudaError_t e = launch_sep_tables(
             PointSource{points, A, z, N, fresnel_scale(lambda, p), d_status, row_origin}, Npad, Nx, Ny,
-            Kp, kind, Lhi, Llo, Rhi, Rlo, s);
+            Kp, kind, sm_count, Lhi, Llo, Rhi, Rlo, s);
         if (e != cudaSuccess) return cuda_fail(e, "separable tables launch");
         tl.done();
     }
