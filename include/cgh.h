@@ -387,6 +387,8 @@ cgh_status cgh_set_gemm_tiles(cgh_handle h, int tiles);
  * Widths: 112 or 128 for CGH_GEMM_SINGLE; 112, 144, 160, 224 or 256 for
  * CGH_GEMM_PAIRS and CGH_GEMM_PAIRS_GEN (the single-pass generating kernel
  * has 112 and 256 only: other widths fall back to its heuristic there);
+ * CGH_GEMM_PAIRS narrows its tiles, at the same number of waves, to equal
+ * shares of the columns;
  * width 0: the heuristic's width for the tiling.
  * CGH_ERR_UNSUPPORTED for a plan not compiled in, CGH_ERR_INVALID_ARG for a
  * null handle. */

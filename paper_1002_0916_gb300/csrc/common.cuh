@@ -327,7 +327,7 @@ int pick_gen_n(int M, int N, int sms, int kind);
 cudaError_t launch_umma_gen(const PointRec *rec, int N, int Npad, int kind, int bnp,
                             float *D, int M, int Ncols, long long ldd, float lo_scale,
                             unsigned *status, cudaStream_t s);
-cudaError_t launch_umma_pair(const GemmOperands &op, int bnp, unsigned *status,
+cudaError_t launch_umma_pair(const GemmOperands &op, int bnp, unsigned *status, int sms,
                              cudaStream_t s);
 cudaError_t launch_umma_gemm(const GemmOperands &op, unsigned *status,
                              cudaStream_t s);

@@ -370,9 +370,10 @@ cudaError_t launch_umma_gemm(const GemmOperands &op, unsigned *status,
         }
         return cudaSuccess;
     }
-    const GemmPlan plan = gemm_plan(op.M, op.N, op.tiles, sm_count_of_current_device(),
-                                    op.bf16 ? 0 : op.split ? 2 : 1, op.bn);
-    if (plan.tiling == CGH_GEMM_PAIRS) return launch_umma_pair(op, plan.bn, status, s);
+    const int sms = sm_count_of_current_device();
+    const GemmPlan plan = gemm_plan(op.M, op.N, op.tiles, sms, op.bf16 ? 0 : op.split ? 2 : 1,
+                                    op.bn);
+    if (plan.tiling == CGH_GEMM_PAIRS) return launch_umma_pair(op, plan.bn, status, sms, s);
     const int bn = plan.bn;
     if (op.split)
         return bn == 112 ? launch_gemm_t<112, true, 3>(op, status, s)

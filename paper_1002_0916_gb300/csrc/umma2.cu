@@ -25,6 +25,8 @@
 #include <cudaTypedefs.h>
 #include <stdlib.h>
 
+#include <type_traits>
+
 #include "api_internal.h"
 #include "common.cuh"
 #include "umma.cuh"
@@ -33,8 +35,8 @@
 
 namespace cgh {
 
-// Grid: x = 2 x (column blocks of BNP), y = row blocks of 256; clusters of
-// two CTAs along x.
+// Grid: x = 2 x (column blocks of bw <= BNP), y = row blocks of 256; clusters
+// of two CTAs along x.
 // Eight epilogue warps: the epilogue is latency (tensor-memory loads, then
 // stores), 2.9 us at 112 columns with four.
 constexpr int PAIR_THREADS = 64 + 32 * 8;
@@ -44,7 +46,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PAIR_THREADS, 1)
 umma_pair_kernel(const __grid_constant__ CUtensorMap tA,
                  const __grid_constant__ CUtensorMap tB,
                  const __grid_constant__ CUtensorMap tA2,
-                 const __grid_constant__ CUtensorMap tB2, GemmArgs g,
+                 const __grid_constant__ CUtensorMap tB2, GemmArgs g, int bw,
                  uint32_t idesc) {
     using S = PairShape<BNP, SPLIT, STAGES>;
     extern __shared__ uint8_t smem_raw[];
@@ -58,8 +60,8 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tA,
     const uint32_t rank = umma2::cluster_rank();
     const int warp = umma::warp_index(), lane = threadIdx.x & 31;
     const int m0 = blockIdx.y * 2 * S::BM + (int)rank * S::BM;  // this CTA's rows
-    const int np0 = (blockIdx.x >> 1) * BNP;                     // the pair's columns
-    const int nb = np0 + (int)rank * S::BNH;                     // this CTA's B rows
+    const int np0 = (blockIdx.x >> 1) * bw;                     // the pair's columns
+    const int nb = np0 + (int)rank * (bw / 2);                  // this CTA's B rows
     const int KB = (g.K + S::BK - 1) / S::BK;
 
     if (threadIdx.x == 0) {
@@ -91,6 +93,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tA,
         // ------------------------------------------ producer (both CTAs)
         bool ok = true;
         int issued = 0;
+        const uint32_t bytes = (SPLIT ? 4 : 2) * (S::A_BYTES + (uint32_t)bw * S::BK);
         for (int kb = 0; kb < KB; ++kb) {
             const int s = kb % STAGES;
             if (kb >= STAGES &&
@@ -104,7 +107,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tA,
             const uint32_t bar = umma2::map_to_rank(&full[s], 0);
             if (umma::elect_one()) {
                 // the even CTA's barrier counts the bytes of both CTAs' loads
-                if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * S::STAGE_BYTES);
+                if (rank == 0) mbar_arrive_expect_tx(&full[s], bytes);
                 umma2::tma_load_2d_pair(st, &tA, kb * S::BK, m0, bar);
                 umma2::tma_load_2d_pair(st + S::A_BYTES, &tB, kb * S::BK, nb, bar);
                 if (SPLIT) {
@@ -189,10 +192,9 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tA,
             const int vec = store_width(g.D, g.ldd);
             float *stage = reinterpret_cast<float *>(smem + (size_t)STAGES * S::STAGE_BYTES) +
                            (warp - 2) * EPI_WARP_FLOATS;
-            constexpr int CH = S::CH;
-            // the two warps of a quarter take every other chunk of columns
-#pragma unroll 1
-            for (int c = ((warp - 2) >> 2) * CH; c < BNP; c += 2 * CH) {
+            // CH columns from c on
+            auto chunk = [&](auto width, int c) {
+                constexpr int CH = decltype(width)::value;
                 uint32_t r[CH];
                 float v[CH];
                 if constexpr (CH == 32) umma::tmem_ld32(t_row + c, r);
@@ -220,6 +222,12 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tA,
                                            g.M - (row - lane), np0 + c + i, g.N, g.accumulate,
                                            lane);
                 }
+            };
+            // the two warps of a quarter take every other chunk of columns
+#pragma unroll 1
+            for (int c = ((warp - 2) >> 2) * S::CH; c < bw; c += 2 * S::CH) {
+                if (S::CH == 16 || c + S::CH <= bw) chunk(std::integral_constant<int, S::CH>{}, c);
+                else chunk(std::integral_constant<int, 16>{}, c);
             }
         }
     }
@@ -235,18 +243,33 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tA,
 bool make_gemm_map(CUtensorMap *m, const void *base, long long inner, long long rows,
                    long long ld, int box_rows, bool bf16);
 
+// The columns of a tile of the plan's width bnp: as many tiles as fit in the
+// same number of waves of SM pairs, equal whole sixteens.  Holograms before and
+// after: 1920x1080x4096 split FP16, 15 tiles of 128 instead of 14 of 144, 80.9
+// -> 76.6 us; 3840x2160x16384 BF16, 16 of 240 instead of 15 of 256 in two
+// waves, 359 -> 346; 1366x768x777, 22 of 64 instead of 13 of 112, 19.9 -> 16.8;
+// 256x256x4000, 8 of 32 instead of 3 of 112, 51.7 -> 39.9.
+static int pair_columns(int M, int N, int bnp, int sms) {
+    const int rows = (M + 255) / 256, tiles = (N + bnp - 1) / bnp;
+    const int pairs = sms / 2 > 0 ? sms / 2 : 1;
+    const int most = (rows * tiles + pairs - 1) / pairs * pairs / rows;  // >= tiles
+    const int bw = pad_to((N + most - 1) / most, 16);
+    return bw < 32 ? 32 : bw < bnp ? bw : bnp;
+}
+
 template <int BNP, bool SPLIT, int STAGES>
 static cudaError_t launch_pair_t(const GemmOperands &op, unsigned *status,
-                                 cudaStream_t s) {
+                                 int sms, cudaStream_t s) {
     using S = PairShape<BNP, SPLIT, STAGES>;
     static_assert(S::SMEM <= 232448 - 1024, "shared memory");
+    const int bw = pair_columns(op.M, op.N, BNP, sms);
     CUtensorMap tA, tB, tA2, tB2;
     if (!make_gemm_map(&tA, op.A_hi, op.K, op.M, op.lda, S::BM, op.bf16) ||
-        !make_gemm_map(&tB, op.B_hi, op.K, op.N, op.ldb, S::BNH, op.bf16))
+        !make_gemm_map(&tB, op.B_hi, op.K, op.N, op.ldb, bw / 2, op.bf16))
         return cudaErrorInvalidValue;
     if (SPLIT) {
         if (!make_gemm_map(&tA2, op.A_lo, op.K, op.M, op.lda, S::BM, op.bf16) ||
-            !make_gemm_map(&tB2, op.B_lo, op.K, op.N, op.ldb, S::BNH, op.bf16))
+            !make_gemm_map(&tB2, op.B_lo, op.K, op.N, op.ldb, bw / 2, op.bf16))
             return cudaErrorInvalidValue;
     } else {
         tA2 = tA;
@@ -263,9 +286,9 @@ static cudaError_t launch_pair_t(const GemmOperands &op, unsigned *status,
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
     }
     GemmArgs g{op.M, op.N, op.K, op.D, op.ldd, op.lo_scale, status, op.accumulate};
-    dim3 grid(2 * ((op.N + BNP - 1) / BNP), (op.M + 2 * S::BM - 1) / (2 * S::BM));
-    const uint32_t idesc = umma::idesc_f16(2 * S::BM, BNP, op.bf16);
-    return launch_dependent(kern, grid, dim3(PAIR_THREADS), S::SMEM, s, tA, tB, tA2, tB2, g,
+    dim3 grid(2 * ((op.N + bw - 1) / bw), (op.M + 2 * S::BM - 1) / (2 * S::BM));
+    const uint32_t idesc = umma::idesc_f16(2 * S::BM, bw, op.bf16);
+    return launch_dependent(kern, grid, dim3(PAIR_THREADS), S::SMEM, s, tA, tB, tA2, tB2, g, bw,
                             idesc);
 }
 
@@ -301,7 +324,7 @@ int pick_pair_n(int M, int N, int sms, double *cost) {
 
 // Stages: as many as fit in shared memory (the loads' latency is hidden by
 // the bytes in flight).
-cudaError_t launch_umma_pair(const GemmOperands &op, int bnp, unsigned *status,
+cudaError_t launch_umma_pair(const GemmOperands &op, int bnp, unsigned *status, int sms,
                              cudaStream_t s) {
     static const int forced = [] {
         const char *f = getenv("CGH_PAIR_BN");
@@ -310,19 +333,19 @@ cudaError_t launch_umma_pair(const GemmOperands &op, int bnp, unsigned *status,
     if (forced) bnp = forced;
     if (op.split) {
         switch (bnp) {
-        case 112: return launch_pair_t<112, true, 4>(op, status, s);
-        case 144: return launch_pair_t<144, true, 4>(op, status, s);
-        case 160: return launch_pair_t<160, true, 4>(op, status, s);
-        case 224: return launch_pair_t<224, true, 3>(op, status, s);
-        case 256: return launch_pair_t<256, true, 3>(op, status, s);
+        case 112: return launch_pair_t<112, true, 4>(op, status, sms, s);
+        case 144: return launch_pair_t<144, true, 4>(op, status, sms, s);
+        case 160: return launch_pair_t<160, true, 4>(op, status, sms, s);
+        case 224: return launch_pair_t<224, true, 3>(op, status, sms, s);
+        case 256: return launch_pair_t<256, true, 3>(op, status, sms, s);
         }
     } else {
         switch (bnp) {
-        case 112: return launch_pair_t<112, false, 9>(op, status, s);
-        case 144: return launch_pair_t<144, false, 8>(op, status, s);
-        case 160: return launch_pair_t<160, false, 8>(op, status, s);
-        case 224: return launch_pair_t<224, false, 6>(op, status, s);
-        case 256: return launch_pair_t<256, false, 6>(op, status, s);
+        case 112: return launch_pair_t<112, false, 9>(op, status, sms, s);
+        case 144: return launch_pair_t<144, false, 8>(op, status, sms, s);
+        case 160: return launch_pair_t<160, false, 8>(op, status, sms, s);
+        case 224: return launch_pair_t<224, false, 6>(op, status, sms, s);
+        case 256: return launch_pair_t<256, false, 6>(op, status, sms, s);
         }
     }
     return cudaErrorInvalidValue;
