@@ -10,9 +10,9 @@
 //   warp 0      TMA producer: 2-D tiled loads (128-byte swizzle) of the
 //               K-blocks of A and B into a STAGES-deep shared-memory ring,
 //               completing on `full` mbarriers;
-//   warp 1      allocates TMEM; its lane 0 issues the MMAs (4 per 64-wide
-//               K-block per product) and releases ring slots through
-//               tcgen05.commit -> `empty` mbarriers;
+//   warp 1      allocates TMEM; an elected lane issues the MMAs (4 per
+//               64-wide K-block per product) and releases ring slots
+//               through tcgen05.commit -> `empty` mbarriers;
 //   warps 2..5  epilogue: tcgen05.ld of the accumulator(s), combine, store.
 // The split form keeps two accumulators (hi*hi and the two cross terms),
 // so the lo planes can be stored pre-scaled by 2^12 and stay normal FP16
