@@ -7,7 +7,7 @@
 //     dL/dy_j = 2 P_j A_j sum G sin(phi) dy
 //     dL/dz_j = (P_j A_j / z_j) sum G sin(phi) (dx^2 + dy^2)
 // The direct method is here: FP32 point-owned sums.  Each thread owns one
-// point and walks a 16-pixel-wide column strip of G over a run of rows; the
+// point and walks a 16- or 32-pixel-wide column strip of G over a run of rows; the
 // cosines and sines of the strip's columns stay in registers, the row angle
 // follows the exact fixed-point form of the paper's Eq. 2 recurrence, and the
 // cosine and sine of each summed phase are expanded by angle addition.  One
@@ -31,60 +31,72 @@ namespace cgh {
 //     sum_x G sin(phi) = cy P + sy Q,
 //     P = sum_x G sx,   Q = sum_x G cx           (per row, across the strip)
 // Per update: 4 FP32 multiply-adds (U, V, P, Q), packed in column pairs; the
-// row's hardware sincos is shared by 16 updates, the columns' (to FP32
+// row's hardware sincos is shared by the strip's updates, the columns' (to FP32
 // rounding) by a whole run of rows.  The offset dx is constant down a column,
 // so the x sums are taken from the columns' sums once at the end.
 //
 // Bound: the FMA pipe, 128 / 4 = 32 updates per clock and SM.  A sincos per
 // update, a quarter of them as polynomials, was bound by the MUFU instead:
-// 2954 us at 1920x1080x4096 against 1446 here (0.58 of the bound; the pipe is
-// 68% busy, a packed multiply-add holding it two cycles, and a row costs 28
-// instructions beside its 32).  Two rows unrolled: 1447 against 1522; split P
-// and Q chains, 3 or 5 CTAs per SM, 64- or 256-thread CTAs: 0 to 6% slower.
-constexpr int BWD_STRIP = 16;            // pixels per column strip
-constexpr int BWD_NP2 = BWD_STRIP / 2;
-constexpr int BWD_THREADS = 128;         // points per CTA
-constexpr int BWD_CTAS = 4;              // per SM (at most 128 registers)
-// rows of the strip per shared-memory stage (two stages): the CTA's threads
-// load the next stage into registers, any alignment and width, before they
-// compute on this one
-constexpr int BWD_RB = 32;
-constexpr int BWD_LOADS = BWD_RB * BWD_STRIP / BWD_THREADS;
+// 2954 us at 1920x1080x4096 against 1273 here (0.66 of the bound; a packed
+// multiply-add holds the pipe two cycles, and a row costs 28 instructions
+// beside its 64).  24 columns with 96 threads: 1775; two rows unrolled at 32
+// columns: 1310; stages of 8, 12, 24 or 32 rows there: 1290 to 1330; split P
+// and Q chains or the columns' phases stepped instead of evaluated: 1330.
+// 16 columns, four CTAs per SM and two rows unrolled: 1446 us there, but less
+// set-up per CTA: 8.2 us against 9.8 at 256x256x64, 29 both at 1023x767x100.
+template <int STRIP>
+struct BwdShape {
+    static constexpr int NP2 = STRIP / 2;
+    static constexpr int CTAS = STRIP == 32 ? 3 : 4;  // per SM (168 or 128 registers)
+    // rows of the strip per shared-memory stage (two stages): the CTA's
+    // threads load the next stage into registers, any alignment and width,
+    // before they compute on this one
+    static constexpr int RB = STRIP == 32 ? 16 : 32;
+    static constexpr int UNROLL = STRIP == 32 ? 1 : 2;  // rows
+};
+constexpr int BWD_THREADS = 128;  // points per CTA
+// Strips of 32 columns from 2^25 updates on.
+static int bwd_strip(int Nx, int Ny, int N) {
+    return (double)Nx * Ny * N < (double)(1 << 25) ? 16 : 32;
+}
 
 // Grid: x = column strips, y = groups of BWD_THREADS points, z = runs of
 // `rows` rows.  part: [strip * runs + run][5][Npad], the sums of G cos, G sin
 // dx, G sin dx^2, G sin dy, G sin dy^2.
-__global__ void __launch_bounds__(BWD_THREADS, BWD_CTAS)
+template <int STRIP>
+__global__ void __launch_bounds__(BWD_THREADS, BwdShape<STRIP>::CTAS)
 direct_bwd_kernel(PointSource src, int Npad, int Nx, int Ny, int rows,
                   const float *__restrict__ G, float *__restrict__ part) {
-    __shared__ __align__(16) float sg[2][BWD_RB][BWD_STRIP];
-    const int strip = blockIdx.x, x0 = strip * BWD_STRIP;
+    constexpr int NP2 = BwdShape<STRIP>::NP2, RB = BwdShape<STRIP>::RB;
+    constexpr int LOADS = RB * STRIP / BWD_THREADS, UNROLL = BwdShape<STRIP>::UNROLL;
+    __shared__ __align__(16) float sg[2][RB][STRIP];
+    const int strip = blockIdx.x, x0 = strip * STRIP;
     const int j = blockIdx.y * BWD_THREADS + threadIdx.x;
     const int ya = blockIdx.z * rows, yb = ya + rows < Ny ? ya + rows : Ny;
-    const int lc = threadIdx.x % BWD_STRIP, lr = threadIdx.x / BWD_STRIP;
+    const int lc = threadIdx.x % STRIP, lr = threadIdx.x / STRIP;
     const float *gcol = G + x0 + lc;
     const bool in_x = x0 + lc < Nx;
-    float next[BWD_LOADS];
+    float next[LOADS];
     auto load = [&](int y0) {
 #pragma unroll
-        for (int k = 0; k < BWD_LOADS; ++k) {
-            const int y = y0 + lr + k * (BWD_THREADS / BWD_STRIP);
+        for (int k = 0; k < LOADS; ++k) {
+            const int y = y0 + lr + k * (BWD_THREADS / STRIP);
             next[k] = in_x && y < yb ? __ldg(gcol + (size_t)y * Nx) : 0.0f;
         }
     };
     auto store = [&](int b) {
 #pragma unroll
-        for (int k = 0; k < BWD_LOADS; ++k)
-            sg[b][lr + k * (BWD_THREADS / BWD_STRIP)][lc] = next[k];
+        for (int k = 0; k < LOADS; ++k)
+            sg[b][lr + k * (BWD_THREADS / STRIP)][lc] = next[k];
     };
     load(ya);
 
     // the point's record (a rejected point reports once per CTA column)
     const PointRec pr = make_point_rec(src.points, src.A, src.z, src.N, j, src.K, src.status);
     const float2 z2 = make_float2(0.0f, 0.0f);
-    float2 cx[BWD_NP2], sx[BWD_NP2], U[BWD_NP2], V[BWD_NP2];
+    float2 cx[NP2], sx[NP2], U[NP2], V[NP2];
 #pragma unroll
-    for (int k = 0; k < BWD_NP2; ++k) {
+    for (int k = 0; k < NP2; ++k) {
         sincos_fixed(axis_phase(pr.c, pr.bx, pr.ax, x0 + 2 * k), sx[k].x, cx[k].x);
         sincos_fixed(axis_phase(pr.c, pr.bx, pr.ax, x0 + 2 * k + 1), sx[k].y, cx[k].y);
         U[k] = V[k] = z2;
@@ -99,11 +111,11 @@ direct_bwd_kernel(PointSource src, int Npad, int Nx, int Ny, int rows,
     store(0);
     __syncthreads();
     int b = 0;
-    for (int y0 = ya; y0 < yb; y0 += BWD_RB, b ^= 1) {
-        const bool more = y0 + BWD_RB < yb;
-        if (more) load(y0 + BWD_RB);
-        const int n = yb - y0 < BWD_RB ? yb - y0 : BWD_RB;
-#pragma unroll 2
+    for (int y0 = ya; y0 < yb; y0 += RB, b ^= 1) {
+        const bool more = y0 + RB < yb;
+        if (more) load(y0 + RB);
+        const int n = yb - y0 < RB ? yb - y0 : RB;
+#pragma unroll UNROLL
         for (int r = 0; r < n; ++r) {
             float sy, cy;
             __sincosf((float)phase_hi(th) * RAD_PER_U32, &sy, &cy);
@@ -113,7 +125,7 @@ direct_bwd_kernel(PointSource src, int Npad, int Nx, int Ny, int rows,
             const float4 *row = reinterpret_cast<const float4 *>(&sg[b][r][0]);
             float2 p = z2, q = z2;
 #pragma unroll
-            for (int k = 0; k < BWD_NP2; k += 2) {
+            for (int k = 0; k < NP2; k += 2) {
                 const float4 v = row[k >> 1];
                 const float2 g[2] = {make_float2(v.x, v.y), make_float2(v.z, v.w)};
 #pragma unroll
@@ -136,7 +148,7 @@ direct_bwd_kernel(PointSource src, int Npad, int Nx, int Ny, int rows,
     const float xj = src.points[2 * j];
     float C = 0.0f, sX = 0.0f, sXX = 0.0f;
 #pragma unroll
-    for (int k = 0; k < BWD_NP2; ++k) {
+    for (int k = 0; k < NP2; ++k) {
         C += fmaf(cx[k].x, U[k].x, -sx[k].x * V[k].x) + fmaf(cx[k].y, U[k].y, -sx[k].y * V[k].y);
         const float dx0 = (float)(x0 + 2 * k) - xj, dx1 = (float)(x0 + 2 * k + 1) - xj;
         const float t0 = fmaf(sx[k].x, U[k].x, cx[k].x * V[k].x) * dx0;
@@ -231,14 +243,16 @@ cudaError_t launch_adjoint_sum(const PointSource &src, const AdjointParts &pp, c
 
 // Rows per run: the fewest runs (each repeats the columns' sincos, worth
 // about 16 rows) whose CTAs fill the SMs' slots in nearly whole waves.
-static int bwd_rows(int Nx, int Ny, int N, int sms) {
-    const long long ctas = (long long)((Nx + BWD_STRIP - 1) / BWD_STRIP) *
+static int bwd_rows(int strip, int Nx, int Ny, int N, int sms) {
+    const int rb = strip == 32 ? BwdShape<32>::RB : BwdShape<16>::RB;
+    const int per_sm = strip == 32 ? BwdShape<32>::CTAS : BwdShape<16>::CTAS;
+    const long long ctas = (long long)((Nx + strip - 1) / strip) *
                            ((N + BWD_THREADS - 1) / BWD_THREADS);
-    const long long slots = (long long)BWD_CTAS * (sms > 0 ? sms : 1);
+    const long long slots = (long long)per_sm * (sms > 0 ? sms : 1);
     int best = Ny;
     double best_cost = 1e300;
     for (int runs = 1; runs <= 16; ++runs) {
-        const int rows = pad_to((Ny + runs - 1) / runs, BWD_RB);
+        const int rows = pad_to((Ny + runs - 1) / runs, rb);
         const long long n = (Ny + rows - 1) / rows;
         const double cost = (double)((ctas * n + slots - 1) / slots) * (rows + 16);
         if (cost < best_cost * 0.99) {
@@ -258,8 +272,8 @@ static cgh_status run_direct_backward(cgh_ctx *h, const float *points, const flo
                                       int Ny, const float *G, float *gpts, float *gA, float *gz,
                                       cudaStream_t s) {
     const int Npad = pad_to(N, 32);
-    const int strips = (Nx + BWD_STRIP - 1) / BWD_STRIP;
-    const int rows = bwd_rows(Nx, Ny, N, h->sm_count), runs = (Ny + rows - 1) / rows;
+    const int strip = bwd_strip(Nx, Ny, N), strips = (Nx + strip - 1) / strip;
+    const int rows = bwd_rows(strip, Nx, Ny, N, h->sm_count), runs = (Ny + rows - 1) / rows;
     const size_t part_b = (size_t)strips * runs * 5 * Npad * sizeof(float);
     cgh_status st = h->ensure(h->ws2, part_b, s, "adjoint workspace");
     if (st) return st;
@@ -268,8 +282,9 @@ static cgh_status run_direct_backward(cgh_ctx *h, const float *points, const flo
     {
         TimedLaunch tl(h, CGH_K_BWD_DIRECT, s);
         const dim3 grid(strips, (N + BWD_THREADS - 1) / BWD_THREADS, runs);
-        cudaError_t e = launch_kernel(false, direct_bwd_kernel, grid, dim3(BWD_THREADS), 0, s,
-                                      src, Npad, Nx, Ny, rows, G, part);
+        cudaError_t e = launch_kernel(
+            false, strip == 32 ? direct_bwd_kernel<32> : direct_bwd_kernel<16>, grid,
+            dim3(BWD_THREADS), 0, s, src, Npad, Nx, Ny, rows, G, part);
         if (e != cudaSuccess) return h->cuda_fail(e, "direct adjoint launch");
         tl.done();
     }

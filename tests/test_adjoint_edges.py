@@ -53,7 +53,9 @@ def _reference(c, G):
 @pytest.mark.parametrize("method", ["sep_fp32", "direct"])
 @pytest.mark.parametrize("Nx,Ny,N", [
     (1, 1, 1), (1, 300, 5), (300, 1, 129), (17, 33, 127), (257, 225, 128), (64, 1100, 130),
-    (515, 66, 257), (449, 193, 33), (32768, 3, 4300)])
+    (515, 66, 257), (449, 193, 33), (32768, 3, 4300),
+    # strips of 32 columns of the direct adjoint (2^25 updates on)
+    (31, 1111, 1000), (33, 1025, 1001), (96, 399, 900)])
 def test_edges(cg, method, Nx, Ny, N):
     import torch
     c = make_cloud(3 + Nx + N, N, Nx, Ny, integer=bool(N & 1), zlo=0.2, zhi=0.9, lam=532e-9,
