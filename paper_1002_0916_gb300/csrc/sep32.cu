@@ -36,9 +36,11 @@
 // arrivals relaxed: tensor memory is ordered by the tcgen05 fences, and no
 // generic memory is handed over).
 // Measured, whole call, against an FP32 product on the FMA pipe (0.70 of its
-// bound): 1920x1024x3584 543 -> 73 us, 3840x2160x16384 9.85 -> 1.07 ms;
+// bound): 1920x1024x3584 543 -> 73 us, 3840x2160x16384 9.85 -> 1.05 ms;
 // relative RMS error against FP64 6.8e-7 -> 2.3e-7 and 1.6e-6 -> 4.3e-7.
 //
+// A tile's columns are equal shares at the plan's number of waves, as in
+// umma2.cu (3840x2160x16384 1060 -> 1040 us, 640x480x300 13.3 -> 12.2).
 // Long products on few tiles are cut along K into S slices: each slice's
 // CTA writes its partial tile, and the last slice of a tile to finish adds
 // the S partials in slice order (deterministic).
@@ -164,6 +166,7 @@ constexpr int S32_ROLE_REGS = 56, S32_EPI_REGS = 224;
 
 struct Sep32Args {
     int units, tiles_m, tiles_n, KB;  // forward: tiles, K blocks; units of either
+    int bw;                           // columns per tile, at most BNP
     int M, N;
     float *D;
     long long ldd;
@@ -220,6 +223,7 @@ __device__ __forceinline__ void sep32_store(const Sep32Args &g, bool ok, int mt,
     using C = Sep32Cols<BNP>;
     constexpr int BM = 128;
     const int nu = half ? C::U1 : C::U0, c0 = half * C::U0 * 16;
+    const int end = np0 + g.bw < g.N ? np0 + g.bw : g.N;  // of the tile's columns
     bool store = ok;
     if (g.S > 1) {
         const size_t tile = (size_t)mt * g.tiles_n + nt;
@@ -265,7 +269,7 @@ __device__ __forceinline__ void sep32_store(const Sep32Args &g, bool ok, int mt,
         for (int u = 0; u < C::U0; ++u)
             if (u < nu)
                 epilogue_store_odd(stage, acc + u * 16, g.D + (long long)row0 * g.ldd, g.ldd,
-                                   g.M - row0, np0 + c0 + u * 16, g.N, false, lane);
+                                   g.M - row0, np0 + c0 + u * 16, end, false, lane);
         return;
     }
     if (row >= g.M) return;
@@ -273,10 +277,10 @@ __device__ __forceinline__ void sep32_store(const Sep32Args &g, bool ok, int mt,
 #pragma unroll
     for (int c = 0; c < C::U0 * 16; c += 8) {
         const int col = np0 + c0 + c;
-        if (c >= nu * 16 || col >= g.N) break;
-        if (g.vec == 2 && col + 8 <= g.N) {
+        if (c >= nu * 16 || col >= end) break;
+        if (g.vec == 2 && col + 8 <= end) {
             store8(drow + col, acc + c);
-        } else if (col + 8 <= g.N) {
+        } else if (col + 8 <= end) {
             *reinterpret_cast<float4 *>(drow + col) =
                 make_float4(acc[c], acc[c + 1], acc[c + 2], acc[c + 3]);
             *reinterpret_cast<float4 *>(drow + col + 4) =
@@ -284,7 +288,7 @@ __device__ __forceinline__ void sep32_store(const Sep32Args &g, bool ok, int mt,
         } else {
 #pragma unroll
             for (int e = 0; e < 8; ++e)
-                if (col + e < g.N) drow[col + e] = acc[c + e];
+                if (col + e < end) drow[col + e] = acc[c + e];
         }
     }
 }
@@ -442,13 +446,15 @@ sep32_pair_kernel(const __grid_constant__ Sep32Maps maps0,
             // -------------------------------------- producer (both CTAs)
             unsigned n = 0;  // K blocks issued
             bool ok = true;
+            const int bw = ADJ ? BNP : g.bw;
+            const uint32_t bytes = 4 * (S::A_BYTES + (uint32_t)bw * S::BK);
             for (int r = 0; r * ncl < g.units && ok; ++r) {
                 const int u = group_item_index(r, cl, ncl);
                 if (u >= g.units) break;
                 const Sep32Unit w = sep32_unit<ADJ>(u, g, ga);
                 const Sep32Maps *maps = w.which ? &maps1 : &maps0;
                 const int m0 = w.mt * 2 * S::BM + (int)rank * S::BM;  // this CTA's rows
-                const int nb = w.nt * BNP + (int)rank * S::BNH;       // its B rows
+                const int nb = w.nt * bw + (int)rank * (bw / 2);      // its B rows
                 for (int i = 0; i < w.nkb; ++i, ++n) {
                     const int s = (int)(n % STAGES);
                     if (n >= STAGES && !mbar_wait_bounded(&empty[s], ((n / STAGES) - 1) & 1)) {
@@ -462,7 +468,7 @@ sep32_pair_kernel(const __grid_constant__ Sep32Maps maps0,
                     const int k = (w.kb0 + i) * S::BK;
                     if (umma::elect_one()) {
                         // the even CTA's barrier counts the bytes of both CTAs' loads
-                        if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * S::STAGE_BYTES);
+                        if (rank == 0) mbar_arrive_expect_tx(&full[s], bytes);
                         umma2::tma_load_2d_pair(st, &maps->A, k, m0, bar);
                         umma2::tma_load_2d_pair(st + S::A_BYTES, &maps->B, k, nb, bar);
                         umma2::tma_load_2d_pair(st + S::A_BYTES + S::B_BYTES, &maps->A2, k, m0,
@@ -577,7 +583,7 @@ sep32_pair_kernel(const __grid_constant__ Sep32Maps maps0,
             } else {
                 // (every warp, also after a timeout: it meets at barriers)
                 sep32_store<BNP>(g, ok, w.mt, w.nt, w.slice, (int)rank, half, lrow, m0,
-                                 w.nt * BNP, &s_last, stage, acc);
+                                 w.nt * g.bw, &s_last, stage, acc);
             }
         }
     }
@@ -624,17 +630,17 @@ static Sep32Plan sep32_plan(int M, int N, int KB, int sms) {
     return best;
 }
 
-template <int BNP>
-static bool make_sep32_maps(Sep32Maps *m, const Sep32Operands &op, int M, int N, int K) {
+static bool make_sep32_maps(Sep32Maps *m, const Sep32Operands &op, int M, int N, int K, int bw) {
     return make_gemm_map(&m->A, op.A_hi, K, M, op.lda, 128, false) &&
-           make_gemm_map(&m->B, op.B_hi, K, N, op.ldb, BNP / 2, false) &&
+           make_gemm_map(&m->B, op.B_hi, K, N, op.ldb, bw / 2, false) &&
            make_gemm_map(&m->A2, op.A_lo, K, M, op.lda, 128, false) &&
-           make_gemm_map(&m->B2, op.B_lo, K, N, op.ldb, BNP / 2, false);
+           make_gemm_map(&m->B2, op.B_lo, K, N, op.ldb, bw / 2, false);
 }
 
 template <int BNP, int STAGES, bool ADJ>
 static cudaError_t launch_sep32_kernel(const Sep32Maps &m0, const Sep32Maps &m1,
-                                       const Sep32Args &g, const Adj32Args &ga, cudaStream_t s) {
+                                       const Sep32Args &g, const Adj32Args &ga, int bw,
+                                       cudaStream_t s) {
     using S = PairShape<BNP, true, STAGES>;
     constexpr size_t SMEM = ADJ ? S::RING : S::SMEM;
     static_assert(SMEM <= 232448 - 1024, "shared memory");
@@ -651,14 +657,14 @@ static cudaError_t launch_sep32_kernel(const Sep32Maps &m0, const Sep32Maps &m1,
     const int pairs = sm_count_of_current_device() / 2;
     const int clusters = g.units < pairs ? g.units : pairs > 0 ? pairs : 1;
     return launch_dependent(kern, dim3(2 * clusters), dim3(S32_THREADS), SMEM, s, m0, m1, g, ga,
-                            umma::idesc_f16(2 * S::BM, BNP, false));
+                            umma::idesc_f16(2 * S::BM, bw, false));
 }
 
 template <int BNP, int STAGES>
 static cudaError_t launch_sep32_t(const Sep32Operands &op, const Sep32Args &g, cudaStream_t s) {
     Sep32Maps m;
-    if (!make_sep32_maps<BNP>(&m, op, g.M, g.N, 64 * g.KB)) return cudaErrorInvalidValue;
-    return launch_sep32_kernel<BNP, STAGES, false>(m, m, g, Adj32Args{}, s);
+    if (!make_sep32_maps(&m, op, g.M, g.N, 64 * g.KB, g.bw)) return cudaErrorInvalidValue;
+    return launch_sep32_kernel<BNP, STAGES, false>(m, m, g, Adj32Args{}, g.bw, s);
 }
 
 static cudaError_t launch_sep32(int bn, const Sep32Operands &op, const Sep32Args &g,
@@ -721,11 +727,11 @@ static cudaError_t launch_adj32_t(const Sep32Operands (&op)[2], const int (&N)[2
                                   cudaStream_t s) {
     Sep32Maps m[2];
     for (int i = 0; i < 2; ++i)
-        if (!make_sep32_maps<BNP>(&m[i], op[i], 2 * ga.n, N[i], K[i])) return cudaErrorInvalidValue;
+        if (!make_sep32_maps(&m[i], op[i], 2 * ga.n, N[i], K[i], BNP)) return cudaErrorInvalidValue;
     Sep32Args g{};
     g.status = status;
     g.units = ga.p[0].units + ga.p[1].units;
-    return launch_sep32_kernel<BNP, STAGES, true>(m[0], m[1], g, ga, s);
+    return launch_sep32_kernel<BNP, STAGES, true>(m[0], m[1], g, ga, BNP, s);
 }
 
 cudaError_t launch_adj32(int bn, const Sep32Operands (&op)[2], const int (&N)[2],
@@ -749,7 +755,8 @@ cgh_status cgh_ctx::forward_sep32(const float *points, const float *A, const flo
     const int Kp = pad_to(2 * N, 64);
     const int Npad = Kp / 2;
     const Sep32Plan plan = sep32_plan(Ny, Nx, Kp / 64, sm_count);
-    const size_t tiles = (size_t)((Ny + 255) / 256) * ((Nx + plan.bn - 1) / plan.bn);
+    const int bw = pair_columns(Ny, Nx, plan.bn, sm_count, plan.S);
+    const size_t tiles = (size_t)((Ny + 255) / 256) * ((Nx + bw - 1) / bw);
     const size_t l_b = align256((size_t)Nx * Kp * 2);
     const size_t r_b = align256((size_t)Ny * Kp * 2);
     const size_t sc_b = align256((size_t)(Kp / 64) * sizeof(float));
@@ -784,7 +791,8 @@ cgh_status cgh_ctx::forward_sep32(const float *points, const float *A, const flo
         g.M = Ny;
         g.N = Nx;
         g.tiles_m = (Ny + 255) / 256;
-        g.tiles_n = (Nx + plan.bn - 1) / plan.bn;
+        g.tiles_n = (Nx + bw - 1) / bw;
+        g.bw = bw;
         g.units = g.tiles_m * g.tiles_n * plan.S;
         g.KB = Kp / 64;
         g.D = out;

@@ -249,8 +249,8 @@ bool make_gemm_map(CUtensorMap *m, const void *base, long long inner, long long 
 // -> 76.6 us; 3840x2160x16384 BF16, 16 of 240 instead of 15 of 256 in two
 // waves, 359 -> 346; 1366x768x777, 22 of 64 instead of 13 of 112, 19.9 -> 16.8;
 // 256x256x4000, 8 of 32 instead of 3 of 112, 51.7 -> 39.9.
-static int pair_columns(int M, int N, int bnp, int sms) {
-    const int rows = (M + 255) / 256, tiles = (N + bnp - 1) / bnp;
+int pair_columns(int M, int N, int bnp, int sms, int slices) {
+    const int rows = (M + 255) / 256 * slices, tiles = (N + bnp - 1) / bnp;
     const int pairs = sms / 2 > 0 ? sms / 2 : 1;
     const int most = (rows * tiles + pairs - 1) / pairs * pairs / rows;  // >= tiles
     const int bw = pad_to((N + most - 1) / most, 16);
