@@ -36,7 +36,7 @@
 // arrivals relaxed: tensor memory is ordered by the tcgen05 fences, and no
 // generic memory is handed over).
 // Measured, whole call, against an FP32 product on the FMA pipe (0.70 of its
-// bound): 1920x1024x3584 543 -> 73 us, 3840x2160x16384 9.85 -> 1.05 ms;
+// bound): 1920x1024x3584 543 -> 73 us, 3840x2160x16384 9.85 -> 1.02 ms;
 // relative RMS error against FP64 6.8e-7 -> 2.3e-7 and 1.6e-6 -> 4.3e-7.
 //
 // A tile's columns are equal shares at the plan's number of waves, as in
