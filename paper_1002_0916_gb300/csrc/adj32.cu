@@ -15,7 +15,8 @@
 // Both run on the product kernel of sep32.cu: every FP32 factor as two FP16
 // numbers, partial sums added in FP32 every 64 values of k.  U', V' are
 // scaled by 2^14 and G by the power of two that brings max |G| into [2^13,
-// 2^14).  Four launches:
+// 2^14); the sums come out in units of 2^floor(log2 max |G|), an FP32 number
+// for every G.  Four launches:
 //   1. the largest |G| of a run of pixels per block, and, in the blocks
 //      behind those, the tables U', V' with their point records;
 //   2. G to FP16 hi and lo in both orientations;
@@ -157,7 +158,7 @@ constexpr int GC_T = 64;
 
 __global__ void __launch_bounds__(A32_THREADS)
 adj32_convert_kernel(const float *__restrict__ G, int Nx, int Ny, const float *__restrict__ gmax,
-                     int nmax, float *__restrict__ gscale, __half *__restrict__ Gr_hi,
+                     int nmax, float *__restrict__ gunit, __half *__restrict__ Gr_hi,
                      __half *__restrict__ Gr_lo, int ldx, __half *__restrict__ Gt_hi,
                      __half *__restrict__ Gt_lo, int ldy) {
     __shared__ float tile[GC_T][GC_T + 1];
@@ -166,12 +167,12 @@ adj32_convert_kernel(const float *__restrict__ G, int Nx, int Ny, const float *_
     float m = 0.0f;
     for (int i = threadIdx.x; i < nmax; i += A32_THREADS) m = nan_max(m, gmax[i]);
     m = block_max(m, sm);
-    // 1 if max |G| is 0 or not finite
-    const float s = m > 0.0f && isfinite(m)
-                        ? scalbnf(1.0f, S32_EXP - 1 - (ilogbf(m) < -110 ? -110 : ilogbf(m)))
-                        : 1.0f;
-    // (the products' other factor is scaled by S32_R_SCALE)
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *gscale = s * S32_R_SCALE;
+    // (no scaling if max |G| is 0 or not finite)
+    const int e = m > 0.0f && isfinite(m) ? ilogbf(m) : S32_EXP - 1;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *gunit = scalbnf(1.0f, e);
+    // in two steps: 2^(S32_EXP - 1 - e) itself is no FP32 number for a small G
+    const int k = S32_EXP - 1 - e;
+    const float s0 = scalbnf(1.0f, k / 2), s1 = scalbnf(1.0f, k - k / 2);
     const int bx = blockIdx.x * GC_T, by = blockIdx.y * GC_T;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -179,7 +180,8 @@ adj32_convert_kernel(const float *__restrict__ G, int Nx, int Ny, const float *_
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int y = by + r, x = bx + lane + 32 * h;
-            tile[r][lane + 32 * h] = y < Ny && x < Nx ? __ldg(G + (size_t)y * Nx + x) * s : 0.0f;
+            tile[r][lane + 32 * h] =
+                y < Ny && x < Nx ? __ldg(G + (size_t)y * Nx + x) * s0 * s1 : 0.0f;
         }
     __syncthreads();
 #pragma unroll
@@ -247,7 +249,7 @@ cgh_status cgh_ctx::backward_sep32(const float *points, const float *A, const fl
         b += bytes;
         return q;
     };
-    float *gmax = (float *)take(max_b), *gscale = gmax + A32_MAX_BLOCKS;
+    float *gmax = (float *)take(max_b), *gunit = gmax + A32_MAX_BLOCKS;
     PointRec *rec = (PointRec *)take(rec_b);
     float *part[2] = {(float *)take(part_b[0]), (float *)take(part_b[1])};
     __half *Uhi = (__half *)take(u_b), *Ulo = (__half *)take(u_b);
@@ -281,7 +283,7 @@ cgh_status cgh_ctx::backward_sep32(const float *points, const float *A, const fl
             dim3 grid((ldx + GC_T - 1) / GC_T, (ldy + GC_T - 1) / GC_T);
             cudaError_t e =
                 launch_dependent(adj32_convert_kernel, grid, dim3(A32_THREADS), 0, s, G, Nx, Ny,
-                                 (const float *)gmax, (int)nmax, gscale, Grh, Grl, ldx, Gth, Gtl,
+                                 (const float *)gmax, (int)nmax, gunit, Grh, Grl, ldx, Gth, Gtl,
                                  ldy);
             if (e != cudaSuccess) return cuda_fail(e, "G convert launch");
             tl.done();
@@ -315,7 +317,7 @@ cgh_status cgh_ctx::backward_sep32(const float *points, const float *A, const fl
             const int ix = axis[0] == 0 ? 0 : 1, iy = 1 - ix;
             const AdjointParts pp{part[ix], part[iy] + npad, T[ix],       T[iy],
                                   3 * (size_t)npad, (size_t)npad};
-            cudaError_t e = launch_adjoint_sum(src, pp, gscale,
+            cudaError_t e = launch_adjoint_sum(src, pp, gunit,
                                                gpts ? gpts + 2 * (size_t)j0 : nullptr,
                                                gA ? gA + j0 : nullptr, gz ? gz + j0 : nullptr, s);
             if (e != cudaSuccess) return cuda_fail(e, "adjoint reduce launch");

@@ -183,7 +183,7 @@ __device__ __forceinline__ void two_sum(float &s, float &e, float v) {
 }
 
 __global__ void __launch_bounds__(RD_PTS * RD_SL)
-adjoint_sum_kernel(PointSource src, AdjointParts pp, const float *__restrict__ scale, float *gpts,
+adjoint_sum_kernel(PointSource src, AdjointParts pp, const float *__restrict__ unit, float *gpts,
                    float *gA, float *gz) {
     __shared__ float2 part[RD_SL][5][RD_PTS];
     __shared__ double sums[5][RD_PTS];
@@ -221,24 +221,24 @@ adjoint_sum_kernel(PointSource src, AdjointParts pp, const float *__restrict__ s
     const PointRec r =
         make_point_rec(src.points, src.A, src.z, src.N, j, src.K, (unsigned *)nullptr);
     const bool ok = r.Q32 > 0.0f;
-    const double inv = scale ? 1.0 / (double)*scale : 1.0;
+    const double g = unit ? (double)*unit : 1.0;  // the unit of the sums
     const double P = 6.283185307179586 * (double)r.Q32;
     const double a = (double)r.A;
-    if (gA) gA[j] = ok ? (float)(sums[0][lj] * inv) : 0.0f;
+    if (gA) gA[j] = ok ? (float)(sums[0][lj] * g) : 0.0f;
     if (gpts) {
-        gpts[2 * j] = ok ? (float)(2.0 * P * a * sums[1][lj] * inv) : 0.0f;
-        gpts[2 * j + 1] = ok ? (float)(2.0 * P * a * sums[3][lj] * inv) : 0.0f;
+        gpts[2 * j] = ok ? (float)(2.0 * P * a * sums[1][lj] * g) : 0.0f;
+        gpts[2 * j + 1] = ok ? (float)(2.0 * P * a * sums[3][lj] * g) : 0.0f;
     }
     if (gz)
-        gz[j] = ok ? (float)(P * a / (double)src.z[j] * (sums[2][lj] + sums[4][lj]) * inv) : 0.0f;
+        gz[j] = ok ? (float)(P * a / (double)src.z[j] * (sums[2][lj] + sums[4][lj]) * g) : 0.0f;
 }
 
-cudaError_t launch_adjoint_sum(const PointSource &src, const AdjointParts &pp, const float *scale,
+cudaError_t launch_adjoint_sum(const PointSource &src, const AdjointParts &pp, const float *unit,
                                float *gpts, float *gA, float *gz, cudaStream_t s) {
     const int tiles = pp.Tx > pp.Ty ? pp.Tx : pp.Ty;
     const int slices = tiles > 64 ? RD_SL : 8;  // (few tiles: the slices' own sum dominates)
     return launch_dependent(adjoint_sum_kernel, dim3((src.N + RD_PTS - 1) / RD_PTS),
-                            dim3(RD_PTS * slices), 0, s, src, pp, scale, gpts, gA, gz);
+                            dim3(RD_PTS * slices), 0, s, src, pp, unit, gpts, gA, gz);
 }
 
 // Rows per run: the fewest runs (each repeats the columns' sincos, worth

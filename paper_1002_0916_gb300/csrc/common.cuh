@@ -237,9 +237,9 @@ struct AdjointParts {
     int Tx, Ty;
     size_t stride, npad;
 };
-// Adds them in a fixed order, divides by *scale (nullptr: 1) and applies the
+// Adds them in a fixed order, multiplies by *unit (nullptr: 1) and applies the
 // per-point factors; any of the three outputs may be null.
-cudaError_t launch_adjoint_sum(const PointSource &src, const AdjointParts &pp, const float *scale,
+cudaError_t launch_adjoint_sum(const PointSource &src, const AdjointParts &pp, const float *unit,
                                float *gpts, float *gA, float *gz, cudaStream_t s);
 // The same tables with the records built inside the kernel (no prologue).
 cudaError_t launch_direct_tables_fused(const PointSource &src, int Npad, int Nx,

@@ -556,7 +556,7 @@ sep32_pair_kernel(const __grid_constant__ Sep32Maps maps0,
             float acc[C::U0 * 16];
 #pragma unroll
             for (int i = 0; i < C::U0 * 16; ++i) acc[i] = 0.0f;
-            float f_next = ADJ ? 1.0f : __ldg(g.scale + w.kb0);
+            float f_next = ADJ ? S32_ADJ_FACTOR : __ldg(g.scale + w.kb0);
             for (int i = 0; i < w.nkb && ok; ++i, ++n) {
                 const int b = (int)(n % C::NBUF);
                 const float f = f_next;

@@ -13,6 +13,10 @@ namespace cgh {
 // R entries are scaled by 2^S32_EXP, a block's L entries to below it.
 constexpr int S32_EXP = 14;
 constexpr float S32_R_SCALE = 16384.0f;
+// The adjoint's products are taken out of both factors' scales, 2^S32_EXP and
+// 2^(S32_EXP - 1), as they are added up: sums in units of max |G| rounded down
+// to a power of two, whatever its size.
+constexpr float S32_ADJ_FACTOR = 1.0f / 134217728.0f;  // 2^-27
 
 // sin and cos of a 0.64 fixed-point phase: the nearest quarter turn is taken
 // off in fixed point, so that the remainder x (quarter turns, |x| <= 1/2)
