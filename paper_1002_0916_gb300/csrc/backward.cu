@@ -60,19 +60,20 @@ static int bwd_strip(int Nx, int Ny, int N) {
     return (double)Nx * Ny * N < (double)(1 << 25) ? 16 : 32;
 }
 
-// Grid: x = column strips, y = groups of BWD_THREADS points, z = runs of
-// `rows` rows.  part: [strip * runs + run][5][Npad], the sums of G cos, G sin
+// Grid: x = column strips (fastest) of every group of BWD_THREADS points, one
+// dimension for both since 2^24 points are more groups than grid y takes; y =
+// runs of `rows` rows.  part: [strip * runs + run][5][Npad], the sums of G cos, G sin
 // dx, G sin dx^2, G sin dy, G sin dy^2.
 template <int STRIP>
 __global__ void __launch_bounds__(BWD_THREADS, BwdShape<STRIP>::CTAS)
-direct_bwd_kernel(PointSource src, int Npad, int Nx, int Ny, int rows,
+direct_bwd_kernel(PointSource src, int Npad, int Nx, int Ny, int strips, int rows,
                   const float *__restrict__ G, float *__restrict__ part) {
     constexpr int NP2 = BwdShape<STRIP>::NP2, RB = BwdShape<STRIP>::RB;
     constexpr int LOADS = RB * STRIP / BWD_THREADS, UNROLL = BwdShape<STRIP>::UNROLL;
     __shared__ __align__(16) float sg[2][RB][STRIP];
-    const int strip = blockIdx.x, x0 = strip * STRIP;
-    const int j = blockIdx.y * BWD_THREADS + threadIdx.x;
-    const int ya = blockIdx.z * rows, yb = ya + rows < Ny ? ya + rows : Ny;
+    const int strip = blockIdx.x % strips, x0 = strip * STRIP;
+    const int j = blockIdx.x / strips * BWD_THREADS + threadIdx.x;
+    const int ya = blockIdx.y * rows, yb = ya + rows < Ny ? ya + rows : Ny;
     const int lc = threadIdx.x % STRIP, lr = threadIdx.x / STRIP;
     const float *gcol = G + x0 + lc;
     const bool in_x = x0 + lc < Nx;
@@ -156,7 +157,7 @@ direct_bwd_kernel(PointSource src, int Npad, int Nx, int Ny, int rows,
         sX += t0 + t1;
         sXX = fmaf(t0, dx0, fmaf(t1, dx1, sXX));
     }
-    float *dst = part + ((size_t)(strip * gridDim.z + blockIdx.z) * 5) * Npad + j;
+    float *dst = part + ((size_t)(strip * gridDim.y + blockIdx.y) * 5) * Npad + j;
     dst[0] = C;
     dst[(size_t)Npad] = sX;
     dst[(size_t)2 * Npad] = sXX;
@@ -281,10 +282,10 @@ static cgh_status run_direct_backward(cgh_ctx *h, const float *points, const flo
     const PointSource src{points, A, z, N, fresnel_scale(lambda, p), h->d_status};
     {
         TimedLaunch tl(h, CGH_K_BWD_DIRECT, s);
-        const dim3 grid(strips, (N + BWD_THREADS - 1) / BWD_THREADS, runs);
+        const dim3 grid((unsigned)strips * ((N + BWD_THREADS - 1) / BWD_THREADS), runs);
         cudaError_t e = launch_kernel(
             false, strip == 32 ? direct_bwd_kernel<32> : direct_bwd_kernel<16>, grid,
-            dim3(BWD_THREADS), 0, s, src, Npad, Nx, Ny, rows, G, part);
+            dim3(BWD_THREADS), 0, s, src, Npad, Nx, Ny, strips, rows, G, part);
         if (e != cudaSuccess) return h->cuda_fail(e, "direct adjoint launch");
         tl.done();
     }

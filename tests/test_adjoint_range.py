@@ -44,3 +44,15 @@ def test_size_of_the_gradient_field(cg, method, scale):
     assert np.abs(G).max() > 0
     for v, ref, bound in zip(_backward(cg, c, G, method), *_reference(c, G)):
         assert np.all(np.abs(v - ref) <= EPS * bound + 2.0 ** -149)
+
+
+# more points than 65535 groups of 128, in strips of 16 columns (1 x 3 pixels)
+# and of 32 (5 x 1), and in the separable adjoint two chunks of points
+@pytest.mark.parametrize("Nx,Ny", [(1, 3), (5, 1)])
+@pytest.mark.parametrize("method", ["direct", "sep_fp32"])
+def test_many_points(cg, method, Nx, Ny):
+    N = 65535 * 128 + 1000
+    c = make_cloud(5, N, Nx, Ny, integer=False, zlo=0.2, zhi=0.9, lam=532e-9, p=6.4e-6)
+    G = grad_field(6, Nx, Ny)
+    for v, ref, bound in zip(_backward(cg, c, G, method), *_reference(c, G)):
+        assert np.all(np.abs(v - ref) <= EPS * bound)
