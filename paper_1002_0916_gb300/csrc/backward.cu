@@ -215,7 +215,17 @@ adjoint_sum_kernel(PointSource src, AdjointParts pp, const float *__restrict__ u
             two_sum(v, w, part[q][k][lj].x);
             w += part[q][k][lj].y;
         }
-        sums[k][lj] = (double)v + (double)w;
+        double sum = (double)v + (double)w;
+        if (!isfinite(sum) && j < src.N) {
+            // an infinite partial sum, whose rounding error is NaN, or a
+            // total past FP32's range: once more in FP64
+            const bool is_x = k < 3;
+            const float *p = (is_x ? pp.x + k * pp.npad : pp.y + (k - 3) * pp.npad) + j;
+            const int T = is_x ? pp.Tx : pp.Ty;
+            sum = 0.0;
+            for (int t = 0; t < T; ++t) sum += (double)__ldcg(p + t * pp.stride);
+        }
+        sums[k][lj] = sum;
     }
     __syncthreads();
     if (sl != 0 || j >= src.N) return;

@@ -56,3 +56,26 @@ def test_many_points(cg, method, Nx, Ny):
     G = grad_field(6, Nx, Ny)
     for v, ref, bound in zip(_backward(cg, c, G, method), *_reference(c, G)):
         assert np.all(np.abs(v - ref) <= EPS * bound)
+
+
+def test_sums_past_the_range_of_fp32(cg):
+    """A field with the sign of sin(phi) (x - x_j) of one point.  Partial sums
+    that are FP32 numbers but not their total, which 2 P A brings back into range;
+    and infinite partial sums: an infinite gradient, not NaN."""
+    c = make_cloud(8, 1, 512, 64, integer=False, zlo=0.4, zhi=0.5, lam=532e-9, p=3.74e-6)
+    c.A[:] = 0.5
+    P = np.pi * c.p * c.p / (c.lam * float(c.z[0]))
+    dx, dy = np.arange(512) - float(c.xy[0, 0]), np.arange(64) - float(c.xy[0, 1])
+    w = np.sin(P * (dx[None, :] ** 2 + dy[:, None] ** 2)) * dx[None, :]
+    top, strip = 2.0 ** 128, np.abs(w).reshape(64, 32, 16).sum((0, 2)).max()
+    size = 1.2e33
+    assert np.abs(w).sum() * size > 4 * top and strip * size < top
+    G = (np.sign(w) * size).astype(np.float32)
+    got = _backward(cg, c, G, "direct")
+    ref, bound = _reference(c, G)
+    for k in (0, 1):
+        assert abs(ref[k][0]) < top and abs(got[k][0] - ref[k][0]) <= EPS * bound[k][0]
+    # (no column's sum of G sin(phi) is past the range, its product with x - x_j is)
+    size = 4e36
+    assert 64 * size < top < strip * size
+    assert _backward(cg, c, (np.sign(w) * size).astype(np.float32), "direct")[0][0] == np.inf
