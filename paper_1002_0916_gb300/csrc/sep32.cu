@@ -561,14 +561,11 @@ sep32_pair_kernel(const __grid_constant__ Sep32Maps maps0,
                 const int b = (int)(n % C::NBUF);
                 const float f = f_next;
                 if (!ADJ) f_next = __ldg(g.scale + w.kb0 + (i + 1 < w.nkb ? i + 1 : i));
-                ok = __all_sync(0xffffffffu,
-                                mbar_wait_bounded(&acc_full[b], (n / C::NBUF) & 1));
+                const bool landed = mbar_wait_bounded(&acc_full[b], (n / C::NBUF) & 1);
+                if (!landed) set_status(g.status, DEV_TIMEOUT);
+                ok = __all_sync(0xffffffffu, landed && !abort_flag);
+                if (!ok) break;
                 umma::fence_after_sync();
-                if (!ok || abort_flag) {
-                    if (!ok) set_status(g.status, DEV_TIMEOUT);
-                    ok = false;
-                    break;
-                }
                 sep32_promote<C::U0>(t0 + (uint32_t)b * C::STRIDE, nu, f, acc);
                 umma::fence_before_sync();
                 __syncwarp();

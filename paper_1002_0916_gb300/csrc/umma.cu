@@ -180,13 +180,14 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tA,
         // ----------------------------------------------------- epilogue
         const int q = warp & 3;  // the 32-lane quarter of TMEM this warp reads
         const int row = m0 + q * 32 + lane;
+        const bool done = mbar_wait_bounded(&accum_bar, 0);
+        if (!done) set_status(g.status, DEV_TIMEOUT);
         // warp-uniform, so the .sync.aligned TMEM loads below are executed by
         // whole warps
-        const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&accum_bar, 0));
+        const bool ok = __all_sync(0xffffffffu, done && !abort_flag);
         umma::fence_after_sync();
         pdl_trigger();  // only the epilogue is left
-        if (!ok) set_status(g.status, DEV_TIMEOUT);
-        if (ok && !abort_flag) {
+        if (ok) {
             const uint32_t t_row = tmem + ((uint32_t)(q * 32) << 16);
             float *drow = g.D + (long long)row * g.ldd;
             const int vec = store_width(g.D, g.ldd);
@@ -531,13 +532,10 @@ umma_grouped_kernel(const GroupProb *__restrict__ probs,
         int n = 0;
         for (int it = blockIdx.x; it < nitems; it += gridDim.x, ++n) {
             const int b = n & 1;
-            const bool ok = __all_sync(
-                0xffffffffu, mbar_wait_bounded(&acc_full[b], (uint32_t)((n >> 1) & 1)));
+            const bool done = mbar_wait_bounded(&acc_full[b], (uint32_t)((n >> 1) & 1));
+            if (!done) set_status(status, DEV_TIMEOUT);
+            if (!__all_sync(0xffffffffu, done && !abort_flag)) break;
             umma::fence_after_sync();
-            if (!ok || abort_flag) {
-                if (!ok) set_status(status, DEV_TIMEOUT);
-                break;
-            }
             const uint2 w = items[it];
             const GroupProb *gp = probs + w.x;
             const int m0 = (int)(w.y & 0xffffu) * S::BM, n0 = (int)(w.y >> 16) * BN;

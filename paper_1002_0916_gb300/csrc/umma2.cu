@@ -182,11 +182,12 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tA,
         // --------------------------------------- epilogue (both CTAs)
         const int q = warp & 3;  // the 32-lane quarter of TMEM this warp reads
         const int row = m0 + q * 32 + lane;
-        const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&accum_bar, 0));
+        const bool done = mbar_wait_bounded(&accum_bar, 0);
+        if (!done) set_status(g.status, DEV_TIMEOUT);
+        const bool ok = __all_sync(0xffffffffu, done && !abort_flag);
         umma::fence_after_sync();
         pdl_trigger();  // only the epilogue is left
-        if (!ok) set_status(g.status, DEV_TIMEOUT);
-        if (ok && !abort_flag) {
+        if (ok) {
             const uint32_t t_row = tmem + ((uint32_t)(q * 32) << 16);
             float *drow = g.D + (long long)row * g.ldd;
             const int vec = store_width(g.D, g.ldd);
@@ -531,14 +532,10 @@ umma_grouped_pair_kernel(const GroupProb *__restrict__ probs,
         for (int n = 0; n * ncl < nitems; ++n) {
             const int it = group_item_index(n, cl, ncl), b = n % NBUF;
             if (it >= nitems) break;
-            const bool ok = __all_sync(
-                0xffffffffu,
-                mbar_wait_bounded(&acc_full[b], (uint32_t)((n / NBUF) & 1)));
+            const bool done = mbar_wait_bounded(&acc_full[b], (uint32_t)((n / NBUF) & 1));
+            if (!done) set_status(status, DEV_TIMEOUT);
+            if (!__all_sync(0xffffffffu, done && !abort_flag)) break;
             umma::fence_after_sync();
-            if (!ok || abort_flag) {
-                if (!ok) set_status(status, DEV_TIMEOUT);
-                break;
-            }
             const uint2 w = items[it];
             const GroupProb *gp = probs + w.x;
             const int m0 = (int)(w.y & 0xffffu) * 2 * S::BM + (int)rank * S::BM;

@@ -212,17 +212,12 @@ umma_gen_pair_kernel(GenArgs ga, GemmArgs g, uint32_t idesc) {
         const uint32_t full_even0 = umma2::map_to_rank(&full[0], 0);
         for (int kb = 0; kb < KB; ++kb) {
             const int s = kb % STAGES;
-            if (kb >= STAGES) {
-                bool ok = true;
-                if (lane == 0)
-                    ok = mbar_wait_bounded(&empty[s], (uint32_t)(((kb / STAGES) - 1) & 1));
-                ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-                if (!ok) {
-                    abort_flag = 1;
-                    set_status(g.status, DEV_TIMEOUT);
-                }
+            if (kb >= STAGES && lane == 0 &&
+                !mbar_wait_bounded(&empty[s], (uint32_t)(((kb / STAGES) - 1) & 1))) {
+                abort_flag = 1;
+                set_status(g.status, DEV_TIMEOUT);
             }
-            if (abort_flag) break;
+            if (!__all_sync(0xffffffffu, !abort_flag)) break;
             uint8_t *st = smem + (size_t)s * S::STAGE_BYTES;
             if (on_a)
                 gen_run<KIND, false>(ga, kb, lane, r0, r1, m0, g.M, st,
@@ -249,12 +244,12 @@ umma_gen_pair_kernel(GenArgs ga, GemmArgs g, uint32_t idesc) {
         if (warp <= 4) {
             const int qq = warp & 3;  // the 32-lane quarter of TMEM this warp reads
             const int row = m0 + qq * 32 + lane;
-            const bool ok =
-                __all_sync(0xffffffffu, umma2::wait_cluster_bounded(&accum_bar, 0));
+            const bool done = umma2::wait_cluster_bounded(&accum_bar, 0);
+            if (!done) set_status(g.status, DEV_TIMEOUT);
+            const bool ok = __all_sync(0xffffffffu, done && !abort_flag);
             umma::fence_after_sync();
             pdl_trigger();  // only the epilogue is left
-            if (!ok) set_status(g.status, DEV_TIMEOUT);
-            if (ok && !abort_flag) {
+            if (ok) {
                 const uint32_t t_row = tmem + ((uint32_t)(qq * 32) << 16);
                 float *drow = g.D + (long long)row * g.ldd;
                 const bool vec = ((g.ldd & 3) == 0) && ((((uintptr_t)g.D) & 15) == 0);
