@@ -405,6 +405,7 @@ sep32_pair_kernel(const __grid_constant__ Sep32Maps maps0,
     __shared__ __align__(8) uint64_t empty[STAGES];
     __shared__ __align__(8) uint64_t acc_full[C::NBUF];
     __shared__ __align__(8) uint64_t acc_empty[C::NBUF];  // (even CTA) both epilogues done
+    __shared__ __align__(8) uint64_t drain;  // (even CTA) after a timeout: MMAs done
     __shared__ uint32_t tmem_base;
     __shared__ volatile int abort_flag;
     __shared__ int s_last;
@@ -424,6 +425,7 @@ sep32_pair_kernel(const __grid_constant__ Sep32Maps maps0,
             mbar_init(&acc_full[b], 1);
             mbar_init(&acc_empty[b], 2 * S32_EPI_WARPS);
         }
+        mbar_init(&drain, 1);
         mbar_fence_init();
         umma::prefetch_tmap(&maps0.A);
         umma::prefetch_tmap(&maps0.B);
@@ -533,6 +535,12 @@ sep32_pair_kernel(const __grid_constant__ Sep32Maps maps0,
                     }
                     __syncwarp();
                 }
+            }
+            if (!ok) {
+                // the blocks issued so far use the stages and tensor memory of
+                // both CTAs, which are released after the closing barrier
+                if (umma::elect_one()) umma2::commit2(&drain, 0x1);
+                mbar_wait_bounded(&drain, 0);
             }
         }
     } else {

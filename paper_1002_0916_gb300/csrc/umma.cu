@@ -403,6 +403,7 @@ umma_grouped_kernel(const GroupProb *__restrict__ probs,
     __shared__ __align__(8) uint64_t empty[STAGES];
     __shared__ __align__(8) uint64_t acc_full[2];
     __shared__ __align__(8) uint64_t acc_empty[2];
+    __shared__ __align__(8) uint64_t drain;  // after a timeout: MMAs done
     __shared__ uint32_t tmem_base;
     __shared__ volatile int abort_flag;
 
@@ -419,6 +420,7 @@ umma_grouped_kernel(const GroupProb *__restrict__ probs,
             mbar_init(&acc_full[b], 1);
             mbar_init(&acc_empty[b], 4);  // one arrival per epilogue warp
         }
+        mbar_init(&drain, 1);
         mbar_fence_init();
     }
     if (warp == 1) {
@@ -525,6 +527,12 @@ umma_grouped_kernel(const GroupProb *__restrict__ probs,
             }
             if (umma::elect_one()) umma::mma_commit(&acc_full[b]);
             __syncwarp();
+        }
+        if (!ok) {
+            // the MMAs issued so far use the stages and tensor memory, which are
+            // released after the closing barrier
+            if (umma::elect_one()) umma::mma_commit(&drain);
+            mbar_wait_bounded(&drain, 0);
         }
     } else if (warp >= 2) {
         // ----------------------------------------------------- epilogue

@@ -391,6 +391,7 @@ umma_grouped_pair_kernel(const GroupProb *__restrict__ probs,
     __shared__ __align__(8) uint64_t empty[STAGES];
     __shared__ __align__(8) uint64_t acc_full[NBUF];
     __shared__ __align__(8) uint64_t acc_empty[NBUF];
+    __shared__ __align__(8) uint64_t drain;  // (even CTA) after a timeout: MMAs done
     __shared__ uint32_t tmem_base;
     __shared__ volatile int abort_flag;
 
@@ -409,6 +410,7 @@ umma_grouped_pair_kernel(const GroupProb *__restrict__ probs,
             mbar_init(&acc_full[b], 1);
             mbar_init(&acc_empty[b], 2 * GP_EPI_WARPS);
         }
+        mbar_init(&drain, 1);
         mbar_fence_init();
     }
     if (warp == 1) {
@@ -524,6 +526,12 @@ umma_grouped_pair_kernel(const GroupProb *__restrict__ probs,
             // wait runs out); this CTA's epilogue learns that its MMAs ended
             if (umma::elect_one()) umma2::commit2(&acc_full[b], ok ? 0x3 : 0x1);
             __syncwarp();
+        }
+        if (!ok) {
+            // the MMAs issued so far use the stages and tensor memory of both
+            // CTAs, which are released after the closing barrier
+            if (umma::elect_one()) umma2::commit2(&drain, 0x1);
+            mbar_wait_bounded(&drain, 0);
         }
     } else if (warp >= 2) {
         // --------------------------------------- epilogue (both CTAs)
