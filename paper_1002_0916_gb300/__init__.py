@@ -204,9 +204,12 @@ def _stream_ptr(stream) -> Optional[int]:
     if stream is None:
         # the current stream of the current device; without the Stream object
         # torch.cuda.current_stream() makes for it (3 us of a call's 23) where
-        # PyTorch has its CUDA state already
+        # PyTorch has its CUDA state already and these two internal functions
         if torch.cuda.is_initialized():
-            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+            try:
+                return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+            except AttributeError:
+                pass
         stream = torch.cuda.current_stream()
     return int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream)
 
