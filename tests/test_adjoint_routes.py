@@ -1,0 +1,48 @@
+"""The separable methods' adjoint on both sides of the lines that choose how it
+runs, against FP64 sums in numpy; bounds as in test_adjoint_edges.py."""
+import numpy as np
+import pytest
+
+from gpu_util import to_dev
+from test_adjoint_edges import EPS, _reference
+from workloads import grad_field, make_cloud
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def cg():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    import paper_1002_0916_gb300 as cg
+    return cg
+
+
+def _check(cg, Nx, Ny, N):
+    import torch
+    c = make_cloud(40 + Nx + N, N, Nx, Ny, integer=bool(N & 1), zlo=0.2, zhi=0.9, lam=532e-9,
+                   p=6.4e-6)
+    G = grad_field(41 + N, Nx, Ny, scale=3.0)
+    h = cg.cgh_create(0)
+    out = []
+    try:
+        for method in ("sep_fp32", "sep_fp16x3"):
+            gp, gA, gz = cg.cgh_backward(*to_dev(c), c.lam, c.p, Nx, Ny,
+                                         torch.from_numpy(G).cuda(), method=method, handle=h)
+            torch.cuda.synchronize()
+            assert cg.cgh_last_device_status(h) == cg.CGH_OK
+            gp = gp.cpu().numpy()
+            out.append([gp[:, 0], gp[:, 1], gA.cpu().numpy(), gz.cpu().numpy()])
+    finally:
+        cg.cgh_destroy(h)
+    for u, v in zip(*out):
+        assert np.array_equal(u, v)
+    for v, ref, bound in zip(out[0], *_reference(c, G)):
+        assert np.all(np.abs(v - ref) <= EPS * bound)
+
+
+# the K of the longer axis cut into slices, along either axis
+@pytest.mark.parametrize("Nx,Ny,N", [(32768, 33, 129), (33, 32768, 200), (8192, 50, 1000)])
+def test_slices_of_a_long_axis(cg, Nx, Ny, N):
+    _check(cg, Nx, Ny, N)
