@@ -204,7 +204,8 @@ cgh_status cgh_host_wait_ticket(cgh_handle h, uint64_t ticket);
  * CGH_SEP_FP32 or CGH_SEP_FP16X3 (both: two tensor-core products, G V and
  * G^T U, at the accuracy of CGH_SEP_FP32's forward -- every FP32 factor split
  * into two FP16 numbers, partial sums added in FP32 -- with the pixel sums
- * fused into their epilogues; deterministic).  Other methods:
+ * fused into their epilogues; deterministic; small and low frames by the
+ * direct method's sums instead).  Other methods:
  * CGH_ERR_INVALID_ARG.  Errors as cgh_forward. */
 cgh_status cgh_backward(cgh_handle h, const float *points, const float *A,
                         const float *z, int N, double lambda, double p,

@@ -14,7 +14,8 @@
 // reduction kernel adds the strips' and runs' partial sums in a fixed order
 // (deterministic) and applies the per-point factors.
 //
-// The separable methods run on the tensor cores (adj32.cu).
+// The separable methods run on the tensor cores (adj32.cu), small and low
+// frames (sep_by_strips) on the same sums.
 #include <math.h>
 
 #include "api_internal.h"
@@ -64,7 +65,8 @@ static int bwd_strip(int Nx, int Ny, int N) {
 // dimension for both since 2^24 points are more groups than grid y takes; y =
 // runs of `rows` rows.  part: [strip * runs + run][5][Npad], the sums of G cos, G sin
 // dx, G sin dx^2, G sin dy, G sin dy^2.
-template <int STRIP>
+// ROW32: the rows' sines and cosines to FP32 rounding too (sep_by_strips).
+template <int STRIP, bool ROW32>
 __global__ void __launch_bounds__(BWD_THREADS, BwdShape<STRIP>::CTAS)
 direct_bwd_kernel(PointSource src, int Npad, int Nx, int Ny, int strips, int rows,
                   const float *__restrict__ G, float *__restrict__ part) {
@@ -119,7 +121,8 @@ direct_bwd_kernel(PointSource src, int Npad, int Nx, int Ny, int strips, int row
 #pragma unroll UNROLL
         for (int r = 0; r < n; ++r) {
             float sy, cy;
-            __sincosf((float)phase_hi(th) * RAD_PER_U32, &sy, &cy);
+            if constexpr (ROW32) sincos_fixed(th, sy, cy);
+            else __sincosf((float)phase_hi(th) * RAD_PER_U32, &sy, &cy);
             th += dth;
             dth += d2;
             const float2 cy2 = make_float2(cy, cy), sy2 = make_float2(sy, sy);
@@ -252,6 +255,23 @@ cudaError_t launch_adjoint_sum(const PointSource &src, const AdjointParts &pp, c
                             dim3(RD_PTS * slices), 0, s, src, pp, unit, gpts, gA, gz);
 }
 
+// Frames whose adjoint the separable methods take by the strips: the products
+// of adj32.cu (four launches; K in 64s, columns in 192s at least) are mostly
+// padding on small and on low frames.  Strips against products, us: 16x16x16384
+// 8.5 and 39, 64x64x4000 11.8 and 20, 512x32x1000 14.7 and 19, 181x181x300 13.7
+// and 19, 2048x16x4000 50 and 61, 32768x3x500 76 and 375; on the other side of
+// the lines 91x91x100000 184 and 180, 256x128x760 20 and 18.5, 48x200x16384 54
+// and 44, 2048x24x1000 27 and 26, 32768x16x16 69 and 53.  With the rows' sines to
+// FP32 rounding (3% of the time) the strips are no less accurate: 64x64x4000 x
+// 1.4e-7, A 1.6e-7, z 1.3e-7 from FP64, the products 2.3e-7, 1.9e-7, 2.5e-7.
+static bool sep_by_strips(int N, int Nx, int Ny) {
+    const long long pixels = (long long)Nx * Ny;
+    const bool small = Nx <= 8192 && Ny <= 1024 &&
+                       (pixels <= 8192 ||
+                        (pixels <= 32768 && pixels * N <= (Ny <= 64 ? 25000000 : 12000000)));
+    return small || (Ny <= 20 && N >= 256);
+}
+
 // Rows per run: the fewest runs (each repeats the columns' sincos, worth
 // about 16 rows) whose CTAs fill the SMs' slots in nearly whole waves.
 static int bwd_rows(int strip, int Nx, int Ny, int N, int sms) {
@@ -278,10 +298,11 @@ static int bwd_rows(int strip, int Nx, int Ny, int N, int sms) {
 
 using namespace cgh;
 
+// timer: the cgh_kernel_id of the strips' launch
 static cgh_status run_direct_backward(cgh_ctx *h, const float *points, const float *A,
                                       const float *z, int N, double lambda, double p, int Nx,
                                       int Ny, const float *G, float *gpts, float *gA, float *gz,
-                                      cudaStream_t s) {
+                                      bool row32, int timer, cudaStream_t s) {
     const int Npad = pad_to(N, 32);
     const int strip = bwd_strip(Nx, Ny, N), strips = (Nx + strip - 1) / strip;
     const int rows = bwd_rows(strip, Nx, Ny, N, h->sm_count), runs = (Ny + rows - 1) / rows;
@@ -291,11 +312,12 @@ static cgh_status run_direct_backward(cgh_ctx *h, const float *points, const flo
     float *part = (float *)h->ws2.ptr;
     const PointSource src{points, A, z, N, fresnel_scale(lambda, p), h->d_status};
     {
-        TimedLaunch tl(h, CGH_K_BWD_DIRECT, s);
+        TimedLaunch tl(h, timer, s);
         const dim3 grid((unsigned)strips * ((N + BWD_THREADS - 1) / BWD_THREADS), runs);
+        auto kern = strip == 32 ? (row32 ? direct_bwd_kernel<32, true> : direct_bwd_kernel<32, false>)
+                                : (row32 ? direct_bwd_kernel<16, true> : direct_bwd_kernel<16, false>);
         cudaError_t e = launch_kernel(
-            false, strip == 32 ? direct_bwd_kernel<32> : direct_bwd_kernel<16>, grid,
-            dim3(BWD_THREADS), 0, s, src, Npad, Nx, Ny, strips, rows, G, part);
+            false, kern, grid, dim3(BWD_THREADS), 0, s, src, Npad, Nx, Ny, strips, rows, G, part);
         if (e != cudaSuccess) return h->cuda_fail(e, "direct adjoint launch");
         tl.done();
     }
@@ -332,13 +354,19 @@ extern "C" cgh_status cgh_backward(cgh_handle h, const float *points,
         st = h->fail(CGH_ERR_INVALID_ARG, "gradient arrays must be 4-byte aligned");
     if (st == CGH_OK && N > 0 && (grad_points || grad_A || grad_z)) {
         if (method == CGH_DIRECT_FP32)
-            st = run_direct_backward(h, points, A, z, N, lambda, p, Nx, Ny, grad_out,
-                                     grad_points, grad_A, grad_z, (cudaStream_t)stream);
-        else
-            st = h->backward_sep32(points, A, z, N, lambda, p, Nx, Ny, grad_out, grad_points,
-                                   grad_A, grad_z,
-                                   method == CGH_SEP_FP32 ? CGH_K_BWD_SIMT : CGH_K_BWD_GEMM,
-                                   (cudaStream_t)stream);
+            st = run_direct_backward(h, points, A, z, N, lambda, p, Nx, Ny, grad_out, grad_points,
+                                     grad_A, grad_z, false, CGH_K_BWD_DIRECT,
+                                     (cudaStream_t)stream);
+        else {
+            const int timer = method == CGH_SEP_FP32 ? CGH_K_BWD_SIMT : CGH_K_BWD_GEMM;
+            if (sep_by_strips(N, Nx, Ny))
+                st = run_direct_backward(h, points, A, z, N, lambda, p, Nx, Ny, grad_out,
+                                         grad_points, grad_A, grad_z, true, timer,
+                                         (cudaStream_t)stream);
+            else
+                st = h->backward_sep32(points, A, z, N, lambda, p, Nx, Ny, grad_out, grad_points,
+                                       grad_A, grad_z, timer, (cudaStream_t)stream);
+        }
     }
     if (prev != h->device) cudaSetDevice(prev);
     return st;

@@ -46,3 +46,30 @@ def _check(cg, Nx, Ny, N):
 @pytest.mark.parametrize("Nx,Ny,N", [(32768, 33, 129), (33, 32768, 200), (8192, 50, 1000)])
 def test_slices_of_a_long_axis(cg, Nx, Ny, N):
     _check(cg, Nx, Ny, N)
+
+
+# the strips of the direct adjoint (small and low frames) and the products, each
+# side of every line between them, and the products at the edges of their tiles
+@pytest.mark.parametrize("Nx,Ny,N", [
+    (1, 1, 1), (91, 90, 5000), (128, 64, 5000), (129, 64, 3000), (129, 65, 3000), (256, 128, 366),
+    (256, 128, 367), (257, 128, 64), (512, 64, 762), (512, 64, 763), (2000, 20, 256),
+    (2000, 20, 255), (2000, 21, 256), (8192, 1, 7), (8193, 1, 255), (7, 1024, 64), (7, 1025, 64),
+    (1, 1100, 1), (3, 1500, 127), (17, 1030, 128), (40, 1025, 257), (32768, 2, 100)])
+def test_strips_and_products(cg, Nx, Ny, N):
+    _check(cg, Nx, Ny, N)
+
+
+def test_accuracy_of_a_small_frame(cg):
+    """Phases of a small part of a turn, where sin(phi) is small and needs a
+    relative error: every gradient within 1e-6 of FP64 (the strips with the
+    hardware's sines are 2e-6 off here)."""
+    import torch
+    for seed in range(3):
+        c = make_cloud(seed, 1000, 16, 16, integer=False, zlo=0.5, zhi=1.5, lam=532e-9, p=6.4e-6)
+        G = grad_field(seed + 9, 16, 16)
+        gp, gA, gz = cg.cgh_backward(*to_dev(c), c.lam, c.p, 16, 16, torch.from_numpy(G).cuda(),
+                                     method="sep_fp32")
+        got = [gp[:, 0], gp[:, 1], gA, gz]
+        for v, ref in zip(got, _reference(c, G)[0]):
+            v = v.cpu().numpy().astype(np.float64)
+            assert np.linalg.norm(v - ref) <= 1e-6 * np.linalg.norm(ref)
