@@ -233,8 +233,8 @@ typedef struct {
  * call runs many such frames (of any size) as one piece of device work.  probs: host array of `count` problems
  * (1 <= count <= 4096).  The work list of (problem, tile) items is built on
  * the host, sorted longest-first; the direct method runs one CTA per item in
- * that order, the tensor-core method persistent CTAs that pull the items from
- * an atomic counter.  method: CGH_DIRECT_FP32 or CGH_SEP_FP16X3.
+ * that order, the tensor-core method persistent CTAs that the items are dealt
+ * to (CTA pairs back and forth, single CTAs round robin).  method: CGH_DIRECT_FP32 or CGH_SEP_FP16X3.
  * The launches are captured once per batch geometry (problem count, sizes,
  * constants and buffer addresses) into a CUDA graph that later calls of the
  * same geometry replay; the graph reads the buffers' current contents.
@@ -366,8 +366,8 @@ cgh_status cgh_set_direct_schedule(cgh_handle h, int schedule);
  *                    cgh_batch takes CGH_GEMM_PAIRS then);
  *   CGH_GEMM_AUTO:   the handle's tuned plan for the size (cgh_tune), else
  *                    CTA pairs for single holograms of more
- *                    than 128 rows and for cgh_batch, one-CTA tiles
- *                    otherwise.
+ *                    than 128 rows and for cgh_batch unless its low frames
+ *                    pad the pairs' tiles, one-CTA tiles otherwise.
  * Every mode computes the same products with FP32 accumulation; results
  * agree to rounding.  The adjoint has one tiling of its own (CTA pairs) and
  * does not depend on this setting. */
@@ -492,7 +492,7 @@ cgh_status cgh_kernel_time(cgh_handle h, int kernel, double *total_ms,
  * NULL).  CGH_SEP_FP16X3: time the persistent grouped GEMM's two item
  * shapes (one-CTA 128 x 128 items and CTA-pair 256 x 128 items) and keep
  * the faster for batches of the same sizes (*chosen, if not NULL, is
- * zeroed).  The built-in choice (the heuristic's tile; one-CTA items) is
+ * zeroed).  The built-in choice (the heuristic's tile or kind of items) is
  * kept unless another is more than 1% faster.  Later cgh_batch calls of
  * that method and these sizes use the choice (with the GEMM tiling
  * CGH_GEMM_AUTO for the separable batch);

@@ -17,6 +17,7 @@
 // launches are captured once per batch geometry into a CUDA graph on a
 // private stream and replayed on the caller's stream.  If the caller's
 // stream is itself being captured, the same nodes are enqueued on it instead.
+#include <math.h>
 #include <stdio.h>
 #include <string.h>
 
@@ -486,6 +487,32 @@ extern "C" cgh_status cgh_batch_plan(cgh_handle h, const cgh_problem *probs, int
     return CGH_ERR_INVALID_ARG;
 }
 
+// Untuned: CTA-pair items (256 x 128), which read half the operand bytes per
+// SM of one-CTA items (128 x 128): batches of 64, 16 and 8 holograms of 512 to
+// 2048 pixels a side took 4.05, 1.00 and 0.50 ms with them, 4.16, 1.20 and 0.58
+// with one-CTA items (64 holograms over and over, at the power cap: 4.4 ms with
+// either).  But one-CTA items where pairs pad their last row tiles by a quarter
+// of the work and that is a third of the waves: 16 of 1024x100x4000 218 us against
+// 245 in pairs, 6 of 1920x120x2000 96 and 115, 5 of 1024x300x4000 125 and 160 (32
+// of those, 684 and 664; uneven batches a few percent over a wave, 450 and 391).
+// An item counts as its share of the longest K.
+static bool default_sep_pairs(const cgh_problem *probs, int count, int sms) {
+    double single = 0.0, pairs = 0.0, most = 0.0;
+    for (int i = 0; i < count; ++i) {
+        const cgh_problem &p = probs[i];
+        const double K = p.N > 0 ? pad_to(2 * p.N, 64) : 0;
+        if (K <= 0 || K > gemm_k_chunk(true)) continue;  // (not in the work list)
+        const double cols = (p.Nx + 127) / 128;
+        single += K * cols * ((p.Ny + 127) / 128);
+        pairs += K * cols * ((p.Ny + 255) / 256);
+        most = K > most ? K : most;
+    }
+    if (most <= 0.0 || sms < 2) return true;
+    single /= most * sms;  // waves
+    pairs /= most * (sms / 2);
+    return pairs < 1.25 * single || ceil(pairs) < 1.5 * ceil(single);
+}
+
 extern "C" cgh_status cgh_tune_batch(cgh_handle h, const cgh_problem *probs,
                                      int count, int method, void *stream,
                                      cgh_direct_tile *chosen) {
@@ -500,9 +527,9 @@ extern "C" cgh_status cgh_tune_batch(cgh_handle h, const cgh_problem *probs,
     cudaStream_t s = (cudaStream_t)stream;
     if (method == CGH_SEP_FP16X3) {
         // the grouped split-FP16 GEMM's two kinds of items: one-CTA items and
-        // CTA-pair items (the default), each timed on its captured graph
+        // CTA-pair items, each timed on its captured graph
         int best_pairs = -1;
-        cgh_status st = tune_pick(h, 2, 1, TUNE_KEEP, s,
+        cgh_status st = tune_pick(h, 2, default_sep_pairs(probs, count, h->sm_count), TUNE_KEEP, s,
                                   [&](int pairs) {
                                       return h->batch(probs, count, method, s, -1, pairs);
                                   },
@@ -588,11 +615,7 @@ bool cgh_ctx::batch_sep_pairs(const cgh_problem *probs, int count, bool *tuned_o
         if (tuned_out) *tuned_out = true;
         return it->second / 1000 == CGH_GEMM_PAIRS;
     }
-    // CTA-pair items (256 x 128): batches of 64, 16 and 8 holograms of 512 to
-    // 2048 pixels a side took 4.05, 1.00 and 0.50 ms with them, 4.16, 1.20 and
-    // 0.58 with one-CTA items (128 x 128), which read twice the operand bytes
-    // per SM (64 holograms over and over, at the power cap: 4.4 ms with either)
-    return true;
+    return default_sep_pairs(probs, count, sm_count);
 }
 
 // Columns per CTA-pair item of a problem of Nx columns: equal whole
