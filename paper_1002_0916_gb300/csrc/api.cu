@@ -255,7 +255,7 @@ cgh_status cgh_ctx::forward(const float *points, const float *A,
 
 // ------------------------------------------------------------- release
 void cgh_ctx::release_all() {
-    for (Buffer *b : {&ws, &ws2, &io, &part, &meta, &bws, &hout[0], &hout[1]}) {
+    for (Buffer *b : {&ws, &ws2, &io, &meta, &bws, &hout[0], &hout[1]}) {
         if (b->ptr) cudaFree(b->ptr);
         b->ptr = nullptr;
         b->bytes = 0;

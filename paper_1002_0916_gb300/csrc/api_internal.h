@@ -38,7 +38,6 @@ struct cgh_ctx {
     Buffer ws;    // forward workspace: point records and tables
     Buffer ws2;   // second workspace: split planes / backward / batch
     Buffer io;    // staging for cgh_forward_host
-    Buffer part;  // partial sums of the adjoint
     Buffer meta;  // small per-call metadata (tensor maps, work lists)
     Buffer bws;   // batch workspace: per-problem records and tables
 
