@@ -61,21 +61,20 @@ static int bwd_strip(int Nx, int Ny, int N) {
     return (double)Nx * Ny * N < (double)(1 << 25) ? 16 : 32;
 }
 
-// Grid: x = column strips (fastest) of every group of BWD_THREADS points, one
-// dimension for both since 2^24 points are more groups than grid y takes; y =
-// runs of `rows` rows.  part: [strip * runs + run][5][Npad], the sums of G cos, G sin
+// Grid: x = column strips, y = groups of BWD_THREADS points, z = runs of
+// `rows` rows.  part: [strip * runs + run][5][Npad], the sums of G cos, G sin
 // dx, G sin dx^2, G sin dy, G sin dy^2.
 // ROW32: the rows' sines and cosines to FP32 rounding too (sep_by_strips).
 template <int STRIP, bool ROW32>
 __global__ void __launch_bounds__(BWD_THREADS, BwdShape<STRIP>::CTAS)
-direct_bwd_kernel(PointSource src, int Npad, int Nx, int Ny, int strips, int rows,
+direct_bwd_kernel(PointSource src, int Npad, int Nx, int Ny, int rows,
                   const float *__restrict__ G, float *__restrict__ part) {
     constexpr int NP2 = BwdShape<STRIP>::NP2, RB = BwdShape<STRIP>::RB;
     constexpr int LOADS = RB * STRIP / BWD_THREADS, UNROLL = BwdShape<STRIP>::UNROLL;
     __shared__ __align__(16) float sg[2][RB][STRIP];
-    const int strip = blockIdx.x % strips, x0 = strip * STRIP;
-    const int j = blockIdx.x / strips * BWD_THREADS + threadIdx.x;
-    const int ya = blockIdx.y * rows, yb = ya + rows < Ny ? ya + rows : Ny;
+    const int strip = blockIdx.x, x0 = strip * STRIP;
+    const int j = blockIdx.y * BWD_THREADS + threadIdx.x;
+    const int ya = blockIdx.z * rows, yb = ya + rows < Ny ? ya + rows : Ny;
     const int lc = threadIdx.x % STRIP, lr = threadIdx.x / STRIP;
     const float *gcol = G + x0 + lc;
     const bool in_x = x0 + lc < Nx;
@@ -160,7 +159,7 @@ direct_bwd_kernel(PointSource src, int Npad, int Nx, int Ny, int strips, int row
         sX += t0 + t1;
         sXX = fmaf(t0, dx0, fmaf(t1, dx1, sXX));
     }
-    float *dst = part + ((size_t)(strip * gridDim.y + blockIdx.y) * 5) * Npad + j;
+    float *dst = part + ((size_t)(strip * gridDim.z + blockIdx.z) * 5) * Npad + j;
     dst[0] = C;
     dst[(size_t)Npad] = sX;
     dst[(size_t)2 * Npad] = sXX;
@@ -312,14 +311,21 @@ static cgh_status run_direct_backward(cgh_ctx *h, const float *points, const flo
     float *part = (float *)h->ws2.ptr;
     const PointSource src{points, A, z, N, fresnel_scale(lambda, p), h->d_status};
     {
-        TimedLaunch tl(h, timer, s);
-        const dim3 grid((unsigned)strips * ((N + BWD_THREADS - 1) / BWD_THREADS), runs);
         auto kern = strip == 32 ? (row32 ? direct_bwd_kernel<32, true> : direct_bwd_kernel<32, false>)
                                 : (row32 ? direct_bwd_kernel<16, true> : direct_bwd_kernel<16, false>);
-        cudaError_t e = launch_kernel(
-            false, kern, grid, dim3(BWD_THREADS), 0, s, src, Npad, Nx, Ny, strips, rows, G, part);
-        if (e != cudaSuccess) return h->cuda_fail(e, "direct adjoint launch");
-        tl.done();
+        // as many groups of points as grid y takes (one grid dimension for
+        // strips and groups together made the kernel 4% slower)
+        const int most = 65535 * BWD_THREADS;
+        for (int j0 = 0; j0 < N; j0 += most) {
+            TimedLaunch tl(h, timer, s);
+            const int n = N - j0 < most ? N - j0 : most;
+            const PointSource some{points + 2 * (size_t)j0, A + j0, z + j0, n, src.K, src.status};
+            const dim3 grid(strips, (n + BWD_THREADS - 1) / BWD_THREADS, runs);
+            cudaError_t e = launch_kernel(false, kern, grid, dim3(BWD_THREADS), 0, s, some, Npad,
+                                          Nx, Ny, rows, G, part + j0);
+            if (e != cudaSuccess) return h->cuda_fail(e, "direct adjoint launch");
+            tl.done();
+        }
     }
     {
         TimedLaunch tl(h, CGH_K_BWD_REDUCE, s);
