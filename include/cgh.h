@@ -205,7 +205,11 @@ cgh_status cgh_host_wait_ticket(cgh_handle h, uint64_t ticket);
  * G^T U, at the accuracy of CGH_SEP_FP32's forward -- every FP32 factor split
  * into two FP16 numbers, partial sums added in FP32 -- with the pixel sums
  * fused into their epilogues; deterministic; small and low frames by the
- * direct method's sums instead).  Other methods:
+ * direct method's sums instead).  The handle's workspace holds the direct sums'
+ * partial sums, up to 20 B per point for every 16 columns and run of rows; for
+ * the products up to 1 GiB of tables, two FP16 pairs per pixel of G (8 B, rows
+ * and columns padded to whole eights) and partial sums of 24 B per point, tile of
+ * 192 columns and slice.  G may have any 4-byte alignment.  Other methods:
  * CGH_ERR_INVALID_ARG.  Errors as cgh_forward. */
 cgh_status cgh_backward(cgh_handle h, const float *points, const float *A,
                         const float *z, int N, double lambda, double p,

@@ -393,7 +393,7 @@ struct DirectTileLoop {
             // 46.6, 43.7); with the loads, 41.5 against 38.1 row by row and
             // 38.0 scalar at 3840x2160x4096.  What is left is the shared-
             // memory path, 128 bytes per clock into the registers: 10 16-byte
-            // loads per point for 64 pixels keep it 84% busy.  (16x6 blocks
+            // loads per point for 64 pixels keep it 76% busy.  (16x6 blocks
             // in four point groups, 168 registers and 12 warps per SM, reach
             // 43.7, but their FP32 chains are twice as long: 6.5e-7 from FP64
             // at 2048 points against 5.3e-7; in two halves, 42.7.)

@@ -324,7 +324,8 @@ __device__ __forceinline__ void adj32_reduce(const Adj32Prod &pr, const Adj32Arg
     }
     // (C by eights of columns: one chain of two roundings a column left the
     // amplitudes' gradient at 2.2e-7 from FP64, against 1.7e-7; what is left is
-    // the tensor cores' truncation, a shrink of 7e-8 in each product)
+    // the tensor cores' truncation, a shrink of 7e-8 in each product on random
+    // phases)
     float C = 0.0f, C8 = 0.0f, S0 = 0.0f, S1 = 0.0f, S2 = 0.0f;
 #pragma unroll
     for (int i = 0; i < RUN; ++i) {
@@ -612,8 +613,9 @@ constexpr int S32_MAX_SPLIT = 64;
 // waves of the SM pairs times (K blocks of a slice + fill and epilogue), plus
 // the partial tiles of a split.  The constants are fits in microseconds to a
 // sweep of every width and 1 to 64 slices over 13 frames (128 x 128 to
-// 3840 x 2160, 64 to 16,384 points): a K block takes 0.44 us at 112 columns
-// and 0.87 at 256, and a small frame is better cut along K: 128x128x16384 31 us
+// 3840 x 2160, 64 to 16,384 points), taken with slower MMA issue: a K block of
+// 0.44 us at 112 columns and 0.87 at 256 (0.37 and 0.81 since).  A small frame is
+// better cut along K: 128x128x16384 31 us
 // in 24 slices against 187 in one, 640x480x2000 21 us in 5 against 39.
 static Sep32Plan sep32_plan(int M, int N, int KB, int sms) {
     Sep32Plan best{256, 1};
