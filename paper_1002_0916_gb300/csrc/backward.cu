@@ -263,12 +263,14 @@ cudaError_t launch_adjoint_sum(const PointSource &src, const AdjointParts &pp, c
 // and 44, 2048x24x1000 27 and 26, 32768x16x16 69 and 53.  With the rows' sines to
 // FP32 rounding (3% of the time) the strips are no less accurate: 64x64x4000 x
 // 1.4e-7, A 1.6e-7, z 1.3e-7 from FP64, the products 2.3e-7, 1.9e-7, 2.5e-7.
+// Their partial sums, 20 bytes per point and 32 columns, take 1 GiB at most, like
+// the products' tables.
 static bool sep_by_strips(int N, int Nx, int Ny) {
     const long long pixels = (long long)Nx * Ny;
     const bool small = Nx <= 8192 && Ny <= 1024 &&
                        (pixels <= 8192 ||
                         (pixels <= 32768 && pixels * N <= (Ny <= 64 ? 25000000 : 12000000)));
-    return small || (Ny <= 20 && N >= 256);
+    return (small || (Ny <= 20 && N >= 256)) && (long long)Nx * N <= 1700000000;
 }
 
 // Rows per run: the fewest runs (each repeats the columns' sincos, worth

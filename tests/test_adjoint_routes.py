@@ -73,3 +73,29 @@ def test_accuracy_of_a_small_frame(cg):
         for v, ref in zip(got, _reference(c, G)[0]):
             v = v.cpu().numpy().astype(np.float64)
             assert np.linalg.norm(v - ref) <= 1e-6 * np.linalg.norm(ref)
+
+
+def test_scratch_of_a_low_frame_and_many_points(cg):
+    """The strips' partial sums would take 5 GiB here, the products work in chunks
+    of 1 GiB; 40 points against FP64."""
+    import torch
+    c = make_cloud(77, 1000000, 8192, 1, integer=False, zlo=0.2, zhi=0.9, lam=532e-9, p=6.4e-6)
+    G = grad_field(78, 8192, 1)
+    h = cg.cgh_create(0)
+    try:
+        args = (*to_dev(c), c.lam, c.p, c.Nx, c.Ny, torch.from_numpy(G).cuda())
+        outs = [torch.empty((c.N, 5), device="cuda")]  # (the outputs' memory, held before)
+        del outs
+        free = torch.cuda.mem_get_info()[0]
+        gp, gA, gz = cg.cgh_backward(*args, method="sep_fp32", handle=h)
+        torch.cuda.synchronize()
+        assert cg.cgh_last_device_status(h) == cg.CGH_OK
+        assert free - torch.cuda.mem_get_info()[0] < 2.5 * 2 ** 30
+    finally:
+        cg.cgh_destroy(h)
+    some = np.linspace(0, c.N - 1, 40).astype(int)
+    c.xy, c.A, c.z = c.xy[some], c.A[some], c.z[some]
+    gp = gp.cpu().numpy()[some]
+    got = [gp[:, 0], gp[:, 1], gA.cpu().numpy()[some], gz.cpu().numpy()[some]]
+    for v, ref, bound in zip(got, *_reference(c, G)):
+        assert np.all(np.abs(v - ref) <= EPS * bound)
